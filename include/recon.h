@@ -338,10 +338,10 @@ enum {
                                    sorting the positions again; the caller guarantees they did not
                                    change in between.  While that order is held, shifts of other
                                    catalogues take the direct path.                              */
-  RECON_OPT_KSPACE_GENERIC = 4, /* 0 (default): for N = 512 the source update and the projection
-                                   pass run in kernels that keep the first and last FFT stages
-                                   (and the c2r/r2c pairing) in registers; 1: the generic staged
-                                   kernels (same butterflies)                                     */
+  RECON_OPT_KSPACE_GENERIC = 4, /* 0 (default): for N = 256, 384, 512 and 1024 the source update, the
+                                   x passes and the projection run in kernels that keep the first and
+                                   last FFT stages (and the c2r/r2c pairing) in registers and carry
+                                   vectors in reduced form; 1: the generic staged kernels         */
   RECON_OPT_KITER_TMA = 8,      /* N = 512 register-fused path: 0 (default) one CTA per tile loading its
                                    inputs itself; 1 persistent CTAs whose inputs (A, P_y, delta(k), S)
                                    are streamed into shared memory by the tensor memory accelerator,
@@ -354,12 +354,12 @@ enum {
                                    paper's nearest grid point (Sec. 3: node floor(x N / L + 1/2)),
                                    always on the direct (unsorted) deposit kernel.  The shift still
                                    interpolates Psi with CIC.                                     */
-  RECON_OPT_FFT_RADIX = 9,      /* radix order of every FFT plan of the handle's mesh: 0 (default)
-                                   largest radix first; 1 smallest first, for N = 256 (4 8 8, its
-                                   z half-length plan 4 4 8) and N = 384 (6 8 8; 3 8 8), other
-                                   meshes UNSUPPORTED.  Same transforms up to float32 rounding;
+  RECON_OPT_FFT_RADIX = 9,      /* radix order of every FFT plan of the handle's mesh: 0 (default);
+                                   1 smallest first, in the generic staged kernels, for N = 256
+                                   (4 8 8, its z half-length plan 4 4 8) and N = 384 (6 8 8; 3 8 8),
+                                   other meshes UNSUPPORTED.  Same transforms up to float32 rounding;
                                    the batch autotuner times both.                               */
-  RECON_OPT_PLANE_BATCH = 6     /* register-fused path (N = 512): 0 (off) or 16, 32, 64 y-planes per
+  RECON_OPT_PLANE_BATCH = 6     /* register-fused path: 0 (off) or 16, 32, 64 y-planes per
                                    batch; each update then runs its inverse x, projection and forward
                                    x passes batch by batch, so a batch's fields stay in the L2 between
                                    the three passes (same arithmetic, fewer HBM round trips).  A
@@ -406,8 +406,8 @@ typedef struct recon_batch_item {
  * Otherwise the items run one after another through the handle API.  flags is a bitwise OR of
  * RECON_BATCH_*.  With RECON_BATCH_TUNE, a size class not seen before in this process is first
  * tuned on its first item, before the batch runs and outside every item's time: the deposit path,
- * the x-line FFT tile width, at N = 512 the k-space kernel family (register-fused or generic), at
- * N = 256 and 384 the FFT radix order, and the shift path; the fastest are kept for the process
+ * the x-line FFT tile width, at N = 256, 384, 512 and 1024 the k-space kernel family (register-fused
+ * or generic), at N = 256 and 384 the FFT radix order, and the shift path; the fastest are kept for the process
  * (recon_batch_plan).  With RECON_BATCH_ONE_GRAPH the whole batch is one CUDA graph, built before
  * it is launched, with one chain of items per size class and the chains side by side (one item
  * per class in flight).  Other bits: INVALID_ARG.  Returns the first error of any item (per-item

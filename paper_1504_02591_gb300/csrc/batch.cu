@@ -14,8 +14,8 @@
 // Before the first mock of a size class not seen before in this process, the autotuner times the
 // class's candidate schedules on that mock (outside the items' times) and keeps the fastest for the
 // process: the deposit path (direct atomics or brick-sorted), the x-line FFT tile width (16 or 8
-// columns), for N = 512 the k-space kernel family (register-fused or generic staged), for N = 256
-// and 384 the FFT radix order (largest or smallest radix first) and the shift path.
+// columns), the k-space kernel family where the mesh has two (register-fused or generic staged), for
+// N = 256 and 384 the FFT radix order and the shift path.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -23,6 +23,7 @@
 
 #include "../../include/recon.h"
 #include "batch_graph.h"
+#include "types.h"
 
 namespace {
 
@@ -91,7 +92,8 @@ recon_status tune(recon_handle* h, recon_batch_item& it, cudaStream_t st, Plan* 
   if ((s = recon_smooth(h)) != RECON_OK) return s;
   // iteration schedules, each on the same delta(k) for a fixed number of updates
   best = 1e30f;
-  const int fams = it.params.nmesh[0] == 512 ? 2 : 1;   // the register-fused family exists at N = 512
+  // the register-fused family, where the mesh has one, and the generic kernels
+  const int fams = rg::mesh_kernels(it.params.nmesh[0])->kspace_fused ? 2 : 1;
   // the alternative radix order exists where the option accepts it
   const int orders = recon_set_option(h, RECON_OPT_FFT_RADIX, 1) == RECON_OK ? 2 : 1;
   int n_it = 0;

@@ -12,7 +12,7 @@
 #include <stdint.h>
 
 // Radix order of the plans of the mesh sides that have two (see the plan table at the end): 0 the
-// default, largest radix first; 1 the alternative, smallest radix first.  A translation unit
+// default, symmetric (256, 384) or largest radix first; 1 the alternative, smallest radix first.  A translation unit
 // compiles one order, and its kernels live in that order's inline namespace, so the kernels of
 // both orders link into one library under distinct names.
 #ifndef RG_RADIX_ORDER
@@ -27,8 +27,16 @@
 namespace rg {
 inline namespace RG_KNS {
 
+#ifdef RG_PACKED
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+#elif defined(RG_PACKED2)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+#else
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+#endif
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -94,6 +102,38 @@ struct Dft<8, INV> {
   }
 };
 
+// 16 = 4 x 4: y[k1 + 4 k2] = sum_n2 w16^(n2 k1) w4^(n2 k2) sum_n1 w4^(n1 k1) x[4 n1 + n2]
+template <bool INV>
+struct Dft<16, INV> {
+  __device__ __forceinline__ static void run(float2* v) {
+    const float h = 0.70710678118654752f, c = 0.92387953251128676f, s = 0.38268343236508977f;
+    const float sg = INV ? 1.f : -1.f;
+    float2 t[4][4];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1) t[n2][n1] = v[4 * n1 + n2];
+      Dft<4, INV>::run(t[n2]);
+    }
+    t[1][1] = cmul(t[1][1], make_float2(c, sg * s));
+    t[1][2] = cmul(t[1][2], make_float2(h, sg * h));
+    t[1][3] = cmul(t[1][3], make_float2(s, sg * c));
+    t[2][1] = cmul(t[2][1], make_float2(h, sg * h));
+    t[2][2] = rot<INV>(t[2][2]);
+    t[2][3] = cmul(t[2][3], make_float2(-h, sg * h));
+    t[3][1] = cmul(t[3][1], make_float2(s, sg * c));
+    t[3][2] = cmul(t[3][2], make_float2(-h, sg * h));
+    t[3][3] = cmul(t[3][3], make_float2(-c, -sg * s));
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) {
+      float2 b[4] = {t[0][k1], t[1][k1], t[2][k1], t[3][k1]};
+      Dft<4, INV>::run(b);
+#pragma unroll
+      for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = b[k2];
+    }
+  }
+};
+
 template <bool INV>
 struct Dft<3, INV> {
   __device__ __forceinline__ static void run(float2* v) {
@@ -130,6 +170,66 @@ struct Dft<6, INV> {
     v[5] = csub(e[2], o2);
   }
 };
+
+// Radix 8 Q = Q x 8 (Q = 3, 4): y[k1 + 8 k2] = sum_n2 w^(n2 k1) wQ^(n2 k2) sum_n1 w8^(n1 k1) x[Q n1 + n2],
+// w = exp(-+ 2 pi i / (8 Q)); the factors w^m from the cosine table of the radix (sin(m) = cos(m - R/4)).
+template <int R>
+__device__ __forceinline__ constexpr float dft_cos(int m);
+template <>
+__device__ __forceinline__ constexpr float dft_cos<24>(int m) {
+  constexpr float c[24] = {
+      1.f, 0.96592582628906831f, 0.86602540378443871f, 0.70710678118654757f,
+      0.5f, 0.25881904510252074f, 0.f, -0.25881904510252063f,
+      -0.5f, -0.70710678118654746f, -0.86602540378443871f, -0.9659258262890682f,
+      -1.f, -0.96592582628906831f, -0.86602540378443882f, -0.70710678118654791f,
+      -0.5f, -0.25881904510252063f, 0.f, 0.2588190451025203f,
+      0.5f, 0.70710678118654735f, 0.86602540378443837f, 0.96592582628906809f};
+  return c[((m % 24) + 24) % 24];
+}
+template <>
+__device__ __forceinline__ constexpr float dft_cos<32>(int m) {
+  constexpr float c[32] = {
+      1.f, 0.98078528040323043f, 0.92387953251128674f, 0.83146961230254524f,
+      0.70710678118654757f, 0.55557023301960229f, 0.38268343236508984f, 0.19509032201612833f,
+      0.f, -0.19509032201612819f, -0.38268343236508973f, -0.55557023301960196f,
+      -0.70710678118654746f, -0.83146961230254535f, -0.92387953251128674f, -0.98078528040323043f,
+      -1.f, -0.98078528040323043f, -0.92387953251128685f, -0.83146961230254546f,
+      -0.70710678118654768f, -0.55557023301960218f, -0.38268343236509034f, -0.19509032201612866f,
+      0.f, 0.1950903220161283f, 0.38268343236509f, 0.55557023301960184f,
+      0.70710678118654735f, 0.83146961230254524f, 0.92387953251128652f, 0.98078528040323032f};
+  return c[((m % 32) + 32) % 32];
+}
+
+template <int Q, bool INV>
+struct Dft8Q {
+  static constexpr int R = 8 * Q;
+  __device__ __forceinline__ static void run(float2* v) {
+    float2 t[Q][8];
+#pragma unroll
+    for (int n2 = 0; n2 < Q; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 8; ++n1) t[n2][n1] = v[Q * n1 + n2];
+      Dft<8, INV>::run(t[n2]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 8; ++k1) {
+      float2 b[Q];
+#pragma unroll
+      for (int n2 = 0; n2 < Q; ++n2) {
+        const int m = n2 * k1;
+        const float c = dft_cos<R>(m), sn = dft_cos<R>(m - R / 4);
+        b[n2] = m == 0 ? t[n2][k1] : cmul(t[n2][k1], make_float2(c, INV ? sn : -sn));
+      }
+      Dft<Q, INV>::run(b);
+#pragma unroll
+      for (int k2 = 0; k2 < Q; ++k2) v[k1 + 8 * k2] = b[k2];
+    }
+  }
+};
+template <bool INV>
+struct Dft<24, INV> : Dft8Q<3, INV> {};
+template <bool INV>
+struct Dft<32, INV> : Dft8Q<4, INV> {};
 
 // ----------------------------------------------------------------------------------------------
 // Shared-memory layouts.  Element i of line col lives at phys(i, col).  The swizzles make every
@@ -268,8 +368,9 @@ RG_PLAN(96, 8, 4, 3)
 #if RG_RADIX_ORDER == 0
 RG_PLAN(128, 8, 4, 4)
 RG_PLAN(192, 8, 8, 3)
-RG_PLAN(256, 8, 8, 4)
-RG_PLAN(384, 8, 8, 6)
+// symmetric plans (first radix = last): the register-fused passes of N = 256, 384, 512 and 1024
+RG_PLAN(256, 8, 4, 8)
+RG_PLAN(384, 8, 6, 8)
 #else   // the 256 and 384 meshes (and their half-length z plans) smallest radix first
 RG_PLAN(128, 4, 4, 8)
 RG_PLAN(192, 3, 8, 8)
@@ -277,7 +378,7 @@ RG_PLAN(256, 4, 8, 8)
 RG_PLAN(384, 6, 8, 8)
 #endif
 RG_PLAN(512, 8, 8, 8)
-RG_PLAN(1024, 8, 8, 4, 4)
+RG_PLAN(1024, 8, 16, 8)
 #undef RG_PLAN
 
 }  // namespace RG_KNS

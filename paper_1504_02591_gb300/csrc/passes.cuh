@@ -17,15 +17,12 @@ inline namespace RG_KNS {   // the radix order's namespace (fft_core.cuh)
 
 constexpr int kZThreads = 256;
 
-// columns of one N = 512 k-space (y) tile: 4 adjacent kz (one 32-byte sector per row)
-#ifndef RECON_KITER_COLS
-#define RECON_KITER_COLS 4
-#endif
 template <int N, int MODE = 0, int NARROW = 0>
 struct SCols {  // adjacent columns in one strided tile (the 3-component k-space tiles are narrower)
   static constexpr bool kK = (MODE == S_DELTA || MODE == S_ITER);
   static constexpr int kWide = ((N / 2) % 16 == 0 && N < 1024 && !NARROW) ? 16 : 8;   // must divide N / 2
-  static constexpr int v = kK ? (N == 512 ? RECON_KITER_COLS : 4) : kWide;
+  // k-space (y) tiles: 4 adjacent kz (one 32-byte sector per row); 8 on the 256 mesh, whose lines leave room
+  static constexpr int v = kK ? (N == 256 ? 8 : 4) : kWide;
   static_assert((N / 2) % v == 0 && N % v == 0, "tile columns must divide the half-grid rows");
 };
 
@@ -454,142 +451,151 @@ __global__ void __launch_bounds__(kZThreads, kZMinBlocks<N>) zpass_kernel(const 
 }
 
 // ------------------------------------------------------------------------------------------------
-// The projection pass for N = 512 (rows of L = 256 complex values, radices 8 x 8 x 4), one warp per
-// row.  Lane l holds the points l + 32 r (r = 0..7) of each component.  The c2r merge pairs point
-// m with L - m, which for l >= 1 sits on lane 32 - l (lane 0 pairs with itself and the Nyquist
-// value), so the merge runs on shuffles straight after the global loads and feeds the first
-// inverse stage in registers.  The last inverse stage (radix 4, butterflies l and l + 32) leaves
-// exactly the points l + 32 r on lane l, so the projection and the first forward stage run in
-// registers too; the r2c split again pairs lanes l and 32 - l, and the results go straight to
-// global memory.  Shared memory carries only the two middle stages of each transform.  The
-// butterflies, twiddles and merge/split formulas are those of the generic pass.
+// The register-fused family (N = 256, 384, 512, 1024): transforms whose first stage takes its inputs
+// straight from global memory (or from the previous transform's last stage) and whose last stage's
+// outputs go straight on, in registers, so that shared memory carries only what changes hands between
+// stages.  That needs plans whose last stage leaves on a thread exactly the points its first stage
+// reads:
+//   lines of N (k-space and x passes):  8 x N/64 x 8, butterfly j at the points j + (N/8) r
+//   rows of L = N/2 (z pass):           E x G with G lanes a row and E points a lane, lane l at the
+//                                       points l + G r: one exchange per transform
+// The other mesh sides, and the alternative radix order, use the staged kernels above and below.
 // ------------------------------------------------------------------------------------------------
 template <int N>
-struct ZProj8 {
-  static_assert(N == 512, "radices 8 x 8 x 4 of the 256-point row transform");
+constexpr bool kFusedMesh = RG_RADIX_ORDER == 0 && (N == 256 || N == 384 || N == 512 || N == 1024);
+
+// The z passes of the family.  A group of G lanes transforms one row of L = G E complex points, E a
+// lane; a warp holds RPW = 32 / G rows: the two fields (C, Psi_z) of RPW / 2 mesh rows (x, y), field q
+// of a mesh row on lane group 2 p + q.  Stage 1 is a radix-E butterfly per lane on its own points
+// l + G r; one exchange through shared memory (the row's buffer, one pad word per E so that writes at
+// stride E and reads fall in distinct banks); stage 2 is E / G radix-G butterflies per lane, which
+// leave the points l + G r again.  The c2r merge pairs point m with L - m on lane G - l (lane 0 with
+// itself and the Nyquist value), so it and the r2c split run on shuffles.
+// The pass is bound by the L1's shared-memory pipe (the three-stage warp-per-row form used it 80% of
+// the time): one exchange instead of two and twiddles shared by the warp's rows cut its wavefronts.
+template <int N>
+struct ZRow {
   static constexpr int L = N / 2;
-  static constexpr int TABZ = (Plan<L>::kTab + 1) & ~1;
-  static constexpr int kWarp = L + L / 2;      // FFT buffer + the coarse correction row (Z_WARM)
-  static constexpr size_t smem = sizeof(float2) * ((size_t)L + 2 + TABZ + (size_t)kZWarps * kWarp);
+  static constexpr int G = (N >= 512) ? 16 : 8;
+  static constexpr int E = L / G;              // 16, 24, 16, 32
+  static constexpr int Q = E / G;              // stage-2 butterflies a lane
+  static_assert(E % G == 0, "stage 2 divides evenly over the row's lanes");
+  static constexpr int RPW = 32 / G;           // rows a warp
+  static constexpr int PPW = RPW / 2;          // mesh rows (two fields each) a warp
+  static constexpr int kRow = (E + 1) * G;     // float2 of one row's buffer
+  static constexpr int kTab = (G - 1) * E;     // stage-2 twiddles
+  static constexpr int kHead = (L + 1 + kTab + 1) & ~1;
+  static constexpr size_t smem = sizeof(float2) * ((size_t)kHead + (size_t)kZWarps * RPW * kRow);
+  // CTAs per SM that the points a lane holds leave registers for (measured: 512 at 2, 3, 4 CTAs 576,
+  // 534, 529 us; 384 at 2, 3 304, 275 us)
+  static constexpr int kMinBlocks = E == 16 ? 4 : (E == 24 ? 3 : 2);
 };
 
-// the middle stage (NS = 8, radix 8): butterfly l reads l + 32 r, writes (l / 8) 64 + l mod 8 + 8 r
-template <bool INV>
-__device__ __forceinline__ void zrow_mid(float2* __restrict__ s, const float2* __restrict__ tab, int lane) {
-  using Lay = RowLayout<256>;
-  float2 v[8];
-  const int k = lane & 7;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) v[r] = s[Lay::phys(lane + 32 * r, 0)];
-#pragma unroll
-  for (int r = 1; r < 8; ++r) {
-    float2 w = tab[(r - 1) * 8 + k];
-    if (INV) w.y = -w.y;
-    v[r] = cmul(v[r], w);
-  }
-  Dft<8, INV>::run(v);
-  __syncwarp();
-  const int base = (lane >> 3) * 64 + k;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) s[Lay::phys(base + 8 * r, 0)] = v[r];
-  __syncwarp();
+// Twiddles of the pass: tw[m] = exp(-2 pi i m / N), m <= L, and the stage-2 table [r - 1][j] =
+// exp(-2 pi i r j / L).
+template <int N>
+__device__ __forceinline__ void zrow_tables(const ZArgs& a, float2* tw, float2* tab) {
+  using Z = ZRow<N>;
+  for (int m = threadIdx.x; m <= Z::L; m += kZThreads) tw[m] = a.tw[m];
+  for (int e = threadIdx.x; e < Z::kTab; e += kZThreads) tab[e] = a.tw[2 * (1 + e / Z::E) * (e % Z::E)];
+  __syncthreads();
 }
 
-// One 256-point transform: in, z[l + 32 r] (registers, r = 0..7); out, Z[j + 64 r] for the two
-// butterflies j = l (A[r]) and j = l + 32 (B[r]), r = 0..3.
-template <bool INV>
-__device__ __forceinline__ void zrow_fft(float2 (&v)[8], float2 (&A)[4], float2 (&B)[4], float2* __restrict__ s,
-                                         const float2* __restrict__ tab, int lane) {
-  using Lay = RowLayout<256>;
-  Dft<8, INV>::run(v);                                   // stage 1 (NS = 1): butterfly l, no twiddles
+// The L-point transforms of the warp's rows: v[r] = x[l + G r] in, X[l + G r] out; s is the row's buffer.
+template <bool INV, int N>
+__device__ __forceinline__ void zrow_fft(float2 (&v)[ZRow<N>::E], float2* __restrict__ s,
+                                         const float2* __restrict__ tab, int l) {
+  using Z = ZRow<N>;
+  constexpr int E = Z::E, G = Z::G;
+  Dft<E, INV>::run(v);
 #pragma unroll
-  for (int r = 0; r < 8; ++r) s[Lay::phys(8 * lane + r, 0)] = v[r];
+  for (int r = 0; r < E; ++r) s[(E + 1) * l + r] = v[r];
   __syncwarp();
-  zrow_mid<INV>(s, tab, lane);
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {                          // stage 3 (NS = 64, radix 4): butterflies l, l + 32
-    const int j = lane + 32 * h;
-    float2 u[4];
+  for (int h = 0; h < Z::Q; ++h) {
+    const int j = l + G * h;
+    float2 u[G];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) u[r] = s[Lay::phys(j + 64 * r, 0)];
+    for (int r = 0; r < G; ++r) u[r] = s[(E + 1) * r + j];
 #pragma unroll
-    for (int r = 1; r < 4; ++r) {
-      float2 w = tab[56 + (r - 1) * 64 + j];
+    for (int r = 1; r < G; ++r) {
+      float2 w = tab[(r - 1) * E + j];
       if (INV) w.y = -w.y;
       u[r] = cmul(u[r], w);
     }
-    Dft<4, INV>::run(u);
+    Dft<G, INV>::run(u);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) (h ? B : A)[r] = u[r];
+    for (int r = 0; r < G; ++r) v[h + Z::Q * r] = u[r];
   }
-  __syncwarp();                                          // s is reused by the next line
+  __syncwarp();                                            // s is reused by the next transform
 }
 
-// c2r of one component's row (loaded by zrow_load: X[l + 32 r] and the Nyquist value): merge with
-// the mirror X[L - l - 32 r] (on lane 32 - l; lane 0 with itself and the Nyquist value), inverse
-// transform; out A[r] = x[l + 64 r], B[r] = x[l + 32 + 64 r] (complex points = real pairs 2m, 2m + 1).
-__device__ __forceinline__ void zrow_load(const Field& f, size_t row, int lane, float2 (&x)[8], float2& xl) {
-  const float2* src = f.M + row * 256;
+template <int N>
+__device__ __forceinline__ void zrow_load(const Field& f, size_t row, int l, float2 (&x)[ZRow<N>::E], float2& xl) {
+  const float2* src = f.M + row * ZRow<N>::L;
 #pragma unroll
-  for (int r = 0; r < 8; ++r) x[r] = src[lane + 32 * r];
+  for (int r = 0; r < ZRow<N>::E; ++r) x[r] = src[l + ZRow<N>::G * r];
   xl = f.Q[row];
 }
 
-__device__ __forceinline__ void zrow_c2r(const float2 (&x)[8], float2 xl, int lane, int partner,
-                                         const float2* __restrict__ tw, float2* __restrict__ s,
-                                         const float2* __restrict__ tab, float2 (&A)[4], float2 (&B)[4]) {
-  float2 z[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    float2 xm;
-    xm.x = __shfl_sync(0xffffffffu, x[7 - r].x, partner);
-    xm.y = __shfl_sync(0xffffffffu, x[7 - r].y, partner);
-    if (lane == 0) xm = (r == 0) ? xl : x[(8 - r) & 7];
-    const float2 w = cconj(tw[lane + 32 * r]);
-    const float2 xk = x[r];
-    const float2 ev = make_float2(xk.x + xm.x, xk.y - xm.y);
-    const float2 o = cmul(make_float2(xk.x - xm.x, xk.y + xm.y), w);
-    z[r] = cadd(ev, mul_i(o));
-  }
-  zrow_fft<true>(z, A, B, s, tab, lane);
+__device__ __forceinline__ float2 shfl2(float2 v, int src) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+__device__ __forceinline__ float2 shfl2_xor(float2 v, int m) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
 }
 
-// r2c of one component's row from the real points v[r] = (x[2m], x[2m + 1]), m = l + 32 r: forward
-// transform, split (pairs k, L - k on lanes l and 32 - l), store the half-complex row and Nyquist value.
-__device__ __forceinline__ void zrow_r2c(float2 (&v)[8], const Field& f, size_t row, int lane, int partner,
-                                         const float2* __restrict__ tw, float2* __restrict__ s,
-                                         const float2* __restrict__ tab) {
-  constexpr int L = 256;
-  float2 Y0[4], Y1[4];
-  zrow_fft<false>(v, Y0, Y1, s, tab, lane);
-  float2* dst = f.M + row * L;
+// Walk the mirror pairs of a row in place: fn(r, x[r], mirror) for every point, both values original.
+// Point r of lane l >= 1 mirrors point E - 1 - r of lane G - l; on lane 0 point r mirrors E - r, and
+// point 0's mirror is xl.
+template <int N, class Fn>
+__device__ __forceinline__ void zrow_mirror(float2 (&x)[ZRow<N>::E], float2 xl, int l, int partner, Fn&& fn) {
+  constexpr int E = ZRow<N>::E;
+  float2 prev = xl;                     // lane 0: the original x[E - r]
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    float2 pa, pb;
-    pa.x = __shfl_sync(0xffffffffu, Y1[3 - r].x, partner);
-    pa.y = __shfl_sync(0xffffffffu, Y1[3 - r].y, partner);
-    pb.x = __shfl_sync(0xffffffffu, Y0[3 - r].x, partner);
-    pb.y = __shfl_sync(0xffffffffu, Y0[3 - r].y, partner);
-    if (lane == 0) {
-      pa = Y0[(4 - r) & 3];
-      pb = Y1[3 - r];
+  for (int r = 0; r < E / 2; ++r) {
+    const float2 a = x[r], b = x[E - 1 - r];
+    float2 am = shfl2(b, partner), bm = shfl2(a, partner);
+    if (l == 0) {
+      am = prev;
+      bm = r + 1 < E / 2 ? x[r + 1] : b;
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = lane + 32 * h + 64 * r;
-      const float2 zk = h ? Y1[r] : Y0[r], zm = h ? pb : pa;
-      float2 xk;
-      if (k == 0) {
-        xk = make_float2(zk.x + zk.y, 0.f);
-        f.Q[row] = make_float2(zk.x - zk.y, 0.f);
-      } else {
-        const float2 ev = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-        const float2 o = make_float2(0.5f * (zk.x - zm.x), 0.5f * (zk.y + zm.y));
-        xk = cadd(ev, cmul(make_float2(o.y, -o.x), tw[k]));
-      }
-      dst[k] = xk;
-    }
+    prev = b;
+    fn(r, x[r], a, am);
+    fn(E - 1 - r, x[E - 1 - r], b, bm);
   }
+}
+
+// c2r merge of the rows in registers: X[m], the Nyquist value -> the inverse transform's inputs.
+template <int N>
+__device__ __forceinline__ void zrow_merge(float2 (&x)[ZRow<N>::E], float2 xl, int l, int partner,
+                                           const float2* __restrict__ tw) {
+  zrow_mirror<N>(x, xl, l, partner, [&](int r, float2& out, float2 xk, float2 xm) {
+    const float2 w = cconj(tw[l + ZRow<N>::G * r]);
+    const float2 ev = make_float2(xk.x + xm.x, xk.y - xm.y);
+    const float2 o = cmul(make_float2(xk.x - xm.x, xk.y + xm.y), w);
+    out = cadd(ev, mul_i(o));
+  });
+}
+
+// r2c split of the transformed rows, stored as a half-complex row and its Nyquist value.
+template <int N>
+__device__ __forceinline__ void zrow_split_store(float2 (&y)[ZRow<N>::E], const Field& f, size_t row, int l, int partner,
+                                                 const float2* __restrict__ tw) {
+  float2* dst = f.M + row * ZRow<N>::L;
+  zrow_mirror<N>(y, y[0], l, partner, [&](int r, float2&, float2 zk, float2 zm) {
+    const int k = l + ZRow<N>::G * r;
+    float2 xk;
+    if (r == 0 && l == 0) {
+      xk = make_float2(zk.x + zk.y, 0.f);
+      f.Q[row] = make_float2(zk.x - zk.y, 0.f);
+    } else {
+      const float2 ev = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+      const float2 o = make_float2(0.5f * (zk.x - zm.x), 0.5f * (zk.y + zm.y));
+      xk = cadd(ev, cmul(make_float2(o.y, -o.x), tw[k]));
+    }
+    dst[k] = xk;
+  });
 }
 
 // The observer offset d = (dx, dy, dz) of a node and w with r = w d the line of sight (radial: w =
@@ -602,68 +608,69 @@ __device__ __forceinline__ void zrow_dw(const Geometry& g, float dx, float dy, i
     w0 = w1 = 1.f;
     return;
   }
-  const int n = g.n;
-  dz0 = g.off[2 * n + 2 * m];
-  dz1 = g.off[2 * n + 2 * m + 1];
+  const float2 dz = reinterpret_cast<const float2*>(g.off + 2 * g.n)[m];   // n is even, the table 256-byte aligned
+  dz0 = dz.x;
+  dz1 = dz.y;
   const float q0 = fmaf(dx, dx, fmaf(dy, dy, dz0 * dz0));
   const float q1 = fmaf(dx, dx, fmaf(dy, dy, dz1 * dz1));
   w0 = q0 > 0.f ? rsqrtf(q0) : 0.f;
   w1 = q1 > 0.f ? rsqrtf(q1) : 0.f;
 }
 
-// The z passes of the register-fused path, one warp per row.  With r = w d, the projection
-// P = coef (Psi.r) r needs only C = dx Psi_x + dy Psi_y and Psi_z (dx, dy are constant along a z
-// row, so C is formed before the transform):  u = coef w (C + dz Psi_z) and P_j = d_j psi with
-// psi = w u.  So the pass transforms two rows each way and leaves psi^ = r2c(psi) and
-// Z^ = r2c(dz psi) (P_x = dx psi^ and P_y = dy psi^ are formed by the forward x pass).
-//   Z_PROJ:   c2r x2, P, r2c x2; once the device loop has converged, c2r x3 and the real Psi.
-//             With a.cform (while the loop runs) C arrives formed in f[0] and Psi_z in wf.
-//   Z_RADIAL: c2r x2, u as a real row (C form as Z_PROJ).
+// With r = w d, the projection P = coef (Psi.r) r needs only C = dx Psi_x + dy Psi_y and Psi_z (dx,
+// dy are constant along a z row; the inverse x pass forms C):  u = coef w (C + dz Psi_z) and
+// P_j = d_j psi with psi = w u.  So the pass transforms two rows each way and leaves
+// psi^ = r2c(psi) and Z^ = r2c(dz psi) (P_x = dx psi^ and P_y = dy psi^ are formed by the forward x
+// pass).
+//   Z_PROJ:   c2r x2 of C (f[0]) and Psi_z (wf), P, r2c x2; once the device loop has converged,
+//             c2r x3 and the real Psi.
+//   Z_FINAL:  c2r x3 and the real Psi.
+//   Z_RADIAL: c2r x2, u as a real row.
 //   Z_WARM:   u from the real row plus the upsampled coarse correction, r2c x2.
 //   Z_USTART: u from the real row, r2c x2.
 template <int N, int MODE>
-__global__ void __launch_bounds__(kZThreads, 2) zfused8_kernel(const ZArgs a) {
-  constexpr int L = ZProj8<N>::L;
+__global__ void __launch_bounds__(kZThreads, ZRow<N>::kMinBlocks) zfused_kernel(const ZArgs a) {
+  using Z = ZRow<N>;
+  constexpr int L = Z::L, E = Z::E, G = Z::G;
   extern __shared__ float4 zsm[];
   float2* tw = reinterpret_cast<float2*>(zsm);                        // exp(-2 pi i m / N), m <= L
-  float2* tab = tw + L + 2;                                           // stage twiddles (256-point plan)
+  float2* tab = tw + L + 1;                                           // stage-2 twiddles
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* s = tab + ZProj8<N>::TABZ + warp * ZProj8<N>::kWarp;
-  float* crow = reinterpret_cast<float*>(s + L);                      // Z_WARM: this row's coarse correction
-  for (int m = threadIdx.x; m <= L; m += kZThreads) tw[m] = a.tw[m];
-  for (int m = threadIdx.x; m < Plan<L>::kTab; m += kZThreads) tab[m] = a.tab[m];
-  __syncthreads();
-  const bool fin = (MODE == Z_PROJ) && a.loop_flag && *a.loop_flag == 1;
-  const int partner = (32 - lane) & 31;
+  const int l = lane % G, grp = lane / G, q = grp & 1, pr = grp >> 1;
+  float2* sw = tw + Z::kHead + warp * Z::RPW * Z::kRow;
+  float2* s = sw + grp * Z::kRow;
+  zrow_tables<N>(a, tw, tab);
+  const bool fin = MODE == Z_FINAL || (MODE == Z_PROJ && a.loop_flag && *a.loop_flag == 1);
+  const int partner = grp * G + (G - l) % G;
   const Geometry& g = a.g;
   // rows (ix, iy) of every y-plane, or of the planes [ybeg, ybeg + ycount)
-  const size_t nrows = a.ycount ? (size_t)N * a.ycount : (size_t)N * N;
+  const int nrows = a.ycount ? N * a.ycount : N * N;
+  auto row_of = [&](int lr) { return a.ycount ? (lr / a.ycount) * N + a.ybeg + lr % a.ycount : lr; };
 
-  for (size_t lr = (size_t)blockIdx.x * kZWarps + warp; lr < nrows; lr += (size_t)gridDim.x * kZWarps) {
-    const size_t row = a.ycount ? (lr / a.ycount) * N + a.ybeg + lr % a.ycount : lr;
-    const int ix = (int)(row / N), iy = (int)(row % N);
-    if (MODE == Z_PROJ && fin) {
-      float2 x[3][8], xl[3], A[3][4], B[3][4];
+  if (fin) {
+    // the real Psi: RPW rows of one component at a time
+    for (int it = blockIdx.x * kZWarps + warp; it < 3 * (nrows / Z::RPW); it += gridDim.x * kZWarps) {
+      const Field f = a.f[it / (nrows / Z::RPW)];
+      const size_t row = row_of((it % (nrows / Z::RPW)) * Z::RPW + grp);
+      float2 x[E], xl;
+      zrow_load<N>(f, row, l, x, xl);
+      zrow_merge<N>(x, xl, l, partner, tw);
+      zrow_fft<true, N>(x, s, tab, l);
+      float2* dst = f.M + row * L;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) zrow_load(a.f[q], row, lane, x[q], xl[q]);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) zrow_c2r(x[q], xl[q], lane, partner, tw, s, tab, A[q], B[q]);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        float2* dst = a.f[q].M + row * L;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          dst[lane + 64 * r] = A[q][r];
-          dst[lane + 32 + 64 * r] = B[q][r];
-        }
-      }
-      continue;
+      for (int r = 0; r < E; ++r) dst[l + G * r] = x[r];
     }
+    return;
+  }
+  if (MODE == Z_FINAL) return;
+  for (int it = blockIdx.x * kZWarps + warp; it < nrows / Z::PPW; it += gridDim.x * kZWarps) {
+    const int row = row_of(it * Z::PPW + pr);
+    const int ix = row / N, iy = row % N;
     const float dx = g.los_mode == 1 ? g.los.x : g.off[ix], dy = g.los_mode == 1 ? g.los.y : g.off[N + iy];
-    // the rows psi and dz psi at the points l + 64 r (A) and l + 32 + 64 r (B)
-    float2 A[2][4], B[2][4];
+    float2 v[E];   // C or Psi_z, then psi or dz psi, at the points l + G r
     if (MODE == Z_WARM || MODE == Z_USTART) {
-      float inv_f = 1.f, wx = 0.f, wy = 0.f;
+      float* crow = reinterpret_cast<float*>(sw + 2 * pr * Z::kRow);   // Z_WARM: the mesh row's coarse correction
+      float inv_f = 1.f;
       int nc = 1;
       if (MODE == Z_WARM) {
         // u = u_s + U[corr - ucoarse] (see the generic pass)
@@ -672,97 +679,79 @@ __global__ void __launch_bounds__(kZThreads, 2) zfused8_kernel(const ZArgs a) {
         inv_f = 1.f / (float)(1 << fl);
         const float tx = ((float)ix + 0.5f) * inv_f - 0.5f, ty = ((float)iy + 0.5f) * inv_f - 0.5f;
         const float fx = floorf(tx), fy = floorf(ty);
-        wx = tx - fx;
-        wy = ty - fy;
+        const float wx = tx - fx, wy = ty - fy;
         int x0 = (int)fx, y0 = (int)fy;
         x0 = x0 < 0 ? x0 + nc : x0;
         y0 = y0 < 0 ? y0 + nc : y0;
         const int x1 = x0 + 1 == nc ? 0 : x0 + 1, y1 = y0 + 1 == nc ? 0 : y0 + 1;
         const size_t r00 = ((size_t)x0 * nc + y0) * nc, r01 = ((size_t)x0 * nc + y1) * nc;
         const size_t r10 = ((size_t)x1 * nc + y0) * nc, r11 = ((size_t)x1 * nc + y1) * nc;
-        for (int jz = lane; jz < nc; jz += 32) {
+        for (int jz = q * G + l; jz < nc; jz += 2 * G) {
           const float c00 = a.corr[r00 + jz] - a.ucoarse[r00 + jz], c01 = a.corr[r01 + jz] - a.ucoarse[r01 + jz];
           const float c10 = a.corr[r10 + jz] - a.ucoarse[r10 + jz], c11 = a.corr[r11 + jz] - a.ucoarse[r11 + jz];
           crow[jz] = (1.f - wx) * ((1.f - wy) * c00 + wy * c01) + wx * ((1.f - wy) * c10 + wy * c11);
         }
         __syncwarp();
       }
-      const float2* ur = reinterpret_cast<const float2*>(a.u_in + row * N);
+      const float2* ur = reinterpret_cast<const float2*>(a.u_in + (size_t)row * N);
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int r = 0; r < E; ++r) {
+        const int m = l + G * r;
+        float2 uu = ur[m];
+        if (MODE == Z_WARM) {
+          float add[2];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int m = lane + 32 * h + 64 * r;
-          float2 uu = ur[m];
-          if (MODE == Z_WARM) {
-            float add[2];
-#pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-              const float tz = ((float)(2 * m + h2) + 0.5f) * inv_f - 0.5f;
-              const float fz = floorf(tz);
-              const float wz = tz - fz;
-              int z0 = (int)fz;
-              z0 = z0 < 0 ? z0 + nc : z0;
-              const int z1 = z0 + 1 == nc ? 0 : z0 + 1;
-              add[h2] = (1.f - wz) * crow[z0] + wz * crow[z1];
-            }
-            uu.x += add[0];
-            uu.y += add[1];
+          for (int h2 = 0; h2 < 2; ++h2) {
+            const float tz = ((float)(2 * m + h2) + 0.5f) * inv_f - 0.5f;
+            const float fz = floorf(tz);
+            const float wz = tz - fz;
+            int z0 = (int)fz;
+            z0 = z0 < 0 ? z0 + nc : z0;
+            const int z1 = z0 + 1 == nc ? 0 : z0 + 1;
+            add[h2] = (1.f - wz) * crow[z0] + wz * crow[z1];
           }
-          float dz0, dz1, w0, w1;
-          zrow_dw(g, dx, dy, m, dz0, dz1, w0, w1);
-          const float p0 = uu.x * w0, p1 = uu.y * w1;
-          (h ? B : A)[0][r] = make_float2(p0, p1);
-          (h ? B : A)[1][r] = make_float2(dz0 * p0, dz1 * p1);
+          uu.x += add[0];
+          uu.y += add[1];
         }
-      if (MODE == Z_WARM) __syncwarp();   // crow is rewritten by the next row
-    } else {
-      float2 x[3][8], xl[3];
-      if ((MODE == Z_PROJ || MODE == Z_RADIAL) && a.cform) {   // C and Psi_z from the inverse x pass
-        zrow_load(a.f[0], row, lane, x[0], xl[0]);
-        zrow_load(a.wf, row, lane, x[2], xl[2]);
-      } else {
-        // all three rows' loads in flight before the first transform; C = dx Psi_x + dy Psi_y
-#pragma unroll
-        for (int q = 0; q < 3; ++q) zrow_load(a.f[q], row, lane, x[q], xl[q]);
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-          x[0][r] = make_float2(fmaf(dx, x[0][r].x, dy * x[1][r].x), fmaf(dx, x[0][r].y, dy * x[1][r].y));
-        xl[0] = make_float2(fmaf(dx, xl[0].x, dy * xl[1].x), fmaf(dx, xl[0].y, dy * xl[1].y));
+        float dz0, dz1, w0, w1;
+        zrow_dw(g, dx, dy, m, dz0, dz1, w0, w1);
+        const float p0 = uu.x * w0, p1 = uu.y * w1;
+        v[r] = q ? make_float2(dz0 * p0, dz1 * p1) : make_float2(p0, p1);
       }
-      zrow_c2r(x[0], xl[0], lane, partner, tw, s, tab, A[0], B[0]);
-      zrow_c2r(x[2], xl[2], lane, partner, tw, s, tab, A[1], B[1]);
-      // u = coef (Psi . r) at the real points 2m, 2m + 1 of the complex point m (Eq. Nusser)
+      if (MODE == Z_WARM) __syncwarp();   // crow shares the rows' buffers
+    } else {
+      float2 xl;
+      zrow_load<N>(q ? a.wf : a.f[0], row, l, v, xl);
+      zrow_merge<N>(v, xl, l, partner, tw);
+      zrow_fft<true, N>(v, s, tab, l);
+      // u = coef (Psi . r) at the real points 2m, 2m + 1 of the complex point m (Eq. Nusser).  The two
+      // lane groups of a mesh row share the work: field 0's lanes form the points r < E/2 and field 1's
+      // the rest, and they swap what the other needs.
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int m = lane + 32 * h + 64 * r;
-          float dz0, dz1, w0, w1;
-          zrow_dw(g, dx, dy, m, dz0, dz1, w0, w1);
-          const float2 c = h ? B[0][r] : A[0][r], pz = h ? B[1][r] : A[1][r];
-          const float u0 = a.coef * (w0 * fmaf(dz0, pz.x, c.x));
-          const float u1 = a.coef * (w1 * fmaf(dz1, pz.y, c.y));
-          if (MODE == Z_RADIAL) {
-            reinterpret_cast<float2*>(a.u_out + row * N)[m] = make_float2(u0, u1);
-          } else {
-            const float p0 = u0 * w0, p1 = u1 * w1;
-            (h ? B : A)[0][r] = make_float2(p0, p1);
-            (h ? B : A)[1][r] = make_float2(dz0 * p0, dz1 * p1);
-          }
+      for (int r = 0; r < E / 2; ++r) {
+        const int rm = q ? r + E / 2 : r, m = l + G * rm;
+        const float2 mine = q ? v[r + E / 2] : v[r];
+        const float2 other = shfl2_xor(q ? v[r] : v[r + E / 2], G);
+        const float2 c = q ? other : mine, pz = q ? mine : other;
+        float dz0, dz1, w0, w1;
+        zrow_dw(g, dx, dy, m, dz0, dz1, w0, w1);
+        const float u0 = a.coef * (w0 * fmaf(dz0, pz.x, c.x));
+        const float u1 = a.coef * (w1 * fmaf(dz1, pz.y, c.y));
+        if (MODE == Z_RADIAL) {
+          reinterpret_cast<float2*>(a.u_out + (size_t)row * N)[m] = make_float2(u0, u1);
+        } else {
+          const float p0 = u0 * w0, p1 = u1 * w1;
+          const float2 psi = make_float2(p0, p1), zpsi = make_float2(dz0 * p0, dz1 * p1);
+          const float2 back = shfl2_xor(q ? psi : zpsi, G);   // the other field's value at this point
+          // field 0 keeps psi at r (own) and r + E/2 (from field 1); field 1 keeps dz psi likewise
+          v[r] = q ? back : psi;
+          v[r + E / 2] = q ? zpsi : back;
         }
+      }
       if (MODE == Z_RADIAL) continue;
     }
-    {
-      // the points l + 32 r of the real rows: A[r/2] (r even), B[(r-1)/2] (r odd)
-      float2 v[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = (r & 1) ? B[0][r >> 1] : A[0][r >> 1];
-      zrow_r2c(v, a.f[0], row, lane, partner, tw, s, tab);                      // psi^
-#pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = (r & 1) ? B[1][r >> 1] : A[1][r >> 1];
-      zrow_r2c(v, a.f[2], row, lane, partner, tw, s, tab);                      // Z^ = (dz psi)^
-    }
+    zrow_fft<false, N>(v, s, tab, l);
+    zrow_split_store<N>(v, q ? a.f[2] : a.f[0], row, l, partner, tw);   // psi^ and Z^ = (dz psi)^
   }
 }
 
@@ -777,28 +766,25 @@ struct ZDelta8 {
   static constexpr int L = N / 2, KT = 32, V = 16;
   static constexpr int kExt = N + KT + V;                       // staged entries per row
   static constexpr int kExtPad = kExt + kExt / 16 + 1;          // with one pad word per 16
-  static constexpr int TABZ = (Plan<L>::kTab + 1) & ~1;
-  static constexpr int kWarp = L + kExtPad;                      // float2: FFT buffer + two staged rows
-  static constexpr size_t smem = sizeof(float2) * ((size_t)L + 2 + TABZ + (size_t)kZWarps * kWarp);
+  static constexpr int kWarp = ZRow<N>::RPW * ZRow<N>::kRow + kExtPad;   // float2: FFT buffers + two staged rows
+  static constexpr size_t smem = sizeof(float2) * ((size_t)ZRow<N>::kHead + (size_t)kZWarps * kWarp);
   __device__ __forceinline__ static int pad(int p) { return p + (p >> 4); }
 };
 
 template <int N>
 __global__ void __launch_bounds__(kZThreads, 2) zdelta8_kernel(const ZArgs a) {
   using Z = ZDelta8<N>;
-  constexpr int L = Z::L, KT = Z::KT, V = Z::V;
-  using Lay = RowLayout<L>;
+  using ZR = ZRow<N>;
+  constexpr int L = Z::L, KT = Z::KT, V = Z::V, G = ZR::G, E = ZR::E;
   extern __shared__ float4 zsm[];
   float2* tw = reinterpret_cast<float2*>(zsm);
-  float2* tab = tw + L + 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* s = tab + Z::TABZ + warp * Z::kWarp;
-  float* xg = reinterpret_cast<float*>(s + L);                   // staged rho_g row, then rho_r row
+  float2* tab = tw + L + 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % G, grp = lane / G;
+  float2* sw = tw + ZR::kHead + warp * Z::kWarp;                 // the rows' FFT buffers
+  float* xg = reinterpret_cast<float*>(sw + ZR::RPW * ZR::kRow); // staged rho_g row, then rho_r row
   float* xr = xg + Z::kExtPad;
   __shared__ double red_sh[kZWarps];
-  for (int m = threadIdx.x; m <= L; m += kZThreads) tw[m] = a.tw[m];
-  for (int m = threadIdx.x; m < Plan<L>::kTab; m += kZThreads) tab[m] = a.tab[m];
-  __syncthreads();
+  zrow_tables<N>(a, tw, tab);
   float tp[KT];
 #pragma unroll
   for (int jt = 0; jt < KT; ++jt) tp[jt] = jt < a.ntap ? a.taps[jt] : 0.f;
@@ -806,67 +792,72 @@ __global__ void __launch_bounds__(kZThreads, 2) zdelta8_kernel(const ZArgs a) {
   const int nin = a.uniform ? 1 : 2;
   const float inv_alpha = a.uniform ? (float)((double)N * N * N / red[RED_SUM_WG]) : (float)(red[RED_SUM_WR] / red[RED_SUM_WG]);
   const float thr = a.uniform ? 0.f : (float)(a.mask_frac * red[RED_SUM_WR] / red[RED_CNT_RPOS]);
-  const int partner = (32 - lane) & 31;
+  const int partner = grp * G + (G - l) % G;
   float acc0 = 0.f, acc1 = 0.f;
 
-  for (size_t row = (size_t)blockIdx.x * kZWarps + warp; row < (size_t)N * N; row += (size_t)gridDim.x * kZWarps) {
-    const float* rg = reinterpret_cast<const float*>(a.f[0].M) + row * N;
-    const float* rr = reinterpret_cast<const float*>(a.f[1].M) + row * N;
-    for (int p = lane; p < Z::kExt; p += 32) {
-      int i = (p + a.t0) % N;
-      if (i < 0) i += N;
-      xg[Z::pad(p)] = rg[i];
-      if (nin == 2) xr[Z::pad(p)] = rr[i];
-    }
-    __syncwarp();
-    const int z0 = V * lane;
-    float ag[V], ar[V];
+  for (int it = blockIdx.x * kZWarps + warp; it < N * N / ZR::RPW; it += gridDim.x * kZWarps) {
+#pragma unroll 1
+    for (int i = 0; i < ZR::RPW; ++i) {
+      const size_t row = (size_t)it * ZR::RPW + i;
+      const float* rg = reinterpret_cast<const float*>(a.f[0].M) + row * N;
+      const float* rr = reinterpret_cast<const float*>(a.f[1].M) + row * N;
+      for (int p = lane; p < Z::kExt; p += 32) {
+        int src = (p + a.t0) % N;
+        if (src < 0) src += N;
+        xg[Z::pad(p)] = rg[src];
+        if (nin == 2) xr[Z::pad(p)] = rr[src];
+      }
+      __syncwarp();
+      const int z0 = V * lane;
+      float ag[V], ar[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) ag[v] = ar[v] = 0.f;
+      for (int v = 0; v < V; ++v) ag[v] = ar[v] = 0.f;
 #pragma unroll
-    for (int w = 0; w < KT + V - 1; ++w) {
-      const float g = xg[Z::pad(z0 + w)];
-      const float r = nin == 2 ? xr[Z::pad(z0 + w)] : 0.f;
+      for (int w = 0; w < KT + V - 1; ++w) {
+        const float g = xg[Z::pad(z0 + w)];
+        const float r = nin == 2 ? xr[Z::pad(z0 + w)] : 0.f;
 #pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const int jt = w - v;
-        if (jt >= 0 && jt < KT) {
-          ag[v] = fmaf(tp[jt], g, ag[v]);
-          if (nin == 2) ar[v] = fmaf(tp[jt], r, ar[v]);
+        for (int v = 0; v < V; ++v) {
+          const int jt = w - v;
+          if (jt >= 0 && jt < KT) {
+            ag[v] = fmaf(tp[jt], g, ag[v]);
+            if (nin == 2) ar[v] = fmaf(tp[jt], r, ar[v]);
+          }
         }
       }
-    }
-    float d[V];
+      float d[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      float q;   // 1 + delta, kept as the ratio for the logarithm (see the generic pass)
-      if (nin == 1) {
-        q = ag[v] * inv_alpha;
-      } else {
-        const bool in = ar[v] > thr;
-        q = in ? ag[v] * inv_alpha / ar[v] : 1.f;
-        acc1 += in ? 1.f : 0.f;
+      for (int v = 0; v < V; ++v) {
+        float q;   // 1 + delta, kept as the ratio for the logarithm (see the generic pass)
+        if (nin == 1) {
+          q = ag[v] * inv_alpha;
+        } else {
+          const bool in = ar[v] > thr;
+          q = in ? ag[v] * inv_alpha / ar[v] : 1.f;
+          acc1 += in ? 1.f : 0.f;
+        }
+        float dv = q - 1.f;
+        if (a.lognormal) {
+          dv = logf(fmaxf(q, 1e-6f));
+          acc0 += dv;
+        }
+        d[v] = dv;
       }
-      float dv = q - 1.f;
-      if (a.lognormal) {
-        dv = logf(fmaxf(q, 1e-6f));
-        acc0 += dv;
+      if (a.delta_real) {
+        float4* dr = reinterpret_cast<float4*>(a.delta_real + row * N + z0);
+#pragma unroll
+        for (int v4 = 0; v4 < V / 4; ++v4) dr[v4] = make_float4(d[4 * v4], d[4 * v4 + 1], d[4 * v4 + 2], d[4 * v4 + 3]);
       }
-      d[v] = dv;
+#pragma unroll
+      for (int k = 0; k < V / 2; ++k) sw[i * ZR::kRow + z0 / 2 + k] = make_float2(d[2 * k], d[2 * k + 1]);
+      __syncwarp();                       // the staged rows are rewritten by the next one
     }
-    if (a.delta_real) {
-      float4* dr = reinterpret_cast<float4*>(a.delta_real + row * N + z0);
+    float2 y[E];
 #pragma unroll
-      for (int v4 = 0; v4 < V / 4; ++v4) dr[v4] = make_float4(d[4 * v4], d[4 * v4 + 1], d[4 * v4 + 2], d[4 * v4 + 3]);
-    }
-#pragma unroll
-    for (int i = 0; i < V / 2; ++i) s[Lay::phys(z0 / 2 + i, 0)] = make_float2(d[2 * i], d[2 * i + 1]);
+    for (int r = 0; r < E; ++r) y[r] = sw[grp * ZR::kRow + l + G * r];
     __syncwarp();
-    float2 v8[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v8[r] = s[Lay::phys(lane + 32 * r, 0)];
-    __syncwarp();
-    zrow_r2c(v8, a.dout, row, lane, partner, tw, s, tab);
+    zrow_fft<false, N>(y, sw + grp * ZR::kRow, tab, l);
+    zrow_split_store<N>(y, a.dout, (size_t)it * ZR::RPW + grp, l, partner, tw);
   }
   const double r0 = block_sum((double)acc0, red_sh);
   const double r1 = block_sum((double)acc1, red_sh);
@@ -1193,101 +1184,125 @@ constexpr size_t spass_smem(int nslots) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// The k-space update along y for N = 512 = 8 x 8 x 8.  With three radix-8 Stockham stages the
-// butterfly j of the last forward stage produces X[j + 64 r] (r = 0..7), and these are exactly the
-// inputs of butterfly j of the first inverse stage.  So each thread loads its 8 points of a column
-// straight from global memory into the first forward stage, keeps the last forward stage's outputs
-// in registers for the source update, starts the inverse transform on them, and stores the last
-// inverse stage straight to global memory: two shared-memory round trips per transform instead of
-// three plus the staging of loads, stores and the update.  The arithmetic of every butterfly is the
-// same as in the generic stages.
+// The k-space passes along y of the register-fused family, N = 8 x M x 8 (M = N/64): the butterfly j
+// of the last forward stage produces X[j + (N/8) r] (r = 0..7), exactly the inputs of butterfly j of
+// the first inverse stage.  So each thread loads its 8 points of a column straight from global memory
+// into the first forward stage, keeps the last forward stage's outputs in registers for the source
+// update, starts the inverse transform on them, and stores the last inverse stage straight to global
+// memory: two shared-memory round trips per transform instead of three plus the staging of loads,
+// stores and the update.
+// A thread owns the edge butterfly j = tid / C of column tid % C; the middle stage's 64 butterflies of
+// each line are dealt over the same threads (N = 384: 48 threads a column, 192 a CTA and three CTAs per
+// SM, 488 us an update against 533 with 64 threads a column and two).
 // ------------------------------------------------------------------------------------------------
 template <int N, int C>
-struct KIter8 {
-  static_assert(N == 512, "three radix-8 stages");
-  static constexpr int T = (N / 8) * C;        // one butterfly of one column per thread and stage
-  static constexpr int kMinBlocks = T <= 256 ? 2 : 1;
+struct KFused {
+  static constexpr int M = N / 64;             // radix of the middle stage (64 butterflies a line)
+  static constexpr int NB = N / 8;             // edge butterflies a line
+  static constexpr int TPC = NB;               // threads per column, one edge butterfly each
+  static constexpr int T = TPC * C;
+  static constexpr int kMinBlocks = T <= 192 ? 3 : (T <= 256 ? 2 : 1);
+  static constexpr int OFF3 = (M - 1) * 8;     // the last stage's twiddles in the plan's table
   static constexpr int TAB = (Plan<N>::kTab + 1) & ~1;
-  // one buffer per transformed line: the x and z terms share one (see kiter8_kernel)
-  static constexpr size_t smem = sizeof(float2) * ((size_t)TAB + 2 * (size_t)N * C);
+  static constexpr size_t smem = sizeof(float2) * ((size_t)TAB + 2 * (size_t)N * C);   // one buffer per line
 };
 
-// The 512-point transforms of K lines of one column (K = 2 in the update: A and P_y forward, G and
+// Line and butterfly of a thread's p-th item of the middle stage (64 butterflies a line).
+template <int TPC>
+__device__ __forceinline__ int kline_item(int j, int p) {
+  if (64 % TPC == 0) return p / (64 / TPC < 1 ? 1 : 64 / TPC);   // whole lines: known when compiled
+  return (j + TPC * p) >> 6;
+}
+template <int TPC>
+__device__ __forceinline__ int kline_mid(int j, int p) {
+  if (64 % TPC == 0) return j + TPC * (p % (64 / TPC < 1 ? 1 : 64 / TPC));
+  return (j + TPC * p) & 63;
+}
+
+// The N-point transforms of K lines of one column (K = 2 in the update: A and P_y forward, G and
 // Psi_y inverse; K = 1 for delta), stage by stage together (one buffer each, so a stage needs one
-// barrier for all K): v[q][r] = x_q[j + 64 r] in, X_q[j + 64 r] out.
+// barrier for all K): v[q][r] = x_q[j + (N/8) r] in, X_q[j + (N/8) r] out.
 template <bool INV, int N, int C, int K>
-__device__ __forceinline__ void r512_lines(float2 (&v)[K][8], float2* __restrict__ s, const float2* __restrict__ tw,
-                                            int j, int col) {
+__device__ __forceinline__ void kline_fft(float2 (&v)[K][8], float2* __restrict__ s, const float2* __restrict__ tw,
+                                          int j, int col) {
+  using F = KFused<N, C>;
   using Lay = ColLayout<C>;
-  constexpr int B = N * C;
+  constexpr int B = N * C, M = F::M, PM = (64 * K + F::TPC - 1) / F::TPC;
 #pragma unroll
-  for (int q = 0; q < K; ++q) {                          // stage 1 (NS = 1): no twiddles
+  for (int q = 0; q < K; ++q) {                            // stage 1 (NS = 1): no twiddles
     Dft<8, INV>::run(v[q]);
 #pragma unroll
     for (int r = 0; r < 8; ++r) s[q * B + Lay::phys(8 * j + r, col)] = v[q][r];
   }
   __syncthreads();
-  const int k = j & 7;
+  float2 u[PM][M];                                         // stage 2 (NS = 8): items (line, butterfly)
 #pragma unroll
-  for (int q = 0; q < K; ++q) {                          // stage 2 (NS = 8)
+  for (int p = 0; p < PM; ++p) {
+    if ((64 * K) % F::TPC == 0 || j + F::TPC * p < 64 * K) {
+      const int q = kline_item<F::TPC>(j, p), jm = kline_mid<F::TPC>(j, p), k = jm & 7;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) v[q][r] = s[q * B + Lay::phys(j + 64 * r, col)];
+      for (int r = 0; r < M; ++r) u[p][r] = s[q * B + Lay::phys(jm + 64 * r, col)];
+#pragma unroll
+      for (int r = 1; r < M; ++r) {
+        float2 w = tw[(r - 1) * 8 + k];
+        if (INV) w.y = -w.y;
+        u[p][r] = cmul(u[p][r], w);
+      }
+      Dft<M, INV>::run(u[p]);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int p = 0; p < PM; ++p) {
+    if ((64 * K) % F::TPC == 0 || j + F::TPC * p < 64 * K) {
+      const int q = kline_item<F::TPC>(j, p), jm = kline_mid<F::TPC>(j, p), base = (jm >> 3) * (8 * M) + (jm & 7);
+#pragma unroll
+      for (int r = 0; r < M; ++r) s[q * B + Lay::phys(base + 8 * r, col)] = u[p][r];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < K; ++q) {                            // stage 3 (NS = N/8)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[q][r] = s[q * B + Lay::phys(j + F::NB * r, col)];
 #pragma unroll
     for (int r = 1; r < 8; ++r) {
-      float2 w = tw[(r - 1) * 8 + k];
+      float2 w = tw[F::OFF3 + (r - 1) * F::NB + j];
       if (INV) w.y = -w.y;
       v[q][r] = cmul(v[q][r], w);
     }
     Dft<8, INV>::run(v[q]);
   }
-  __syncthreads();
-  const int base = (j >> 3) * 64 + k;
-#pragma unroll
-  for (int q = 0; q < K; ++q)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) s[q * B + Lay::phys(base + 8 * r, col)] = v[q][r];
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < K; ++q) {                          // stage 3 (NS = 64)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[q][r] = s[q * B + Lay::phys(j + 64 * r, col)];
-#pragma unroll
-    for (int r = 1; r < 8; ++r) {
-      float2 w = tw[56 + (r - 1) * 64 + j];
-      if (INV) w.y = -w.y;
-      v[q][r] = cmul(v[q][r], w);
-    }
-    Dft<8, INV>::run(v[q]);
-  }
-  __syncthreads();                                       // the buffers are reused
+  __syncthreads();                                         // the buffers are reused
 }
 
-// The start's k-space pass along y for N = 512 (S_DELTA): the y transform of delta (unless delta(k)
+// The start's k-space pass along y (S_DELTA): the y transform of delta (unless delta(k)
 // is already stored), delta(k) and S_-1 = delta/b stored, Z[delta/b] with two inverse y transforms
 // (G and Psi_y, as the update kernel leaves them), the first and last stages in registers.
 template <int N, int C>
-__global__ void __launch_bounds__(KIter8<N, C>::T, KIter8<N, C>::kMinBlocks) kdelta8_kernel(const SArgs a) {
-  constexpr int T = KIter8<N, C>::T;
+__global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kdelta_fused_kernel(const SArgs a) {
+  constexpr int T = KFused<N, C>::T, NB = KFused<N, C>::NB;
   constexpr int H = N / 2;
   extern __shared__ float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
-  float2* s = tw + KIter8<N, C>::TAB;
+  float2* s = tw + KFused<N, C>::TAB;
   for (int m = threadIdx.x; m < Plan<N>::kTab; m += T) tw[m] = a.tab[m];
   const Tile t = tile_of<N, C, AX_Y>(blockIdx.x);
   const int col = threadIdx.x % C, j = threadIdx.x / C;
   float2* __restrict__ dkp = t.isQ ? a.dk.Q : a.dk.M;
   float2 d[1][8];
 #pragma unroll
-  for (int r = 0; r < 8; ++r) d[0][r] = dkp[t.base + (size_t)(j + 64 * r) * t.ls + (size_t)col * t.cs];
+  for (int r = 0; r < 8; ++r)
+    d[0][r] = dkp[t.base + (size_t)(j + NB * r) * t.ls + (size_t)col * t.cs];
   __syncthreads();   // twiddles
-  if (!a.d_is_k) r512_lines<false, N, C, 1>(d, s, tw, j, col);
+  if (!a.d_is_k) kline_fft<false, N, C, 1>(d, s, tw, j, col);
 
   const Geometry& g = a.g;
   float2* Sp = t.isQ ? a.sbuf.Q : a.sbuf.M;
   float2 v[2][8];
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int ky = j + 64 * r;
+    const int ky = j + NB * r;
     int ix, kz;
     if (!t.isQ) { ix = t.a; kz = t.c0 + col; } else { ix = t.c0 + col; kz = H; }
     const int mx = (ix < H) ? ix : ix - N;
@@ -1309,46 +1324,51 @@ __global__ void __launch_bounds__(KIter8<N, C>::T, KIter8<N, C>::kMinBlocks) kde
     v[0][r] = iS;
     v[1][r] = cscale(iS, kdy);
   }
-  r512_lines<true, N, C, 2>(v, s, tw, j, col);
-  {
-    // G (Psi_x = kdx G, Psi_z = kdz G) in the third field, Psi_y in the second, as the update
-    // kernel leaves them
-    float2* __restrict__ dy = t.isQ ? a.f[1].Q : a.f[1].M;
-    float2* __restrict__ dg = t.isQ ? a.f[2].Q : a.f[2].M;
+  kline_fft<true, N, C, 2>(v, s, tw, j, col);
+  // G (Psi_x = kdx G, Psi_z = kdz G) in the third field, Psi_y in the second, as the update
+  // kernel leaves them
+  float2* __restrict__ dy = t.isQ ? a.f[1].Q : a.f[1].M;
+  float2* __restrict__ dg = t.isQ ? a.f[2].Q : a.f[2].M;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const size_t gi = t.base + (size_t)(j + 64 * r) * t.ls + (size_t)col * t.cs;
-      dy[gi] = v[1][r];
-      dg[gi] = v[0][r];
-    }
+  for (int r = 0; r < 8; ++r) {
+    const size_t gi = t.base + (size_t)(j + NB * r) * t.ls + (size_t)col * t.cs;
+    dy[gi] = v[1][r];
+    dg[gi] = v[0][r];
   }
 }
 
-// The line transform along x for N = 512: the first radix-8 stage reads its inputs straight from
-// global memory and the last writes its outputs straight back, so shared memory carries only the
-// middle stage (the generic pass also stages the loads and stores).  Tiles of C adjacent columns,
-// 64 butterflies per column and stage, NB per thread.
-template <int C>
-struct XLine8 {
-  static constexpr int T = 512;
-  static constexpr int NB = 64 * C / T;        // butterflies per thread and stage
-  static constexpr int TAB = (Plan<512>::kTab + 1) & ~1;
-  static constexpr size_t smem = sizeof(float2) * ((size_t)TAB + (size_t)512 * C);
+// The line transform along x of the family: the first stage reads its inputs straight from global
+// memory and the last writes its outputs straight back, so shared memory carries only the middle
+// stage (the generic pass also stages the loads and stores).  Tiles of C adjacent columns; every
+// thread runs PE edge butterflies and PM middle ones of its column.
+template <int N, int C>
+struct XLine {
+  static constexpr int M = N / 64, NB = N / 8;
+  // 16 points a thread (8 at N = 256); the TPC threads of a column divide its edge butterflies
+  static constexpr int T = N == 384 ? 24 * C : (N == 256 ? 32 * C : (N == 512 ? 512 : 64 * C));
+  static constexpr int TPC = T / C;
+  static constexpr int PE = NB / TPC, PM = (64 + TPC - 1) / TPC;
+  static_assert(NB % TPC == 0, "edge butterflies divide evenly");
+  static constexpr int kMinBlocks = T > 512 ? 1 : (T <= 256 ? 4 : 2);
+  static constexpr int OFF3 = (M - 1) * 8;
+  static constexpr int TAB = (Plan<N>::kTab + 1) & ~1;
+  static constexpr size_t smem = sizeof(float2) * ((size_t)TAB + (size_t)N * C);
 };
 
-// The three radix-8 stages of a 512-point transform over C columns, the thread's NB butterflies
-// (j_b = jb + b T / C) with the first stage's inputs and the last stage's outputs handled one
-// butterfly at a time: ld(b, x) supplies x[r] = X[j_b + 64 r] and st(b, y) takes the outputs
-// y[r] = Y[j_b + 64 r], so only the middle stage holds all NB butterflies in registers (it reads
+// The three stages of an N-point transform over C columns, the thread's PE edge butterflies
+// (j_b = jb + b TPC) with the first stage's inputs and the last stage's outputs handled one
+// butterfly at a time: ld(b, x) supplies x[r] = X[j_b + (N/8) r] and st(b, y) takes the outputs
+// y[r] = Y[j_b + (N/8) r], so only the middle stage holds all its butterflies in registers (it reads
 // and writes shared memory in place).  Starts by writing s: a caller that ran it before syncs first.
-template <bool INV, int C, class Ld, class St>
-__device__ __forceinline__ void xline8_io(float2* __restrict__ s, const float2* __restrict__ tw, int jb, int col,
-                                          Ld&& ld, St&& st) {
-  constexpr int T = XLine8<C>::T, NB = XLine8<C>::NB;
+template <bool INV, int N, int C, class Ld, class St>
+__device__ __forceinline__ void xline_io(float2* __restrict__ s, const float2* __restrict__ tw, int jb, int col,
+                                         Ld&& ld, St&& st) {
+  using X = XLine<N, C>;
   using Lay = ColLayout<C>;
+  constexpr int M = X::M, TPC = X::TPC;
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {                          // stage 1 (NS = 1)
-    const int j = jb + b * (T / C);
+  for (int b = 0; b < X::PE; ++b) {                       // stage 1 (NS = 1)
+    const int j = jb + b * TPC;
     float2 x[8];
     ld(b, x);
     Dft<8, INV>::run(x);
@@ -1356,37 +1376,41 @@ __device__ __forceinline__ void xline8_io(float2* __restrict__ s, const float2* 
     for (int r = 0; r < 8; ++r) s[Lay::phys(8 * j + r, col)] = x[r];
   }
   __syncthreads();
-  float2 v[NB][8];
+  float2 v[X::PM][M];
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {                          // stage 2 (NS = 8)
-    const int j = jb + b * (T / C), k = j & 7;
+  for (int b = 0; b < X::PM; ++b) {                       // stage 2 (NS = 8)
+    const int j = jb + b * TPC, k = j & 7;
+    if (64 % TPC == 0 || j < 64) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) v[b][r] = s[Lay::phys(j + 64 * r, col)];
+      for (int r = 0; r < M; ++r) v[b][r] = s[Lay::phys(j + 64 * r, col)];
 #pragma unroll
-    for (int r = 1; r < 8; ++r) {
-      float2 w = tw[(r - 1) * 8 + k];
-      if (INV) w.y = -w.y;
-      v[b][r] = cmul(v[b][r], w);
+      for (int r = 1; r < M; ++r) {
+        float2 w = tw[(r - 1) * 8 + k];
+        if (INV) w.y = -w.y;
+        v[b][r] = cmul(v[b][r], w);
+      }
+      Dft<M, INV>::run(v[b]);
     }
-    Dft<8, INV>::run(v[b]);
   }
   __syncthreads();
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const int j = jb + b * (T / C), base = (j >> 3) * 64 + (j & 7);
+  for (int b = 0; b < X::PM; ++b) {
+    const int j = jb + b * TPC, base = (j >> 3) * (8 * M) + (j & 7);
+    if (64 % TPC == 0 || j < 64) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) s[Lay::phys(base + 8 * r, col)] = v[b][r];
+      for (int r = 0; r < M; ++r) s[Lay::phys(base + 8 * r, col)] = v[b][r];
+    }
   }
   __syncthreads();
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {                          // stage 3 (NS = 64)
-    const int j = jb + b * (T / C);
+  for (int b = 0; b < X::PE; ++b) {                       // stage 3 (NS = N/8)
+    const int j = jb + b * TPC;
     float2 y[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) y[r] = s[Lay::phys(j + 64 * r, col)];
+    for (int r = 0; r < 8; ++r) y[r] = s[Lay::phys(j + X::NB * r, col)];
 #pragma unroll
     for (int r = 1; r < 8; ++r) {
-      float2 w = tw[56 + (r - 1) * 64 + j];
+      float2 w = tw[X::OFF3 + (r - 1) * X::NB + j];
       if (INV) w.y = -w.y;
       y[r] = cmul(y[r], w);
     }
@@ -1418,12 +1442,12 @@ __device__ __forceinline__ uint32_t opaque_u32(uint32_t x) {
   return x;
 }
 
-template <bool INV, int C, bool PAIR>
-__global__ void __launch_bounds__(XLine8<C>::T, 2) xline8_kernel(const SArgs a) {
-  constexpr int N = 512, H = N / 2, T = XLine8<C>::T, NB = XLine8<C>::NB;
+template <bool INV, int N, int C, bool PAIR>
+__global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline_kernel(const SArgs a) {
+  constexpr int H = N / 2, T = XLine<N, C>::T, TPC = XLine<N, C>::TPC, NB = XLine<N, C>::NB;
   extern __shared__ float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
-  float2* s = tw + XLine8<C>::TAB;
+  float2* s = tw + XLine<N, C>::TAB;
   if (!INV && a.skip_flag && *a.skip_flag != 0) return;   // uniform: device loop already converged
   for (int m = threadIdx.x; m < Plan<N>::kTab; m += T) tw[m] = a.tab[m];
   const int role = PAIR ? (int)(blockIdx.x & 1) : (int)blockIdx.y;
@@ -1441,7 +1465,7 @@ __global__ void __launch_bounds__(XLine8<C>::T, 2) xline8_kernel(const SArgs a) 
   const uint32_t ls = (uint32_t)t.ls;
   // element offset of point (b, r) of this thread; every load and store re-derives the base through
   // an opaque copy, so no offset is kept live across a transform
-  auto off = [&](uint32_t base, int b, int r) { return base + (uint32_t)(b * (T / C) + 64 * r) * ls; };
+  auto off = [&](uint32_t base, int b, int r) { return base + (uint32_t)(b * TPC + NB * r) * ls; };
   auto load = [&](const float2* __restrict__ P) {
     return [=, &off](int b, float2 (&x)[8]) {
 #pragma unroll
@@ -1459,7 +1483,7 @@ __global__ void __launch_bounds__(XLine8<C>::T, 2) xline8_kernel(const SArgs a) 
   const bool cf = PAIR && INV && a.cform && !(a.loop_flag && *a.loop_flag == 1);
   if (!PAIR || (INV && role == 1 && !cf)) {
     float2* __restrict__ P = t.isQ ? a.f[role].Q : a.f[role].M;
-    xline8_io<INV, C>(s, tw, jb, col, load(P), store(P, 1.f));
+    xline_io<INV, N, C>(s, tw, jb, col, load(P), store(P, 1.f));
     return;
   }
   float2* __restrict__ P0 = t.isQ ? a.f[0].Q : a.f[0].M;
@@ -1467,17 +1491,17 @@ __global__ void __launch_bounds__(XLine8<C>::T, 2) xline8_kernel(const SArgs a) 
   float2* __restrict__ P2 = t.isQ ? a.f[2].Q : a.f[2].M;
   const float dy = g.los_mode == 1 ? g.los.y : g.off[N + (t.isQ ? t.c0 + col : t.a)];
   if (!INV && role == 1) {   // P_y = dy FFT_x(psi^)
-    xline8_io<INV, C>(s, tw, jb, col, load(P0), store(P1, dy));
+    xline_io<INV, N, C>(s, tw, jb, col, load(P0), store(P1, dy));
     return;
   }
   const float kf = g.kf;
   const float kdz = t.isQ ? 0.f : kf * (float)(t.c0 + col);   // M tiles: kz < N/2; Q tiles: kz = N/2
   // the line index i is kx in Fourier space and x in configuration space
   auto kdx = [&](int b, int r) {
-    const int i = jb + b * (T / C) + 64 * r;
+    const int i = jb + b * TPC + NB * r;
     return i == H ? 0.f : kf * (float)(i < H ? i : i - N);
   };
-  auto dxv = [&](int b, int r) { return g.los_mode == 1 ? g.los.x : g.off[jb + b * (T / C) + 64 * r]; };
+  auto dxv = [&](int b, int r) { return g.los_mode == 1 ? g.los.x : g.off[jb + b * TPC + NB * r]; };
   // loads of G scaled by kdx (the inverse's x component)
   auto load_kdx_g = [&](int b, float2 (&x)[8]) {
 #pragma unroll
@@ -1487,14 +1511,14 @@ __global__ void __launch_bounds__(XLine8<C>::T, 2) xline8_kernel(const SArgs a) 
     // both roles start on G, so the pair reads it from HBM once
     if (role == 1) {   // Psi_z = kdz IFFT_x(G)
       float2* __restrict__ W = t.isQ ? a.wf.Q : a.wf.M;
-      xline8_io<INV, C>(s, tw, jb, col, load(P2), store(W, kdz));
+      xline_io<INV, N, C>(s, tw, jb, col, load(P2), store(W, kdz));
       return;
     }
     // role 0: Psi_x = IFFT_x(kdx G) parked in the first field, then C = fmaf(dx, Psi_x, dy Psi_y),
     // rounded exactly as the projection pass forms it from the three components
-    xline8_io<INV, C>(s, tw, jb, col, load_kdx_g, store(P0, 1.f));
+    xline_io<INV, N, C>(s, tw, jb, col, load_kdx_g, store(P0, 1.f));
     __syncthreads();   // s is rewritten by the second transform
-    xline8_io<INV, C>(s, tw, jb, col, load(P1), [&](int b, const float2 (&y)[8]) {   // IFFT_x(Psi_y)
+    xline_io<INV, N, C>(s, tw, jb, col, load(P1), [&](int b, const float2 (&y)[8]) {   // IFFT_x(Psi_y)
       const uint32_t o = opaque_u32(o0);
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
@@ -1506,15 +1530,15 @@ __global__ void __launch_bounds__(XLine8<C>::T, 2) xline8_kernel(const SArgs a) 
     return;
   }
   if (INV) {   // three components: Psi_x = IFFT_x(kdx G) into the first field, Psi_z = kdz IFFT_x(G)
-    xline8_io<INV, C>(s, tw, jb, col, load_kdx_g, store(P0, 1.f));
+    xline_io<INV, N, C>(s, tw, jb, col, load_kdx_g, store(P0, 1.f));
     __syncthreads();   // s is rewritten by the second transform
-    xline8_io<INV, C>(s, tw, jb, col, load(P2), store(P2, kdz));
+    xline_io<INV, N, C>(s, tw, jb, col, load(P2), store(P2, kdz));
     return;
   }
   // forward: kdz FFT_x(Z^) into the third field, then A = kdx FFT_x(dx psi^) + that
-  xline8_io<INV, C>(s, tw, jb, col, load(P2), store(P2, kdz));
+  xline_io<INV, N, C>(s, tw, jb, col, load(P2), store(P2, kdz));
   __syncthreads();   // s is rewritten by the second transform
-  xline8_io<INV, C>(s, tw, jb, col,
+  xline_io<INV, N, C>(s, tw, jb, col,
                     [&](int b, float2 (&x)[8]) {
 #pragma unroll
                       for (int r = 0; r < 8; ++r) x[r] = cscale(P0[off(o0, b, r)], dxv(b, r));
@@ -1550,13 +1574,14 @@ __device__ __forceinline__ void kiter_tile(const SArgs& a, const Tile& t, float2
   const float kx = g.kf * mx, kzf = g.kf * kz;
   const float kdx = (ix == H) ? 0.f : kx;
   const float kdz = (kz == H) ? 0.f : kzf;
-  r512_lines<false, N, C, 2>(v, s, tw, j, col);
+  constexpr int NB = KFused<N, C>::NB;
+  kline_fft<false, N, C, 2>(v, s, tw, j, col);
   float2* Sp = t.isQ ? a.sbuf.Q : a.sbuf.M;
   const float kxz2 = kx * kx + kzf * kzf, kdxz2 = kdx * kdx + kdz * kdz;
   const float wgt = (kz == 0 || kz == H) ? 1.f : 2.f;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int ky = j + 64 * r;
+    const int ky = j + NB * r;
     const int my = (ky < H) ? ky : ky - N;
     const float kyf = g.kf * my;
     const float k2 = kxz2 + kyf * kyf;
@@ -1576,12 +1601,12 @@ __device__ __forceinline__ void kiter_tile(const SArgs& a, const Tile& t, float2
     v[0][r] = iS;
     v[1][r] = cscale(iS, kdy);
   }
-  r512_lines<true, N, C, 2>(v, s, tw, j, col);
+  kline_fft<true, N, C, 2>(v, s, tw, j, col);
   float2* __restrict__ dy = t.isQ ? a.f[1].Q : a.f[1].M;
   float2* __restrict__ dg = t.isQ ? a.f[2].Q : a.f[2].M;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const size_t gi = t.base + (size_t)(j + 64 * r) * t.ls + (size_t)col * t.cs;
+    const size_t gi = t.base + (size_t)(j + NB * r) * t.ls + (size_t)col * t.cs;
     dy[gi] = v[1][r];
     dg[gi] = v[0][r];
   }
@@ -1593,9 +1618,10 @@ __device__ __forceinline__ void kiter_load(const SArgs& a, const Tile& t, int j,
                                            float2 (&dk)[8], float2 (&sp)[8]) {
   const float2* __restrict__ dkp = t.isQ ? a.dk.Q : a.dk.M;
   const float2* __restrict__ spp = t.isQ ? a.sbuf.Q : a.sbuf.M;
+  constexpr int NB = KFused<N, C>::NB;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const size_t gi = t.base + (size_t)(j + 64 * r) * t.ls + (size_t)col * t.cs;
+    const size_t gi = t.base + (size_t)(j + NB * r) * t.ls + (size_t)col * t.cs;
     v[0][r] = (t.isQ ? a.f[2].Q : a.f[2].M)[gi];
     v[1][r] = (t.isQ ? a.f[1].Q : a.f[1].M)[gi];
     dk[r] = dkp[gi];
@@ -1604,11 +1630,11 @@ __device__ __forceinline__ void kiter_load(const SArgs& a, const Tile& t, int j,
 }
 
 template <int N, int C>
-__global__ void __launch_bounds__(KIter8<N, C>::T, KIter8<N, C>::kMinBlocks) kiter8_kernel(const SArgs a) {
-  constexpr int T = KIter8<N, C>::T;
+__global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kiter_fused_kernel(const SArgs a) {
+  constexpr int T = KFused<N, C>::T;
   extern __shared__ float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
-  float2* s = tw + KIter8<N, C>::TAB;
+  float2* s = tw + KFused<N, C>::TAB;
   __shared__ double red_sh[T / 32];
   for (int m = threadIdx.x; m < Plan<N>::kTab; m += T) tw[m] = a.tab[m];
   const Tile t = tile_of<N, C, AX_Y>(blockIdx.x);
@@ -1639,8 +1665,8 @@ __global__ void __launch_bounds__(KIter8<N, C>::T, KIter8<N, C>::kMinBlocks) kit
 // stops with RECON_ERR_NONFINITE) and the CTA returns.
 template <int N, int C>
 struct KTma {
-  static constexpr int T = KIter8<N, C>::T;
-  static constexpr size_t kS = sizeof(float2) * ((size_t)KIter8<N, C>::TAB + 2 * (size_t)N * C);
+  static constexpr int T = KFused<N, C>::T;
+  static constexpr size_t kS = sizeof(float2) * ((size_t)KFused<N, C>::TAB + 2 * (size_t)N * C);
   static constexpr size_t kBufOff = (kS + 127) & ~(size_t)127;
   static constexpr size_t kField = sizeof(float2) * (size_t)N * C;   // one field's tile
   static constexpr size_t kBarOff = kBufOff + 4 * kField;
@@ -1672,14 +1698,14 @@ __device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity) {
 }
 
 template <int N, int C>
-__global__ void __launch_bounds__(KIter8<N, C>::T, 2) kiter8_tma_kernel(const SArgs a,
+__global__ void __launch_bounds__(KFused<N, C>::T, 2) kiter_tma_kernel(const SArgs a,
                                                                        const __grid_constant__ KIterMaps maps) {
   using K = KTma<N, C>;
   constexpr int T = K::T, H = N / 2, MT = N * (H / C), QT = N / C;
   constexpr int kGridPartials = MT + QT;   // the regular grid whose partials the reduction reads
   extern __shared__ __align__(128) float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
-  float2* s = tw + KIter8<N, C>::TAB;
+  float2* s = tw + KFused<N, C>::TAB;
   const float2* buf = reinterpret_cast<const float2*>(reinterpret_cast<char*>(ssm) + K::kBufOff);
   uint64_t* bar_p = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ssm) + K::kBarOff);
   __shared__ double red_sh[T / 32];
@@ -1814,10 +1840,10 @@ struct MeshImpl {
 
   template <int M_>
   static cudaError_t zfused(const ZArgs& a, cudaStream_t st, int* grid_out) {
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       static int grid = 0;
-      const void* k = (const void*)zfused8_kernel<N, M_>;
-      const size_t smem = ZProj8<N>::smem;
+      const void* k = (const void*)zfused_kernel<N, M_>;
+      const size_t smem = ZRow<N>::smem;
       if (grid == 0) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1863,8 +1889,11 @@ struct MeshImpl {
   static cudaError_t zpass(int mode, int nc, const ZArgs& a, cudaStream_t st, int* grid_out) {
     if constexpr (N == 512) {
       if (mode == Z_DELTA && nc == 2 && !a.generic && a.ntap <= ZDelta8<N>::KT) return zdelta_fused(a, st, grid_out);
+    }
+    if constexpr (kFusedMesh<N>) {
       if (nc == 3 && !a.generic) {
         if (mode == Z_PROJ) return zfused<Z_PROJ>(a, st, grid_out);
+        if (mode == Z_FINAL) return zfused<Z_FINAL>(a, st, grid_out);
         if (mode == Z_RADIAL) return zfused<Z_RADIAL>(a, st, grid_out);
         if (mode == Z_WARM && a.clevel >= 1) return zfused<Z_WARM>(a, st, grid_out);
         if (mode == Z_USTART) return zfused<Z_USTART>(a, st, grid_out);
@@ -1894,62 +1923,65 @@ struct MeshImpl {
   }
 
   static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       constexpr int C = SCols<N, S_ITER>::v;
-      if (a.tmaps) {   // inputs streamed by TMA into persistent CTAs, two per SM
-        const void* k = (const void*)kiter8_tma_kernel<N, C>;
-        static int grid = 0;
-        if (grid == 0) {
-          cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KTma<N, C>::smem);
-          if (e != cudaSuccess) return e;
-          int dev = 0, sm = 0, occ = 0;
-          if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-          if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-          if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, KTma<N, C>::T, KTma<N, C>::smem)) != cudaSuccess)
-            return e;
-          if (occ < 1) return cudaErrorInvalidConfiguration;
-          grid = occ * sm;
+      if constexpr (N == 512) {
+        if (a.tmaps) {   // inputs streamed by TMA into persistent CTAs, two per SM
+          const void* k = (const void*)kiter_tma_kernel<N, C>;
+          static int grid = 0;
+          if (grid == 0) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KTma<N, C>::smem);
+            if (e != cudaSuccess) return e;
+            int dev = 0, sm = 0, occ = 0;
+            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+            if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, KTma<N, C>::T, KTma<N, C>::smem)) != cudaSuccess)
+              return e;
+            if (occ < 1) return cudaErrorInvalidConfiguration;
+            grid = occ * sm;
+          }
+          void* args[] = {const_cast<SArgs*>(&a), const_cast<KIterMaps*>(a.tmaps)};
+          return cudaLaunchKernel(k, dim3(grid), dim3(KTma<N, C>::T), args, KTma<N, C>::smem, st);
         }
-        void* args[] = {const_cast<SArgs*>(&a), const_cast<KIterMaps*>(a.tmaps)};
-        return cudaLaunchKernel(k, dim3(grid), dim3(KTma<N, C>::T), args, KTma<N, C>::smem, st);
       }
-      const void* k = (const void*)kiter8_kernel<N, C>;
+      const void* k = (const void*)kiter_fused_kernel<N, C>;
       static bool attr = false;
       if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KIter8<N, C>::smem);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KFused<N, C>::smem);
         if (e != cudaSuccess) return e;
         attr = true;
       }
       void* args[] = {const_cast<SArgs*>(&a)};
-      return cudaLaunchKernel(k, dim3(sblocks<S_ITER>()), dim3(KIter8<N, C>::T), args, KIter8<N, C>::smem, st);
+      return cudaLaunchKernel(k, dim3(sblocks<S_ITER>()), dim3(KFused<N, C>::T), args, KFused<N, C>::smem, st);
     }
     return cudaErrorInvalidValue;
   }
 
   static cudaError_t dlaunch(const SArgs& a, cudaStream_t st) {
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       constexpr int C = SCols<N, S_DELTA>::v;
-      const void* k = (const void*)kdelta8_kernel<N, C>;
+      const void* k = (const void*)kdelta_fused_kernel<N, C>;
       static bool attr = false;
       if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KIter8<N, C>::smem);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KFused<N, C>::smem);
         if (e != cudaSuccess) return e;
         attr = true;
       }
       void* args[] = {const_cast<SArgs*>(&a)};
-      return cudaLaunchKernel(k, dim3(sblocks<S_DELTA>()), dim3(KIter8<N, C>::T), args, KIter8<N, C>::smem, st);
+      return cudaLaunchKernel(k, dim3(sblocks<S_DELTA>()), dim3(KFused<N, C>::T), args, KFused<N, C>::smem, st);
     }
     return cudaErrorInvalidValue;
   }
 
-  // x lines for N = 512: C = 16 (128-byte rows) or 8 columns (line tile option); pair: the vector
-  // passes of the register-fused k-space path (two CTA kinds along gridDim.y, see xline8_kernel)
+  // x lines of the family: C = 16 (128-byte rows) or 8 columns (line tile option); pair: the vector
+  // passes of the register-fused k-space path (two CTA kinds on adjacent block indices, see xline_kernel)
   template <int C, bool PAIR>
   static cudaError_t xlaunch_c(bool inv, const SArgs& a, cudaStream_t st, int ncomp) {
-    const void* k = inv ? (const void*)xline8_kernel<true, C, PAIR> : (const void*)xline8_kernel<false, C, PAIR>;
+    using X = XLine<N, C>;
+    const void* k = inv ? (const void*)xline_kernel<true, N, C, PAIR> : (const void*)xline_kernel<false, N, C, PAIR>;
     static bool attr[2] = {false, false};
     if (!attr[inv]) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XLine8<C>::smem);
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::smem);
       if (e != cudaSuccess) return e;
       attr[inv] = true;
     }
@@ -1958,23 +1990,22 @@ struct MeshImpl {
     const int tiles = a.ycount ? a.ycount * ((N / 2) / C) + a.ycount / C : N * ((N / 2) / C) + N / C;
     // pairs: the two CTAs of a tile on adjacent block indices; single fields: components along y
     const dim3 grid = PAIR ? dim3(2 * tiles) : dim3(tiles, ncomp);
-    return cudaLaunchKernel(k, grid, dim3(XLine8<C>::T), args, XLine8<C>::smem, st);
+    return cudaLaunchKernel(k, grid, dim3(X::T), args, X::smem, st);
   }
   static cudaError_t xlaunch(bool inv, const SArgs& a, cudaStream_t st, int ncomp, bool pair) {
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       if (pair) return a.narrow ? xlaunch_c<8, true>(inv, a, st, ncomp) : xlaunch_c<16, true>(inv, a, st, ncomp);
       return xlaunch_c<16, false>(inv, a, st, ncomp);
     }
     return cudaErrorInvalidValue;
   }
 
-
   static cudaError_t spass(int mode, int nc, int axis, const SArgs& a, cudaStream_t st) {
     if (nc < 1 || nc > 3) return cudaErrorInvalidValue;
     // plain passes: one component per CTA, components along gridDim.y
     if (mode == S_FWD && axis == AX_Y) return slaunch<S_FWD, 1, AX_Y>(a, st, nc);
     if (mode == S_INV && axis == AX_Y) return slaunch<S_INV, 1, AX_Y>(a, st, nc);
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       // the vector x passes next to the register-fused k-space passes carry their representation
       if ((mode == S_FWD || mode == S_INV) && axis == AX_X && !a.generic && nc == 3)
         return xlaunch(mode == S_INV, a, st, nc, true);
@@ -1985,16 +2016,12 @@ struct MeshImpl {
       return a.narrow ? slaunch<S_FWD, 1, AX_X, 1>(a, st, nc) : slaunch<S_FWD, 1, AX_X>(a, st, nc);
     if (mode == S_INV && axis == AX_X)
       return a.narrow ? slaunch<S_INV, 1, AX_X, 1>(a, st, nc) : slaunch<S_INV, 1, AX_X>(a, st, nc);
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       if (mode == S_DELTA && axis == AX_Y && !a.generic) return dlaunch(a, st);
+      if (mode == S_ITER && axis == AX_Y && nc == 3 && !a.generic) return klaunch(a, st);
     }
     if (mode == S_DELTA && axis == AX_Y) return slaunch<S_DELTA, 1, AX_Y>(a, st, 1);
-    if (mode == S_ITER && axis == AX_Y && nc == 3) {
-      if constexpr (N == 512) {
-        if (!a.generic) return klaunch(a, st);
-      }
-      return slaunch<S_ITER, 3, AX_Y>(a, st, 1);
-    }
+    if (mode == S_ITER && axis == AX_Y && nc == 3) return slaunch<S_ITER, 3, AX_Y>(a, st, 1);
     return cudaErrorInvalidValue;
   }
 
@@ -2004,7 +2031,7 @@ struct MeshImpl {
   }
 
   static const MeshKernels* table() {
-    static const MeshKernels t = {N, kZBlocks, kSBlocks, Plan<N>::kTab, Plan<N / 2>::kTab, N == 512 ? 1 : 0,
+    static const MeshKernels t = {N, kZBlocks, kSBlocks, Plan<N>::kTab, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0,
                                   &zpass, &spass, &build_tables};
     return &t;
   }

@@ -770,7 +770,7 @@ recon_status recon_create(const recon_params* p, void* stream, void* workspace, 
     rs = RECON_ERR_CUDA;
   }
   if (rs == RECON_OK) rs = configure(h, p);
-  if (rs == RECON_OK && h->mk->kspace_fused) h->tmaps_ok = encode_kiter_maps(h);
+  if (rs == RECON_OK && n == 512) h->tmaps_ok = encode_kiter_maps(h);
   if (rs != RECON_OK) {
     if (h->own_ws) cudaFree(h->ws);
     delete h;
