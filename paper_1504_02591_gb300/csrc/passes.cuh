@@ -1337,85 +1337,67 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kde
   }
 }
 
-// The line transform along x of the family: the first stage reads its inputs straight from global
-// memory and the last writes its outputs straight back, so shared memory carries only the middle
-// stage (the generic pass also stages the loads and stores).  Tiles of C adjacent columns; every
-// thread runs PE edge butterflies and PM middle ones of its column.
+// The line transform along x of the family, N = E x G with G threads a column and E points a thread:
+// a radix-E butterfly per thread straight from global memory (points jb + G r), one exchange through
+// shared memory, and E / G radix-G butterflies per thread straight back (points jb + G h + E r; N = 384
+// has 24 of them for 16 threads, so threads jb < 8 run a second one).  Tiles of C adjacent columns.
+// The three-stage form (8 x M x 8) kept the L1's shared-memory pipe 60% busy and spilled; one exchange
+// and two barriers a transform instead of two and four, inverse / forward us: 256 85 / 76 -> 68 / 70,
+// 384 268 / 246 -> 227 / 230, 512 608 / 585 -> 585 / 573, 1024 5735 / 5660 -> 5580 / 5590.  What is left
+// is load latency: two to four CTAs an SM overlap their load, transform and store phases only partly
+// (reading lines at a 2 KB instead of a 1 MB stride changes nothing, 579 / 556 at 512).
 template <int N, int C>
 struct XLine {
-  static constexpr int M = N / 64, NB = N / 8;
-  // 16 points a thread (8 at N = 256); the TPC threads of a column divide its edge butterflies
-  static constexpr int T = N == 384 ? 24 * C : (N == 256 ? 32 * C : (N == 512 ? 512 : 64 * C));
-  static constexpr int TPC = T / C;
-  static constexpr int PE = NB / TPC, PM = (64 + TPC - 1) / TPC;
-  static_assert(NB % TPC == 0, "edge butterflies divide evenly");
-  static constexpr int kMinBlocks = T > 512 ? 1 : (T <= 256 ? 4 : 2);
-  static constexpr int OFF3 = (M - 1) * 8;
-  static constexpr int TAB = (Plan<N>::kTab + 1) & ~1;
+  static constexpr int G = N == 1024 ? 32 : 16;
+  static constexpr int E = N / G;              // 16, 24, 32, 32
+  static constexpr int H = (E + G - 1) / G;    // second-stage butterflies a thread
+  static constexpr int T = G * C;
+  // CTAs per SM that the points a thread holds leave registers for (384 at 2, 3 CTAs: 274, 227 us inverse)
+  static constexpr int kSM = E == 16 ? 4 : (E == 24 ? 3 : 2);
+  static constexpr int kMinBlocks = T > 256 ? 1 : (T == 256 ? kSM : 2 * kSM);
+  static constexpr int kTab = (G - 1) * E;     // second-stage twiddles [r - 1][j] = exp(-2 pi i r j / N)
+  static constexpr int TAB = (kTab + 1) & ~1;
   static constexpr size_t smem = sizeof(float2) * ((size_t)TAB + (size_t)N * C);
+  // row i of the tile, i = E q + r: with 8 columns a 128-byte wavefront holds two rows, whose low bits
+  // must differ both for writes (consecutive q) and reads (consecutive r)
+  __device__ __forceinline__ static int row(int q, int r, int col) {
+    return (E * q + (C == 8 ? r ^ (q & 1) : r)) * C + col;
+  }
 };
+template <int N>
+constexpr int kXTab = kFusedMesh<N> ? (XLine<N, 16>::kTab + 1) & ~1 : 0;
 
-// The three stages of an N-point transform over C columns, the thread's PE edge butterflies
-// (j_b = jb + b TPC) with the first stage's inputs and the last stage's outputs handled one
-// butterfly at a time: ld(b, x) supplies x[r] = X[j_b + (N/8) r] and st(b, y) takes the outputs
-// y[r] = Y[j_b + (N/8) r], so only the middle stage holds all its butterflies in registers (it reads
-// and writes shared memory in place).  Starts by writing s: a caller that ran it before syncs first.
+// One N-point transform of the tile's columns: ld(x) supplies x[r] = X[jb + G r], st(h, y) takes
+// y[r] = Y[jb + G h + E r].  Starts by writing s: a caller that ran it before syncs first.
 template <bool INV, int N, int C, class Ld, class St>
 __device__ __forceinline__ void xline_io(float2* __restrict__ s, const float2* __restrict__ tw, int jb, int col,
                                          Ld&& ld, St&& st) {
   using X = XLine<N, C>;
-  using Lay = ColLayout<C>;
-  constexpr int M = X::M, TPC = X::TPC;
+  constexpr int E = X::E, G = X::G;
+  {
+    float2 x[E];
+    ld(x);
+    Dft<E, INV>::run(x);
 #pragma unroll
-  for (int b = 0; b < X::PE; ++b) {                       // stage 1 (NS = 1)
-    const int j = jb + b * TPC;
-    float2 x[8];
-    ld(b, x);
-    Dft<8, INV>::run(x);
-#pragma unroll
-    for (int r = 0; r < 8; ++r) s[Lay::phys(8 * j + r, col)] = x[r];
+    for (int r = 0; r < E; ++r) s[X::row(jb, r, col)] = x[r];
   }
   __syncthreads();
-  float2 v[X::PM][M];
 #pragma unroll
-  for (int b = 0; b < X::PM; ++b) {                       // stage 2 (NS = 8)
-    const int j = jb + b * TPC, k = j & 7;
-    if (64 % TPC == 0 || j < 64) {
+  for (int h = 0; h < X::H; ++h) {
+    const int j = jb + G * h;
+    if (E % G == 0 || j < E) {
+      float2 y[G];
 #pragma unroll
-      for (int r = 0; r < M; ++r) v[b][r] = s[Lay::phys(j + 64 * r, col)];
+      for (int r = 0; r < G; ++r) y[r] = s[X::row(r, j, col)];
 #pragma unroll
-      for (int r = 1; r < M; ++r) {
-        float2 w = tw[(r - 1) * 8 + k];
+      for (int r = 1; r < G; ++r) {
+        float2 w = tw[(r - 1) * E + j];
         if (INV) w.y = -w.y;
-        v[b][r] = cmul(v[b][r], w);
+        y[r] = cmul(y[r], w);
       }
-      Dft<M, INV>::run(v[b]);
+      Dft<G, INV>::run(y);
+      st(h, y);
     }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int b = 0; b < X::PM; ++b) {
-    const int j = jb + b * TPC, base = (j >> 3) * (8 * M) + (j & 7);
-    if (64 % TPC == 0 || j < 64) {
-#pragma unroll
-      for (int r = 0; r < M; ++r) s[Lay::phys(base + 8 * r, col)] = v[b][r];
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int b = 0; b < X::PE; ++b) {                       // stage 3 (NS = N/8)
-    const int j = jb + b * TPC;
-    float2 y[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) y[r] = s[Lay::phys(j + X::NB * r, col)];
-#pragma unroll
-    for (int r = 1; r < 8; ++r) {
-      float2 w = tw[X::OFF3 + (r - 1) * X::NB + j];
-      if (INV) w.y = -w.y;
-      y[r] = cmul(y[r], w);
-    }
-    Dft<8, INV>::run(y);
-    st(b, y);
   }
 }
 
@@ -1444,12 +1426,13 @@ __device__ __forceinline__ uint32_t opaque_u32(uint32_t x) {
 
 template <bool INV, int N, int C, bool PAIR>
 __global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline_kernel(const SArgs a) {
-  constexpr int H = N / 2, T = XLine<N, C>::T, TPC = XLine<N, C>::TPC, NB = XLine<N, C>::NB;
+  using X = XLine<N, C>;
+  constexpr int H = N / 2, T = X::T, E = X::E, G = X::G;
   extern __shared__ float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
-  float2* s = tw + XLine<N, C>::TAB;
+  float2* s = tw + X::TAB;
   if (!INV && a.skip_flag && *a.skip_flag != 0) return;   // uniform: device loop already converged
-  for (int m = threadIdx.x; m < Plan<N>::kTab; m += T) tw[m] = a.tab[m];
+  for (int m = threadIdx.x; m < X::kTab; m += T) tw[m] = a.tabx[m];
   const int role = PAIR ? (int)(blockIdx.x & 1) : (int)blockIdx.y;
   // tiles of every y-plane, or of the planes [ybeg, ybeg + ycount): their M tiles (ky, kz block)
   // and the Nyquist tiles that hold their ky columns
@@ -1463,20 +1446,21 @@ __global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline
   // element offsets fit 32 bits (at most N^3 / 2 complex points per field)
   const uint32_t o0 = (uint32_t)t.base + (uint32_t)(col * t.cs) + (uint32_t)jb * (uint32_t)t.ls;
   const uint32_t ls = (uint32_t)t.ls;
-  // element offset of point (b, r) of this thread; every load and store re-derives the base through
-  // an opaque copy, so no offset is kept live across a transform
-  auto off = [&](uint32_t base, int b, int r) { return base + (uint32_t)(b * TPC + NB * r) * ls; };
+  // element offsets of a load's point r and of a store's point (h, r); stores re-derive the base
+  // through an opaque copy, so no offset is kept live across a transform
+  auto off_ld = [&](uint32_t base, int r) { return base + (uint32_t)(G * r) * ls; };
+  auto off_st = [&](uint32_t base, int h, int r) { return base + (uint32_t)(G * h + E * r) * ls; };
   auto load = [&](const float2* __restrict__ P) {
-    return [=, &off](int b, float2 (&x)[8]) {
+    return [=, &off_ld](float2 (&x)[E]) {
 #pragma unroll
-      for (int r = 0; r < 8; ++r) x[r] = P[off(o0, b, r)];
+      for (int r = 0; r < E; ++r) x[r] = P[off_ld(o0, r)];
     };
   };
   auto store = [&](float2* __restrict__ P, float scale) {
-    return [=, &off](int b, const float2 (&y)[8]) {
+    return [=, &off_st](int h, const float2 (&y)[G]) {
       const uint32_t o = opaque_u32(o0);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) P[off(o, b, r)] = cscale(y[r], scale);
+      for (int r = 0; r < G; ++r) P[off_st(o, h, r)] = cscale(y[r], scale);
     };
   };
   const Geometry& g = a.g;
@@ -1497,15 +1481,14 @@ __global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline
   const float kf = g.kf;
   const float kdz = t.isQ ? 0.f : kf * (float)(t.c0 + col);   // M tiles: kz < N/2; Q tiles: kz = N/2
   // the line index i is kx in Fourier space and x in configuration space
-  auto kdx = [&](int b, int r) {
-    const int i = jb + b * TPC + NB * r;
-    return i == H ? 0.f : kf * (float)(i < H ? i : i - N);
-  };
-  auto dxv = [&](int b, int r) { return g.los_mode == 1 ? g.los.x : g.off[jb + b * TPC + NB * r]; };
+  auto kdx = [&](int i) { return i == H ? 0.f : kf * (float)(i < H ? i : i - N); };
+  auto dxv = [&](int i) { return g.los_mode == 1 ? g.los.x : g.off[i]; };
   // loads of G scaled by kdx (the inverse's x component)
-  auto load_kdx_g = [&](int b, float2 (&x)[8]) {
+  auto load_kdx_g = [&](float2 (&x)[E]) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) x[r] = cscale(P2[off(o0, b, r)], kdx(b, r));
+    for (int r = 0; r < E; ++r) x[r] = P2[off_ld(o0, r)];
+#pragma unroll
+    for (int r = 0; r < E; ++r) x[r] = cscale(x[r], kdx(jb + G * r));
   };
   if (cf) {
     // both roles start on G, so the pair reads it from HBM once
@@ -1518,13 +1501,13 @@ __global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline
     // rounded exactly as the projection pass forms it from the three components
     xline_io<INV, N, C>(s, tw, jb, col, load_kdx_g, store(P0, 1.f));
     __syncthreads();   // s is rewritten by the second transform
-    xline_io<INV, N, C>(s, tw, jb, col, load(P1), [&](int b, const float2 (&y)[8]) {   // IFFT_x(Psi_y)
+    xline_io<INV, N, C>(s, tw, jb, col, load(P1), [&](int h, const float2 (&y)[G]) {   // IFFT_x(Psi_y)
       const uint32_t o = opaque_u32(o0);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const float2 x = P0[off(o, b, r)];   // this thread's own Psi_x
-        const float d = dxv(b, r);
-        P0[off(o, b, r)] = make_float2(fmaf(d, x.x, dy * y[r].x), fmaf(d, x.y, dy * y[r].y));
+      for (int r = 0; r < G; ++r) {
+        const float2 x = P0[off_st(o, h, r)];   // this thread's own Psi_x
+        const float d = dxv(jb + G * h + E * r);
+        P0[off_st(o, h, r)] = make_float2(fmaf(d, x.x, dy * y[r].x), fmaf(d, x.y, dy * y[r].y));
       }
     });
     return;
@@ -1539,19 +1522,21 @@ __global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline
   xline_io<INV, N, C>(s, tw, jb, col, load(P2), store(P2, kdz));
   __syncthreads();   // s is rewritten by the second transform
   xline_io<INV, N, C>(s, tw, jb, col,
-                    [&](int b, float2 (&x)[8]) {
+                      [&](float2 (&x)[E]) {
 #pragma unroll
-                      for (int r = 0; r < 8; ++r) x[r] = cscale(P0[off(o0, b, r)], dxv(b, r));
-                    },
-                    [&](int b, const float2 (&y)[8]) {   // FFT_x(dx psi^)
-                      const uint32_t o = opaque_u32(o0);
+                        for (int r = 0; r < E; ++r) x[r] = P0[off_ld(o0, r)];
 #pragma unroll
-                      for (int r = 0; r < 8; ++r) {
-                        const float2 x = P2[off(o, b, r)];   // this thread's own kdz FFT_x(Z^)
-                        const float k = kdx(b, r);
-                        P2[off(o, b, r)] = make_float2(fmaf(k, y[r].x, x.x), fmaf(k, y[r].y, x.y));
-                      }
-                    });
+                        for (int r = 0; r < E; ++r) x[r] = cscale(x[r], dxv(jb + G * r));
+                      },
+                      [&](int h, const float2 (&y)[G]) {   // FFT_x(dx psi^)
+                        const uint32_t o = opaque_u32(o0);
+#pragma unroll
+                        for (int r = 0; r < G; ++r) {
+                          const float2 x = P2[off_st(o, h, r)];   // this thread's own kdz FFT_x(Z^)
+                          const float k = kdx(jb + G * h + E * r);
+                          P2[off_st(o, h, r)] = make_float2(fmaf(k, y[r].x, x.x), fmaf(k, y[r].y, x.y));
+                        }
+                      });
 }
 
 // One tile of the source update (Eq. iterative) from registers: v[0] = A and v[1] = P_y along the y
@@ -1793,6 +1778,11 @@ __global__ void build_tables_kernel(const float2* __restrict__ tw, float2* tabS,
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
   Plan<N>::template fill<1>(tabS, tw, tid, nthr);
   Plan<N / 2>::template fill<2>(tabZ, tw, tid, nthr);
+  if constexpr (kFusedMesh<N>) {   // the x lines' second-stage twiddles behind the N-point plan's
+    using X = XLine<N, 16>;
+    float2* tx = tabS + ((Plan<N>::kTab + 1) & ~1);
+    for (int e = tid; e < X::kTab; e += nthr) tx[e] = tw[(1 + e / X::E) * (e % X::E)];
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1986,7 +1976,9 @@ struct MeshImpl {
       attr[inv] = true;
     }
     if (a.ycount && (a.ycount % C || a.ybeg % C || a.ybeg < 0 || a.ybeg + a.ycount > N)) return cudaErrorInvalidValue;
-    void* args[] = {const_cast<SArgs*>(&a)};
+    SArgs ax = a;
+    ax.tabx = a.tab + ((Plan<N>::kTab + 1) & ~1);
+    void* args[] = {&ax};
     const int tiles = a.ycount ? a.ycount * ((N / 2) / C) + a.ycount / C : N * ((N / 2) / C) + N / C;
     // pairs: the two CTAs of a tile on adjacent block indices; single fields: components along y
     const dim3 grid = PAIR ? dim3(2 * tiles) : dim3(tiles, ncomp);
@@ -2031,7 +2023,7 @@ struct MeshImpl {
   }
 
   static const MeshKernels* table() {
-    static const MeshKernels t = {N, kZBlocks, kSBlocks, Plan<N>::kTab, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0,
+    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0,
                                   &zpass, &spass, &build_tables};
     return &t;
   }

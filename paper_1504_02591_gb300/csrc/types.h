@@ -86,6 +86,7 @@ struct SArgs {
   Field f[3];             // fields transformed in place
   Geometry g;
   const float2* tab;      // stage twiddles of the N-point plan
+  const float2* tabx;     // x lines of the register-fused family: their second-stage twiddles (set at launch)
   double* partials;       // per-block partials (2 per block, S_ITER)
   const double* red;      // reduction block (S_DELTA reads the lognormal sum)
   Field dk;               // delta: partially transformed (S_DELTA input) / k-space (S_ITER)
