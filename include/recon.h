@@ -366,10 +366,12 @@ enum {
                                    multiple of the x-line tile width (16, or 8 with RECON_OPT_LINE_TILE) */
 };
 /* Particle paths: DIRECT handles each particle independently (8 global atomics per deposited
- * particle; 24 scattered reads per interpolated one); SORTED packs the particles, counting-sorts
- * them by 8^3-cell brick and works brick by brick in shared memory (deposit: one global atomic per
- * touched node of the brick; shift: Psi staged once per brick).  Both give the same results up to
- * float32 summation order. */
+ * particle; 24 scattered reads per interpolated one, or 8 of nodes packed first); SORTED packs the
+ * particles, counting-sorts them by 8^3-cell brick and works brick by brick in shared memory (deposit:
+ * one global atomic per touched node of the brick; shift: Psi staged once per brick).  Both give the
+ * same results up to float32 summation order.  A SORTED shift without a retained order
+ * (RECON_OPT_REUSE_SORT) sorts only where that is the faster way: N >= 384 and at least N^3 / 32
+ * particles; otherwise it runs as DIRECT. */
 enum { RECON_PATH_DIRECT = 0, RECON_PATH_SORTED = 1 };
 
 /* Set a handle option (values 0 or 1, RECON_OPT_PLANE_BATCH 0/16/32/64); INVALID_ARG for an unknown

@@ -23,11 +23,10 @@ struct BrickBuffers {
   uint32_t* offs;        // nb^3 + 1 exclusive offsets
   uint32_t* bsum;        // scan block sums (<= 4096)
   uint4* rec;            // kSortChunk sorted records: packed x, y, z (cell << 21 | frac), weight bits
-  uint32_t* perm;        // kSortChunk: sorted slot -> index within the chunk
-  uint32_t* key;         // kSortChunk: brick of each particle (input order)
+  uint32_t* key;         // kSortChunk: brick of each particle (input order), after the sort its sorted slot
   uint32_t* rank;        // kSortChunk: arrival rank of each particle within its brick
-  uint4* pre;            // kSortChunk: packed records in input order (count -> scatter); free after
-                         // the scatter (a retained sort's shift writes its float32 shifts here)
+  uint4* pre;            // kSortChunk: packed records in input order (count -> scatter), then the
+                         // shifts in sorted order (brick_shift -> brick_unsort)
 };
 
 size_t brick_scratch_bytes(int n);
@@ -53,13 +52,16 @@ struct BrickShiftArgs {
   float3 los;
   int periodic;
   double L;
-  const void* pos;       // original positions of the chunk (pos_out only)
+  // brick_unsort, all for its first particle
+  const void* pos;       // original positions (pos_out only)
   int dtype;
-  float* shift;          // chunk outputs, original order
+  float* shift;          // outputs, original order
   double* pos_out;       // or null
 };
 
-// CIC interpolation of Psi and the shift for the sorted chunk (one warp per brick)
+// CIC interpolation of Psi and the shift for the sorted chunk (one warp per brick), in sorted order
 cudaError_t brick_shift(const BrickBuffers& b, const BrickShiftArgs& a, cudaStream_t st);
+// ... and the results of particles [p0, p0 + m) back in catalogue order
+cudaError_t brick_unsort(const BrickBuffers& b, const BrickShiftArgs& a, long long p0, long long m, cudaStream_t st);
 
 }  // namespace rg

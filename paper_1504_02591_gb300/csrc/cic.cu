@@ -11,16 +11,16 @@
 
 namespace rg {
 
-// Nodes and weights of one particle.  u 2^32 = x times scale 2^32 (exact scaling: the same rounding
-// as u), rounded down to an integer T: floor(u) = T >> 32 and t = (T mod 2^32) 2^-32.  Two float64
-// operations per axis (float64 runs at a small fraction of the float32 rate on this GPU).
+// Nodes and weights of one particle.  u 2^32 = x times scale 2^32 (exact scaling) rounded down to an
+// integer T: floor(u) = T >> 32 and t = (T mod 2^32) 2^-32.  One float64 operation per axis (float64
+// runs at a small fraction of the float32 rate on this GPU).
 template <typename PT>
 __device__ __forceinline__ void cic_setup(const PT* __restrict__ pos, long long p, int n, double scale,
                                           int (&i0)[3], int (&i1)[3], float (&t)[3]) {
   const double scale32 = scale * 4294967296.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const long long T = __double2ll_rd((double)pos[3 * p + a] * scale32);
+    const long long T = floor_scaled((double)pos[3 * p + a], scale32, 0.0);
     t[a] = (float)(uint32_t)T * 2.3283064365386963e-10f;   // 2^-32
     int c = (int)(T >> 32);
     if (c < 0 || c >= n) c = ((c % n) + n) % n;   // outside [0, L): periodic image
@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(256) deposit_kernel(const PT* __restrict__ pos
                                                       long long np, int n, double scale,
                                                       float* __restrict__ rho, double* __restrict__ partials) {
   double wsum = 0.0;
+  int count = 0;   // unit weights: a thread's share is far below 2^31
   const size_t nn = (size_t)n;
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
        p += (long long)gridDim.x * blockDim.x) {
@@ -54,7 +55,8 @@ __global__ void __launch_bounds__(256) deposit_kernel(const PT* __restrict__ pos
     float t[3];
     cic_setup(pos, p, n, scale, i0, i1, t);
     const float wp = w ? w[p] : 1.f;
-    wsum += wp;
+    if (w) wsum += wp;
+    else ++count;
     const float wx0 = wp * (1.f - t[0]), wx1 = wp * t[0];
     const float wy0 = 1.f - t[1], wy1 = t[1];
     const float wz0 = 1.f - t[2], wz1 = t[2];
@@ -69,7 +71,7 @@ __global__ void __launch_bounds__(256) deposit_kernel(const PT* __restrict__ pos
     atomicAdd(rho + r11 + i0[2], wx1 * wy1 * wz0);
     atomicAdd(rho + r11 + i1[2], wx1 * wy1 * wz1);
   }
-  const double s = block_sum_d(wsum);
+  const double s = block_sum_d(w ? wsum : (double)count);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
@@ -80,6 +82,7 @@ __global__ void __launch_bounds__(256) ngp_deposit_kernel(const PT* __restrict__
                                                           long long np, int n, double scale,
                                                           float* __restrict__ rho, double* __restrict__ partials) {
   double wsum = 0.0;
+  int count = 0;
   const size_t nn = (size_t)n;
   const double scale32 = scale * 4294967296.0;
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
@@ -87,54 +90,97 @@ __global__ void __launch_bounds__(256) ngp_deposit_kernel(const PT* __restrict__
     int c[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const long long T = __double2ll_rd(fma((double)pos[3 * p + a], scale32, 2147483648.0));
+      const long long T = floor_scaled((double)pos[3 * p + a], scale32, 2147483648.0);
       int k = (int)(T >> 32);
       if (k < 0 || k >= n) k = ((k % n) + n) % n;
       c[a] = k;
     }
     const float wp = w ? w[p] : 1.f;
-    wsum += wp;
+    if (w) wsum += wp;
+    else ++count;
     atomicAdd(rho + ((size_t)c[0] * nn + c[1]) * nn + c[2], wp);
   }
-  const double s = block_sum_d(wsum);
+  const double s = block_sum_d(w ? wsum : (double)count);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
+// Shell of a particle: floor((r - rmin) inv_dr) clamped to [-1, nbins], r its float64 distance from obs.
+// float64 square roots and quotients cost most of a pass here, so the shell is found in float32 (offsets
+// taken in float64) unless the coordinate lies so near a shell's edge that its rounding could matter: the
+// float32 coordinate is off by at most 2^-24 (3.5 r + 2 rmin) inv_dr + 2^-23 |f| (three rounded offsets, two
+// fused sums and a correctly rounded root, then one difference and one product); the margin is five times
+// that.  Near an edge, and for coordinates that are not finite, the float64 expression decides.
+template <typename PT>
+__device__ __forceinline__ int shell_of(const PT* __restrict__ pos, long long p, double3 obs, double rmin, double inv_dr,
+                                        int nbins) {
+  const double dx = (double)pos[3 * p] - obs.x, dy = (double)pos[3 * p + 1] - obs.y, dz = (double)pos[3 * p + 2] - obs.z;
+  const float fx = (float)dx, fy = (float)dy, fz = (float)dz;
+  const float r = __fsqrt_rn(fmaf(fx, fx, fmaf(fy, fy, fz * fz)));
+  const float rm = (float)rmin, inv = (float)inv_dr;
+  const float f = (r - rm) * inv;
+  const float margin = fmaf(1.2e-6f * (r + fabsf(rm)), inv, 6e-7f * fabsf(f));
+  const float k = floorf(f);
+  if (f - k > margin && k + 1.f - f > margin && r > 1e-15f && r < 1e18f && fabsf(f) < 1e6f)
+    return k < 0.f ? -1 : (k >= (float)nbins ? nbins : (int)k);
+  const double b = floor((sqrt(dx * dx + dy * dy + dz * dz) - rmin) * inv_dr);
+  return b >= 0.0 ? (b < (double)nbins ? (int)b : nbins) : -1;
+}
+
 // Radial number density (Sec. 3.2 n(z), in comoving distance from the observer): counts of the
-// particles in nbins equal shells of [rmin, rmax), float64 distances.
+// particles in nbins equal shells of [rmin, rmax), float64 distances; counted per block in shared memory
+// (6e5 galaxies in 50 shells: 120 us when every particle went to a global counter).
 template <typename PT>
 __global__ void __launch_bounds__(256) radial_hist_kernel(const PT* __restrict__ pos, long long np, double3 obs,
                                                           double rmin, double inv_dr, int nbins,
                                                           unsigned long long* __restrict__ counts) {
+  __shared__ unsigned int h[4096];
+  for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0u;
+  __syncthreads();
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
        p += (long long)gridDim.x * blockDim.x) {
-    const double dx = (double)pos[3 * p] - obs.x, dy = (double)pos[3 * p + 1] - obs.y, dz = (double)pos[3 * p + 2] - obs.z;
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    const double b = floor((r - rmin) * inv_dr);
-    if (b >= 0.0 && b < (double)nbins) atomicAdd(counts + (int)b, 1ull);
+    const int b = shell_of(pos, p, obs, rmin, inv_dr, nbins);
+    if (b >= 0 && b < nbins) atomicAdd(h + b, 1u);
   }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nbins; b += blockDim.x)
+    if (h[b]) atomicAdd(counts + b, (unsigned long long)h[b]);
 }
 
-// FKP weights w = 1 / (1 + nbar(r) P0) (Sec. 3.2), nbar of the particle's shell, 0 outside.
+// FKP weights (Sec. 3.2): the table's entry of the particle's shell, its last entry outside the shells.
+// A weight depends on the shell alone, so the quotients are formed once per shell on the host.
 template <typename PT>
 __global__ void __launch_bounds__(256) fkp_kernel(const PT* __restrict__ pos, long long np, double3 obs, double rmin,
-                                                  double inv_dr, int nbins, const double* __restrict__ nbar,
-                                                  double P0, float* __restrict__ w) {
+                                                  double inv_dr, int nbins, const float* __restrict__ wtab,
+                                                  float* __restrict__ w) {
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
        p += (long long)gridDim.x * blockDim.x) {
-    const double dx = (double)pos[3 * p] - obs.x, dy = (double)pos[3 * p + 1] - obs.y, dz = (double)pos[3 * p + 2] - obs.z;
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    const double b = floor((r - rmin) * inv_dr);
-    const double nb = (b >= 0.0 && b < (double)nbins) ? nbar[(int)b] : 0.0;
-    w[p] = (float)(1.0 / (1.0 + nb * P0));
+    const int b = shell_of(pos, p, obs, rmin, inv_dr, nbins);
+    w[p] = __ldg(wtab + (b < 0 ? nbins : b));
   }
 }
 
-template <typename PT>
+__global__ void __launch_bounds__(256) pack_psi_kernel(const float4* __restrict__ x, const float4* __restrict__ y,
+                                                       const float4* __restrict__ z, float4* __restrict__ out, size_t n4) {
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 256) {
+    const float4 a = x[i], b = y[i], c = z[i];
+    out[4 * i] = make_float4(a.x, b.x, c.x, 0.f);
+    out[4 * i + 1] = make_float4(a.y, b.y, c.y, 0.f);
+    out[4 * i + 2] = make_float4(a.z, b.z, c.z, 0.f);
+    out[4 * i + 3] = make_float4(a.w, b.w, c.w, 0.f);
+  }
+}
+
+// The shift of each particle by itself.  Gathers of particles in no order are bound by the L1's look-ups, one
+// per lane and load: 24 of them from three fields, 8 from nodes packed as float4 (PACKED).
+template <typename PT, bool PACKED>
 __global__ void __launch_bounds__(256) shift_kernel(const PT* __restrict__ pos, long long np, ShiftArgs a) {
+  __shared__ double slots_sm[8][96];
+  double* slots = slots_sm[threadIdx.x >> 5];
   const size_t nn = (size_t)a.n;
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
-       p += (long long)gridDim.x * blockDim.x) {
+  // whole warps stay in the loop: the stores go through the warp's slots
+  for (long long p0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); p0 < np;
+       p0 += (long long)gridDim.x * blockDim.x) {
+    const long long pl = p0 + (threadIdx.x & 31), p = pl < np ? pl : np - 1;
     int i0[3], i1[3];
     float t[3];
     cic_setup(pos, p, a.n, a.scale, i0, i1, t);
@@ -145,15 +191,26 @@ __global__ void __launch_bounds__(256) shift_kernel(const PT* __restrict__ pos, 
                            r10 + i0[2], r10 + i1[2], r11 + i0[2], r11 + i1[2]};
     const float cw[8] = {wx0 * wy0 * wz0, wx0 * wy0 * wz1, wx0 * wy1 * wz0, wx0 * wy1 * wz1,
                          wx1 * wy0 * wz0, wx1 * wy0 * wz1, wx1 * wy1 * wz0, wx1 * wy1 * wz1};
-    float ps[3];
+    float ps[3] = {0.f, 0.f, 0.f};
+    if (PACKED) {
+      float4 v[8];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float acc = 0.f;
+      for (int k = 0; k < 8; ++k) v[k] = __ldg(a.psi4 + idx[k]);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc = fmaf(cw[k], __ldg(a.psi[c] + idx[k]), acc);
-      ps[c] = acc;
+      for (int k = 0; k < 8; ++k) {
+        ps[0] = fmaf(cw[k], v[k].x, ps[0]);
+        ps[1] = fmaf(cw[k], v[k].y, ps[1]);
+        ps[2] = fmaf(cw[k], v[k].z, ps[2]);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float acc = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc = fmaf(cw[k], __ldg(a.psi[c] + idx[k]), acc);
+        ps[c] = acc;
+      }
     }
-    const double x0 = (double)pos[3 * p], x1 = (double)pos[3 * p + 1], x2 = (double)pos[3 * p + 2];
     float d[3];
     if (a.is_galaxy) {
       float rx, ry, rz;
@@ -175,21 +232,15 @@ __global__ void __launch_bounds__(256) shift_kernel(const PT* __restrict__ pos, 
     } else {
       d[0] = -ps[0]; d[1] = -ps[1]; d[2] = -ps[2];
     }
-    a.shift[3 * p + 0] = d[0];
-    a.shift[3 * p + 1] = d[1];
-    a.shift[3 * p + 2] = d[2];
+    warp_store3(a.shift, p0, np, d, reinterpret_cast<float*>(slots));
     if (a.pos_out) {
-      double y[3] = {x0 + d[0], x1 + d[1], x2 + d[2]};
-      if (a.periodic) {
+      double y[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          y[c] = y[c] - floor(y[c] / a.L) * a.L;
-          if (y[c] >= a.L) y[c] -= a.L;
-        }
+      for (int c = 0; c < 3; ++c) {
+        y[c] = (double)pos[3 * p + c] + d[c];
+        if (a.periodic) y[c] = wrap_box(y[c], a.L);
       }
-      a.pos_out[3 * p + 0] = y[0];
-      a.pos_out[3 * p + 1] = y[1];
-      a.pos_out[3 * p + 2] = y[2];
+      warp_store3(a.pos_out, p0, np, y, slots);
     }
   }
 }
@@ -262,14 +313,26 @@ cudaError_t launch_deposit(const void* pos, int dtype, const float* w, long long
   return cudaGetLastError();
 }
 
+cudaError_t launch_pack_psi(const float* const psi[3], float4* psi4, size_t n, cudaStream_t st) {
+  const size_t want = (n / 4 + 255) / 256;
+  const int blocks = (int)(want < 152 * 16 ? want : 152 * 16);
+  pack_psi_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(psi[0]), reinterpret_cast<const float4*>(psi[1]),
+                                          reinterpret_cast<const float4*>(psi[2]), psi4, n / 4);
+  return cudaGetLastError();
+}
+
+template <typename PT>
+static void shift_launch(const void* pos, long long np, const ShiftArgs& a, int blocks, cudaStream_t st) {
+  if (a.psi4) shift_kernel<PT, true><<<blocks, 256, 0, st>>>((const PT*)pos, np, a);
+  else shift_kernel<PT, false><<<blocks, 256, 0, st>>>((const PT*)pos, np, a);
+}
+
 cudaError_t launch_shift(const void* pos, int dtype, long long np, const ShiftArgs& a, cudaStream_t st) {
   if (np <= 0) return cudaSuccess;
   long long want = (np + 255) / 256;
   const int blocks = (int)(want < 152 * 16 ? want : 152 * 16);
-  if (dtype == 0)
-    shift_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, a);
-  else
-    shift_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, a);
+  if (dtype == 0) shift_launch<double>(pos, np, a, blocks, st);
+  else shift_launch<float>(pos, np, a, blocks, st);
   return cudaGetLastError();
 }
 
@@ -386,14 +449,14 @@ cudaError_t launch_radial_hist(const void* pos, int dtype, long long np, double3
 }
 
 cudaError_t launch_fkp(const void* pos, int dtype, long long np, double3 obs, double rmin, double rmax, int nbins,
-                       const double* nbar, double P0, float* w, cudaStream_t st) {
+                       const float* wtab, float* w, cudaStream_t st) {
   if (np <= 0) return cudaSuccess;
   const double inv_dr = nbins / (rmax - rmin);
   const int blocks = (int)((np + 255) / 256 < 152 * 16 ? (np + 255) / 256 : 152 * 16);
   if (dtype == 0)
-    fkp_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, obs, rmin, inv_dr, nbins, nbar, P0, w);
+    fkp_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, obs, rmin, inv_dr, nbins, wtab, w);
   else
-    fkp_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, obs, rmin, inv_dr, nbins, nbar, P0, w);
+    fkp_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, obs, rmin, inv_dr, nbins, wtab, w);
   return cudaGetLastError();
 }
 

@@ -1311,6 +1311,20 @@ recon_status recon_get_trace(recon_handle* h, double* rel, int cap, int* n) {
   return RECON_OK;
 }
 
+namespace {
+// A shift that holds no brick order of its catalogue sorts it first only where that pays.  The sort and
+// the sorted gather cost about 75 us per 1e6 tracers plus the staging of every occupied brick; the direct
+// gather 72 us per 1e6 up to N = 128 and, where the three fields pass the L2, 140, 210, 330 and 410 at
+// N = 256, 384, 512 and 1024 for tracers all over the box (half of that for a survey's tenth of it).
+// Measured, uniform tracers, sorted / direct us: N = 64 2e6 419 / 146; 256 1e7 719 / 1403 (packed: 747);
+// 384 2e6 508 / 452, 1e7 979 / 2131; 512 2e6 1014 / 682, 1e7 1499 / 3311; 1024 1e7 10784 / 4186, 3.3e7
+// 13328 / 13825.  The two meet near N^3 / 32 tracers on the meshes that sort at all.
+bool shift_sorts(int n, int64_t count) { return n >= 384 && count >= (int64_t)n * n * n / 32; }
+// Packing the nodes as float4 (28 bytes moved per node: 12 us at N <= 128, 95 at 256) halves the direct
+// gather: 35 us per 1e6 tracers up to N = 128, 65 at 256; from N^3 / 8 tracers on (and 200,000) it pays.
+bool shift_packs(int n, int64_t count) { return n <= 256 && count >= 200000 && count >= (int64_t)n * n * n / 8; }
+}  // namespace
+
 recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galaxy, float* shift_out,
                          double* pos_out, int out_on_device) {
   if (!h) return RECON_ERR_INVALID_ARG;
@@ -1345,20 +1359,38 @@ recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galax
                     cat->on_device == h->memo.on_device;
   if (h->reuse_sort && same && !pos_out && cat->n > 0) {
     // the deposit's brick order of this very catalogue: no second read of the positions
-    float* dst = out_on_device ? shift_out : reinterpret_cast<float*>(h->bb.pre);
     ba.pos = nullptr;
     ba.pos_out = nullptr;
-    ba.shift = dst;
-    RG_CUDA(timed(h, RECON_K_SHIFT, (double)cat->n * (16 + 4 + 12), [&] { return brick_shift(h->bb, ba, h->st); }));
-    if (!out_on_device) {
-      RG_CUDA(cudaMemcpyAsync(shift_out, dst, (size_t)cat->n * 3 * sizeof(float), cudaMemcpyDeviceToHost, h->st));
+    RG_CUDA(timed(h, RECON_K_SHIFT, (double)cat->n * (16 + 16 + 4 + 16 + 12), [&] {
+      const cudaError_t e = brick_shift(h->bb, ba, h->st);
+      if (e != cudaSuccess || !out_on_device) return e;
+      ba.shift = shift_out;
+      return brick_unsort(h->bb, ba, 0, cat->n, h->st);
+    }));
+    if (!out_on_device) {   // catalogue order through the staging buffer
+      const long long part = (long long)(h->lay.stage / (3 * sizeof(float)));
+      for (long long p0 = 0; p0 < cat->n; p0 += part) {
+        const long long m = cat->n - p0 < part ? cat->n - p0 : part;
+        ba.shift = reinterpret_cast<float*>(h->stage);
+        RG_CUDA(timed(h, RECON_K_SHIFT, 0.0, [&] { return brick_unsort(h->bb, ba, p0, m, h->st); }));
+        RG_CUDA(cudaMemcpyAsync(shift_out + 3 * p0, h->stage, (size_t)m * 3 * sizeof(float), cudaMemcpyDeviceToHost, h->st));
+      }
       RG_CUDA(cudaStreamSynchronize(h->st));
     }
     return RECON_OK;
   }
   // with a retained brick order, other catalogues take the direct path so that it survives
-  const bool sorted = h->shift_path == RECON_PATH_SORTED && !(h->reuse_sort && h->memo.valid);
+  const bool keep_order = h->reuse_sort && h->memo.valid;
+  const bool sorted = h->shift_path == RECON_PATH_SORTED && !keep_order && shift_sorts(h->n, cat->n);
   if (sorted) h->memo.valid = 0;
+  if (!sorted && !keep_order && cat->n > 0 && shift_packs(h->n, cat->n)) {
+    // nodes packed as float4, in the sort's scratch
+    float4* psi4 = reinterpret_cast<float4*>(h->bb.hist);
+    h->memo.valid = 0;
+    const size_t nr = (size_t)h->n * h->n * h->n;
+    RG_CUDA(timed(h, RECON_K_SHIFT, 28.0 * nr, [&] { return launch_pack_psi(a.psi, psi4, nr, h->st); }));
+    a.psi4 = psi4;
+  }
   const bool staged = !cat->on_device || !out_on_device;
   const long long chunk = staged ? (kStageParticles < h->bb.chunk ? kStageParticles : h->bb.chunk) : h->bb.chunk;
   if (staged && !h->copy_st) {
@@ -1397,8 +1429,9 @@ recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galax
     if (sorted) {
       RG_CUDA(timed(h, RECON_K_SORT, (double)m * (6 * es + 28),
                     [&] { return brick_sort(h->bb, pin, cat->dtype, nullptr, m, h->st); }));
-      RG_CUDA(timed(h, RECON_K_SHIFT, (double)m * (16 + 4 + 12 + (pos_out ? 3 * es + 24 : 0)),
-                    [&] { return brick_shift(h->bb, ba, h->st); }));
+      RG_CUDA(timed(h, RECON_K_SHIFT, (double)m * (16 + 16 + 4 + 16 + 12 + (pos_out ? 3 * es + 24 : 0)), [&] {
+        const cudaError_t e = brick_shift(h->bb, ba, h->st);
+        return e == cudaSuccess ? brick_unsort(h->bb, ba, 0, m, h->st) : e; }));
     } else {
       a.shift = ba.shift;
       a.pos_out = ba.pos_out;
@@ -1687,12 +1720,16 @@ recon_status recon_fkp_weights(recon_handle* h, const recon_catalog* cat, int nb
   if (!h || !nbar || nbins < 1 || nbins > 4096 || !(rmax > rmin) || !(P0 >= 0)) return RECON_ERR_INVALID_ARG;
   RG_TRY(check_catalog(cat));
   if (cat->n > 0 && (!cat->on_device || !w_out)) return RECON_ERR_INVALID_ARG;
-  double* dnb = h->partials;
-  RG_CUDA(cudaMemcpyAsync(dnb, nbar, nbins * sizeof(double), cudaMemcpyHostToDevice, h->st));
+  // the weight of each shell; the last entry is the weight outside the shells (nbar = 0)
+  std::vector<float> wtab(nbins + 1);
+  for (int b = 0; b < nbins; ++b) wtab[b] = (float)(1.0 / std::fma(nbar[b], P0, 1.0));
+  wtab[nbins] = (float)(1.0 / std::fma(0.0, P0, 1.0));
+  float* dtab = reinterpret_cast<float*>(h->partials);   // at least kDepositBlocks x 4 doubles
+  RG_CUDA(cudaMemcpyAsync(dtab, wtab.data(), wtab.size() * sizeof(float), cudaMemcpyHostToDevice, h->st));
   const double3 obs = make_double3(h->p.observer[0], h->p.observer[1], h->p.observer[2]);
   RG_CUDA(timed(h, RECON_K_OTHER, (double)cat->n * (3 * elem_size(cat->dtype) + 4), [&] {
-    return launch_fkp(cat->pos, cat->dtype, cat->n, obs, rmin, rmax, nbins, dnb, P0, w_out, h->st); }));
-  RG_CUDA(cudaStreamSynchronize(h->st));   // nbar is read from the caller's host memory
+    return launch_fkp(cat->pos, cat->dtype, cat->n, obs, rmin, rmax, nbins, dtab, w_out, h->st); }));
+  RG_CUDA(cudaStreamSynchronize(h->st));   // the host table goes out of scope
   return RECON_OK;
 }
 
