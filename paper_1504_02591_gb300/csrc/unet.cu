@@ -46,190 +46,420 @@ __device__ __forceinline__ void tap_offset(int t, int ntap, int& dx, int& dy, in
   }
 }
 
+// Eight channels of one voxel as float32 (16-byte loads of bfloat16, two of float32).
+__device__ __forceinline__ void load8(const bf16* p, float (&v)[8]) {
+  const uint4 u = *reinterpret_cast<const uint4*>(p);
+  v[0] = __uint_as_float(u.x << 16); v[1] = __uint_as_float(u.x & 0xffff0000u);
+  v[2] = __uint_as_float(u.y << 16); v[3] = __uint_as_float(u.y & 0xffff0000u);
+  v[4] = __uint_as_float(u.z << 16); v[5] = __uint_as_float(u.z & 0xffff0000u);
+  v[6] = __uint_as_float(u.w << 16); v[7] = __uint_as_float(u.w & 0xffff0000u);
+}
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
 // ---- convolution forward: y = act(b + conv(concat(xa, xb))) (+ res for the head) ----------------
+// VPT voxels per thread (blockDim apart, so loads stay contiguous), all COUT channels of each in
+// registers; the weights of TG taps at a time in shared memory, read as broadcasts shared by the
+// thread's voxels; activations as 8-channel loads through the L1 (ca and cb multiples of 8; cin counts
+// the channels of xa that have weights, ca its stride).  Per output the sum runs over the taps and,
+// inside a tap, over the channels, one fused multiply-add each from the bias: the order that fixes
+// which way a stored bfloat16 rounds.
 template <typename T, int COUT>
-__global__ void __launch_bounds__(128) conv_fwd_kernel(const T* __restrict__ xa, int ca, const T* __restrict__ xb,
-                                                       int cb, const T* __restrict__ w, const float* __restrict__ bias,
-                                                       int ntap, int n, int relu, const float* __restrict__ res,
-                                                       int res_stride, T* __restrict__ y, float* __restrict__ yf) {
-  extern __shared__ float wsm[];
-  const int cin = ca + cb;
-  const long long nv = (long long)n * n * n;
-  const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  float acc[COUT];
+struct ConvFwd {
+  static constexpr int VPT = COUT >= 32 ? 1 : 2;
+  static constexpr int TG = 3;
+};
+template <typename T, int COUT>
+__global__ void __launch_bounds__(256) conv_fwd_kernel(const T* __restrict__ xa, int ca, int cina, int up,
+                                                       const T* __restrict__ xb, int cb, const T* __restrict__ w,
+                                                       const float* __restrict__ bias, int n, T* __restrict__ y) {
+  constexpr int VPT = ConvFwd<T, COUT>::VPT, TG = ConvFwd<T, COUT>::TG;
+  extern __shared__ float4 wsm4[];
+  float* wsm = reinterpret_cast<float*>(wsm4);
+  const int cin = cina + cb;
+  const int nv = n * n * n;   // at most 256^3 voxels times 32 channels: 32-bit offsets
+  float2 acc[VPT][COUT / 2];
+  int vx[VPT], vy[VPT], vz[VPT], vv[VPT];
 #pragma unroll
-  for (int co = 0; co < COUT; ++co) acc[co] = bias[co];
-  int ix = 0, iy = 0, iz = 0;
-  if (v < nv) {
-    ix = (int)(v / ((long long)n * n));
-    iy = (int)((v / n) % n);
-    iz = (int)(v % n);
+  for (int k = 0; k < VPT; ++k) {
+    vv[k] = blockIdx.x * (256 * VPT) + k * 256 + threadIdx.x;
+    const int v = vv[k] < nv ? vv[k] : 0;
+    vx[k] = v / (n * n);
+    vy[k] = (v / n) % n;
+    vz[k] = v % n;
+#pragma unroll
+    for (int c = 0; c < COUT / 2; ++c) acc[k][c] = make_float2(bias[2 * c], bias[2 * c + 1]);
   }
-  for (int t = 0; t < ntap; ++t) {
+  for (int t0 = 0; t0 < 27; t0 += TG) {
     __syncthreads();
-    for (int e = threadIdx.x; e < cin * COUT; e += blockDim.x) wsm[e] = tof(w[(size_t)t * cin * COUT + e]);
+    for (int e = threadIdx.x; e < TG * cin * COUT; e += 256) wsm[e] = tof(w[(size_t)t0 * cin * COUT + e]);
     __syncthreads();
-    if (v < nv) {
+    for (int tt = 0; tt < TG; ++tt) {
       int dx, dy, dz;
-      tap_offset(t, ntap, dx, dy, dz);
-      const long long u = ((long long)wrapc(ix + dx, n) * n + wrapc(iy + dy, n)) * n + wrapc(iz + dz, n);
-      const T* pa = xa + u * ca;
-      for (int ci = 0; ci < ca; ++ci) {
-        const float xv = tof(pa[ci]);
+      tap_offset(t0 + tt, 27, dx, dy, dz);
+      int u[VPT], ua[VPT];   // voxel in the fine grid, and in xa's (the coarse one: nearest upsampling)
 #pragma unroll
-        for (int co = 0; co < COUT; ++co) acc[co] = fmaf(xv, wsm[ci * COUT + co], acc[co]);
+      for (int k = 0; k < VPT; ++k) {
+        const int x = wrapc(vx[k] + dx, n), y = wrapc(vy[k] + dy, n), z = wrapc(vz[k] + dz, n);
+        u[k] = (x * n + y) * n + z;
+        ua[k] = up ? ((x >> 1) * (n >> 1) + (y >> 1)) * (n >> 1) + (z >> 1) : u[k];
       }
-      if (cb) {
-        const T* pb = xb + u * cb;
-        for (int ci = 0; ci < cb; ++ci) {
-          const float xv = tof(pb[ci]);
+      const float* wt = wsm + tt * cin * COUT;
+      for (int c0 = 0; c0 < cin; c0 += 8) {
+        float xv[VPT][8];
 #pragma unroll
-          for (int co = 0; co < COUT; ++co) acc[co] = fmaf(xv, wsm[(ca + ci) * COUT + co], acc[co]);
+        for (int k = 0; k < VPT; ++k) {
+          if (c0 < cina) load8(xa + (size_t)ua[k] * ca + c0, xv[k]);
+          else load8(xb + (size_t)u[k] * cb + (c0 - cina), xv[k]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (c0 + i < cin) {   // uniform
+            const float4* w4 = reinterpret_cast<const float4*>(wt + (c0 + i) * COUT);
+#pragma unroll
+            for (int c = 0; c < COUT / 4; ++c) {
+              const float4 ww = w4[c];
+#pragma unroll
+              for (int k = 0; k < VPT; ++k) {
+                const float2 xx = make_float2(xv[k][i], xv[k][i]);
+                acc[k][2 * c] = __ffma2_rn(xx, make_float2(ww.x, ww.y), acc[k][2 * c]);
+                acc[k][2 * c + 1] = __ffma2_rn(xx, make_float2(ww.z, ww.w), acc[k][2 * c + 1]);
+              }
+            }
+          }
         }
       }
     }
   }
-  if (v < nv) {
 #pragma unroll
-    for (int co = 0; co < COUT; ++co) {
-      float o = acc[co];
-      if (relu) o = fmaxf(o, 0.f);
-      if (res) o += res[v * res_stride];
-      if (y) y[v * COUT + co] = fromf<T>(o);
-      if (yf) yf[v * COUT + co] = o;
+  for (int k = 0; k < VPT; ++k) {
+    if (vv[k] < nv) {
+      T* o = y + (size_t)vv[k] * COUT;
+#pragma unroll
+      for (int c = 0; c < COUT; c += 8) {
+        __align__(16) T t8[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          t8[2 * i] = fromf<T>(fmaxf(acc[k][c / 2 + i].x, 0.f));
+          t8[2 * i + 1] = fromf<T>(fmaxf(acc[k][c / 2 + i].y, 0.f));
+        }
+#pragma unroll
+        for (int b = 0; b < (int)sizeof(T) / 2; ++b)
+          reinterpret_cast<uint4*>(o + c)[b] = reinterpret_cast<const uint4*>(t8)[b];
+      }
     }
   }
 }
+
+// The 1x1x1 head: y = res + (b + sum_c x[c] w[c]).
+template <typename T, int CIN>
+__global__ void __launch_bounds__(256) head_fwd_kernel(const T* __restrict__ x, const T* __restrict__ w,
+                                                       const float* __restrict__ bias, const float* __restrict__ res,
+                                                       int res_stride, long long nv, float* __restrict__ y) {
+  const long long v = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (v >= nv) return;
+  float acc = bias[0];
+#pragma unroll
+  for (int c0 = 0; c0 < CIN; c0 += 8) {
+    float xv[8];
+    load8(x + v * CIN + c0, xv);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc = fmaf(xv[i], tof(w[c0 + i]), acc);
+  }
+  y[v] = acc + res[v * res_stride];
+}
+
+// ---- tiles of the backward convolutions: 4 x 4 x 32 voxels with a halo of one --------------------
+constexpr int kBX = 4, kBY = 4, kBZ = 32;
+constexpr int kHX = kBX + 2, kHY = kBY + 2, kHZ = kBZ + 2;
+struct TileGrid {
+  int nx, ny, nz;
+  __host__ __device__ explicit TileGrid(int n)
+      : nx((n + kBX - 1) / kBX), ny((n + kBY - 1) / kBY), nz((n + kBZ - 1) / kBZ) {}
+  __host__ __device__ int count() const { return nx * ny * nz; }
+  __device__ void origin(int t, int& x, int& y, int& z) const {
+    z = (t % nz) * kBZ;
+    y = (t / nz) % ny * kBY;
+    x = t / (nz * ny) * kBX;
+  }
+};
+__device__ __forceinline__ int wrapm(int i, int n) { return ((i % n) + n) % n; }   // any i: tiles may pass the grid
 
 // ---- gradient w.r.t. the input: gx[v][ci] = sum_t sum_co gy[v - d(t)][co] w[t][ci][co] ---------
-constexpr int kDChunk = 16;
+// A block of 128 threads owns one tile and 8 input channels, a thread 4 voxels along z (32 sums).
+// Per 8 output channels it stages gy's halo as float4 planes (4 channels a plane; z skewed by one
+// word in four, so the eight z runs of a quarter warp read distinct banks) and the 27 x 8 x 8 weights
+// (read as broadcasts).  A thread slides over z: six staged positions serve three taps of four voxels,
+// 384 multiply-adds per 30 shared loads.  The one-voxel-per-thread form spent its time on its loads:
+// 6.6 ms of a 128^3 training step for what is 1.2 ms of multiply-adds.
+// With mask the result is zeroed where the activation mask (same layout) is not positive (the ReLU).
+constexpr int kDZ = kHZ + (kHZ >> 2);
+constexpr int kDPlane = kHX * kHY * kDZ;
 template <typename T>
 __global__ void __launch_bounds__(128) conv_dgrad_kernel(const float* __restrict__ gy, int cout,
-                                                         const T* __restrict__ w, int ca, int cb, int ntap, int n,
-                                                         float* __restrict__ gxa, float* __restrict__ gxb, int accum_b) {
-  extern __shared__ float wsm[];   // kDChunk x cout
-  const int cin = ca + cb;
-  const int c0 = blockIdx.y * kDChunk;
-  const long long nv = (long long)n * n * n;
-  const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  float acc[kDChunk];
+                                                         const T* __restrict__ w, int ca, int cb, int n,
+                                                         float* __restrict__ gxa, float* __restrict__ gxb,
+                                                         const T* __restrict__ mask) {
+  extern __shared__ float4 dsm[];
+  float4* pl = dsm;                                           // [2][kHX][kHY][kDZ]
+  float* ws = reinterpret_cast<float*>(dsm + 2 * kDPlane);    // [27][8 co][8 ci], taps reversed
+  const int cin = ca + cb, c0 = blockIdx.y * 8;
+  const TileGrid tg(n);
+  int X, Y, Z;
+  tg.origin(blockIdx.x, X, Y, Z);
+  const int run = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 3, tx = threadIdx.x >> 5;
+  float2 acc[4][4];
 #pragma unroll
-  for (int k = 0; k < kDChunk; ++k) acc[k] = 0.f;
-  int ix = 0, iy = 0, iz = 0;
-  if (v < nv) {
-    ix = (int)(v / ((long long)n * n));
-    iy = (int)((v / n) % n);
-    iz = (int)(v % n);
-  }
-  for (int t = 0; t < ntap; ++t) {
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[k][c] = make_float2(0.f, 0.f);
+  for (int o0 = 0; o0 < cout; o0 += 8) {
     __syncthreads();
-    for (int e = threadIdx.x; e < kDChunk * cout; e += blockDim.x) {
-      const int cl = e / cout, co = e % cout;
-      wsm[e] = (c0 + cl < cin) ? tof(w[((size_t)t * cin + c0 + cl) * cout + co]) : 0.f;
+    for (int e = threadIdx.x; e < kHX * kHY * kHZ; e += 128) {
+      const int hz = e % kHZ, hy = (e / kHZ) % kHY, hx = e / (kHZ * kHY);
+      const int u = (wrapm(X + hx - 1, n) * n + wrapm(Y + hy - 1, n)) * n + wrapm(Z + hz - 1, n);
+      const float4* g = reinterpret_cast<const float4*>(gy + (size_t)u * cout + o0);
+      const int p = (hx * kHY + hy) * kDZ + hz + (hz >> 2);
+      pl[p] = g[0];
+      pl[kDPlane + p] = g[1];
+    }
+    for (int e = threadIdx.x; e < 27 * 64; e += 128) {
+      const int ci = e & 7, co = (e >> 3) & 7, t = e >> 6;
+      ws[e] = tof(w[((size_t)(26 - t) * cin + c0 + ci) * cout + o0 + co]);
     }
     __syncthreads();
-    if (v < nv) {
-      int dx, dy, dz;
-      tap_offset(t, ntap, dx, dy, dz);
-      const long long u = ((long long)wrapc(ix - dx, n) * n + wrapc(iy - dy, n)) * n + wrapc(iz - dz, n);
-      const float* g = gy + u * cout;
-      for (int co = 0; co < cout; ++co) {
-        const float gv = g[co];
+#pragma unroll 1
+    for (int dxy = 0; dxy < 9; ++dxy) {
+      const int p0 = ((tx + dxy / 3) * kHY + ty + dxy % 3) * kDZ + 5 * run;
 #pragma unroll
-        for (int k = 0; k < kDChunk; ++k) acc[k] = fmaf(gv, wsm[k * cout + co], acc[k]);
+      for (int h = 0; h < 2; ++h) {
+        float4 g[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) g[k] = pl[h * kDPlane + p0 + k + (k >> 2)];
+#pragma unroll
+        for (int dz = 0; dz < 3; ++dz) {
+          const float4* w4 = reinterpret_cast<const float4*>(ws + ((dxy * 3 + dz) * 8 + 4 * h) * 8);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 wa = w4[2 * i], wb = w4[2 * i + 1];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float4 gv = g[k + dz];
+              const float s = i == 0 ? gv.x : (i == 1 ? gv.y : (i == 2 ? gv.z : gv.w));
+              const float2 ss = make_float2(s, s);
+              acc[k][0] = __ffma2_rn(ss, make_float2(wa.x, wa.y), acc[k][0]);
+              acc[k][1] = __ffma2_rn(ss, make_float2(wa.z, wa.w), acc[k][1]);
+              acc[k][2] = __ffma2_rn(ss, make_float2(wb.x, wb.y), acc[k][2]);
+              acc[k][3] = __ffma2_rn(ss, make_float2(wb.z, wb.w), acc[k][3]);
+            }
+          }
+        }
       }
     }
   }
-  if (v < nv) {
+  const int x = X + tx, y = Y + ty;
+  if (x >= n || y >= n) return;
 #pragma unroll
-    for (int k = 0; k < kDChunk; ++k) {
-      const int ci = c0 + k;
-      if (ci < ca) {
-        gxa[v * ca + ci] = acc[k];
-      } else if (ci < cin) {
-        float* p = gxb + v * cb + (ci - ca);
-        *p = accum_b ? *p + acc[k] : acc[k];
+  for (int k = 0; k < 4; ++k) {
+    const int z = Z + 4 * run + k;
+    if (z < n) {
+      const size_t v = ((size_t)x * n + y) * n + z;
+      if (mask) {
+        float mv[8];
+        load8(mask + v * ca + c0, mv);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (!(mv[2 * c] > 0.f)) acc[k][c].x = 0.f;
+          if (!(mv[2 * c + 1] > 0.f)) acc[k][c].y = 0.f;
+        }
       }
+      float4* o = reinterpret_cast<float4*>(c0 < ca ? gxa + v * ca + c0 : gxb + v * cb + (c0 - ca));
+      o[0] = make_float4(acc[k][0].x, acc[k][0].y, acc[k][1].x, acc[k][1].y);
+      o[1] = make_float4(acc[k][2].x, acc[k][2].y, acc[k][3].x, acc[k][3].y);
     }
   }
 }
+constexpr size_t kDSmem = 2 * kDPlane * sizeof(float4) + 27 * 64 * sizeof(float);
 
-// ---- gradient w.r.t. the weights: gw[t][ci][co] += sum_v x[v + d(t)][ci] gy[v][co] ---------------
-constexpr int kWVox = 32;       // voxels staged per round
-constexpr int kWPairs = 16;     // (ci, co) pairs per thread (cin * cout <= 4096)
+// ---- gradients w.r.t. the weights and the bias: gw[t][ci][co] += sum_v x[v + d(t)][ci] gy[v][co] ----
+// A block owns one group of 8 input and one of 8 output channels (blockIdx.y) and walks over tiles.
+// Lane t < 27 of every warp is a tap and holds its 8 x 8 sums; the warp's lanes read the same gy
+// voxel (a broadcast) and their own shifted x voxel, one 16-byte load each for 64 multiply-adds (row
+// and plane strides of 3 and 1 mod 8 units put any eight consecutive taps in distinct banks).  Lane 27
+// multiplies by one instead: the bias gradient.  The 8 warps take the tile's rows and are summed at
+// the end, one atomic per block and weight.  The form before (one weight per thread and pass, both
+// factors reloaded from shared memory for every multiply-add) took 40 of a step's 52 ms.
+constexpr int kWRow = 35, kWPlane = 217;                     // voxel strides of the staged x (units of 8 channels)
 template <typename T>
-__global__ void __launch_bounds__(256) conv_wgrad_kernel(const T* __restrict__ xa, int ca, const T* __restrict__ xb,
-                                                         int cb, const float* __restrict__ gy, int cout, int ntap, int n,
-                                                         float* __restrict__ gw) {
-  extern __shared__ float sm[];
-  const int cin = ca + cb;
-  float* xs = sm;                       // kWVox x cin
-  float* gs = sm + kWVox * cin;         // kWVox x cout
-  const int t = blockIdx.y;
-  int dx, dy, dz;
-  tap_offset(t, ntap, dx, dy, dz);
-  const long long nv = (long long)n * n * n;
-  const int P = cin * cout;
-  float acc[kWPairs];
+__global__ void __launch_bounds__(256, 2) conv_wgrad_kernel(const T* __restrict__ xa, int ca, int cina, int up,
+                                                            const T* __restrict__ xb, int cb,
+                                                            const float* __restrict__ gy, int cout, int n,
+                                                            float* __restrict__ gw, float* __restrict__ gb) {
+  constexpr int U = (int)sizeof(T) / 2;                      // 16-byte units per 8 channels
+  extern __shared__ float4 gsm[];
+  uint4* xs = reinterpret_cast<uint4*>(gsm);                 // [U][kHX][kHY][kHZ] (padded strides)
+  float4* gs = gsm + U * kHX * kWPlane;                      // [512][2]
+  const int cin = cina + cb, og = cout / 8;
+  const int cg = blockIdx.y / og, o0 = (blockIdx.y % og) * 8, c0 = cg * 8;
+  const bool from_a = c0 < cina;
+  const T* src = from_a ? xa + c0 : xb + (c0 - cina);
+  const int cs = from_a ? ca : cb, sh = from_a ? up : 0, m = n >> sh;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = lane < 27 ? lane : 26;
+  const int toff = (t / 9) * kWPlane + (t / 3 % 3) * kWRow + t % 3;
+  const bool ones = lane == 27;
+  const TileGrid tg(n);
+  float2 acc[8][4];
 #pragma unroll
-  for (int k = 0; k < kWPairs; ++k) acc[k] = 0.f;
-  for (long long v0 = (long long)blockIdx.x * kWVox; v0 < nv; v0 += (long long)gridDim.x * kWVox) {
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = make_float2(0.f, 0.f);
+  for (int tile = blockIdx.x; tile < tg.count(); tile += gridDim.x) {
+    int X, Y, Z;
+    tg.origin(tile, X, Y, Z);
     __syncthreads();
-    for (int e = threadIdx.x; e < kWVox * cin; e += blockDim.x) {
-      const int lv = e / cin, ci = e % cin;
-      const long long v = v0 + lv;
-      float xv = 0.f;
-      if (v < nv) {
-        const int ix = (int)(v / ((long long)n * n)), iy = (int)((v / n) % n), iz = (int)(v % n);
-        const long long u = ((long long)wrapc(ix + dx, n) * n + wrapc(iy + dy, n)) * n + wrapc(iz + dz, n);
-        xv = ci < ca ? tof(xa[u * ca + ci]) : tof(xb[u * cb + (ci - ca)]);
+    for (int e = threadIdx.x; e < kHX * kHY * kHZ; e += 256) {
+      const int hz = e % kHZ, hy = (e / kHZ) % kHY, hx = e / (kHZ * kHY);
+      const int x = wrapm(X + hx - 1, n) >> sh, y = wrapm(Y + hy - 1, n) >> sh, z = wrapm(Z + hz - 1, n) >> sh;
+      const uint4* p = reinterpret_cast<const uint4*>(src + (size_t)((x * m + y) * m + z) * cs);
+#pragma unroll
+      for (int b = 0; b < U; ++b) xs[b * kHX * kWPlane + hx * kWPlane + hy * kWRow + hz] = p[b];
+    }
+    for (int e = threadIdx.x; e < kBX * kBY * kBZ; e += 256) {
+      const int z = Z + e % kBZ, y = Y + (e / kBZ) % kBY, x = X + e / (kBZ * kBY);
+      float4 g0 = make_float4(0.f, 0.f, 0.f, 0.f), g1 = g0;   // voxels past the grid add nothing
+      if (x < n && y < n && z < n) {
+        const float4* g = reinterpret_cast<const float4*>(gy + ((size_t)(x * n + y) * n + z) * cout + o0);
+        g0 = g[0];
+        g1 = g[1];
       }
-      xs[e] = xv;
-    }
-    for (int e = threadIdx.x; e < kWVox * cout; e += blockDim.x) {
-      const long long v = v0 + e / cout;
-      gs[e] = v < nv ? gy[v * cout + e % cout] : 0.f;
+      gs[2 * e] = g0;
+      gs[2 * e + 1] = g1;
     }
     __syncthreads();
+    for (int row = warp; row < kBX * kBY; row += 8) {
+      const uint4* xr = xs + (row / kBY) * kWPlane + (row % kBY) * kWRow + toff;
+      const float4* gr = gs + 2 * row * kBZ;
+#pragma unroll 4
+      for (int z = 0; z < kBZ; ++z) {
+        float xv[8];
+        if (U == 1) {
+          const uint4 q = xr[z];
+          xv[0] = __uint_as_float(q.x << 16); xv[1] = __uint_as_float(q.x & 0xffff0000u);
+          xv[2] = __uint_as_float(q.y << 16); xv[3] = __uint_as_float(q.y & 0xffff0000u);
+          xv[4] = __uint_as_float(q.z << 16); xv[5] = __uint_as_float(q.z & 0xffff0000u);
+          xv[6] = __uint_as_float(q.w << 16); xv[7] = __uint_as_float(q.w & 0xffff0000u);
+        } else {
+          const uint4 q = xr[z], q2 = xr[z + (U - 1) * kHX * kWPlane];
+          xv[0] = __uint_as_float(q.x); xv[1] = __uint_as_float(q.y); xv[2] = __uint_as_float(q.z); xv[3] = __uint_as_float(q.w);
+          xv[4] = __uint_as_float(q2.x); xv[5] = __uint_as_float(q2.y); xv[6] = __uint_as_float(q2.z); xv[7] = __uint_as_float(q2.w);
+        }
+        if (ones) xv[0] = 1.f;
+        const float4 ga = gr[2 * z], gc = gr[2 * z + 1];
 #pragma unroll
-    for (int k = 0; k < kWPairs; ++k) {
-      const int p = threadIdx.x + k * 256;
-      if (p < P) {
-        const int ci = p / cout, co = p % cout;
-        float a = acc[k];
-        for (int lv = 0; lv < kWVox; ++lv) a = fmaf(xs[lv * cin + ci], gs[lv * cout + co], a);
-        acc[k] = a;
+        for (int i = 0; i < 8; ++i) {
+          const float2 xx = make_float2(xv[i], xv[i]);
+          acc[i][0] = __ffma2_rn(xx, make_float2(ga.x, ga.y), acc[i][0]);
+          acc[i][1] = __ffma2_rn(xx, make_float2(ga.z, ga.w), acc[i][1]);
+          acc[i][2] = __ffma2_rn(xx, make_float2(gc.x, gc.y), acc[i][2]);
+          acc[i][3] = __ffma2_rn(xx, make_float2(gc.z, gc.w), acc[i][3]);
+        }
       }
     }
   }
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(gsm);                // [28][64], padded to 65
+  for (int k = 0; k < 8; ++k) {
+    if (warp == k && lane < 28) {
 #pragma unroll
-  for (int k = 0; k < kWPairs; ++k) {
-    const int p = threadIdx.x + k * 256;
-    if (p < P) atomicAdd(gw + (size_t)t * P + p, acc[k]);
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float* d = red + lane * 65 + 8 * i + 2 * c;
+          d[0] = k ? d[0] + acc[i][c].x : acc[i][c].x;
+          d[1] = k ? d[1] + acc[i][c].y : acc[i][c].y;
+        }
+    }
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < 28 * 64; e += 256) {
+    const int tt = e >> 6, i = (e >> 3) & 7, c = e & 7;
+    const float v = red[tt * 65 + (e & 63)];
+    if (tt < 27) {
+      if (c0 + i < cin) atomicAdd(gw + ((size_t)tt * cin + c0 + i) * cout + o0 + c, v);
+    } else if (cg == 0 && i == 0) {
+      atomicAdd(gb + o0 + c, v);
+    }
   }
 }
-
-__global__ void bias_grad_kernel(const float* __restrict__ gy, int cout, long long nv, float* __restrict__ gb) {
-  __shared__ float sh[256];
-  for (int co = 0; co < cout; ++co) {
-    float s = 0.f;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (long long)gridDim.x * blockDim.x)
-      s += gy[v * cout + co];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(gb + co, sh[0]);
-    __syncthreads();
-  }
-}
-
 template <typename T>
-__global__ void relu_backward_kernel(float* __restrict__ g, const T* __restrict__ y, long long m) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x)
-    if (!(tof(y[i]) > 0.f)) g[i] = 0.f;
+constexpr size_t wgrad_smem() {
+  return (size_t)(sizeof(T) / 2) * kHX * kWPlane * 16 + (size_t)kBX * kBY * kBZ * 32;
+}
+
+// ---- loss and head backward in one pass: d = y - t, loss += d^2 / m, g = 2 d / m; the head's weight and
+// bias gradients; gd = g w masked by the ReLU of its input --------------------------------------------
+template <typename T, int CIN>
+__global__ void __launch_bounds__(256) head_back_kernel(const float* __restrict__ y, const float* __restrict__ t,
+                                                        const T* __restrict__ x, const T* __restrict__ w, long long m,
+                                                        float* __restrict__ gx, float* __restrict__ gw,
+                                                        float* __restrict__ gb, double* __restrict__ loss) {
+  double s = 0.0;
+  const float sc = 2.f / (float)m;
+  float aw[CIN], ab = 0.f, wv[CIN];
+#pragma unroll
+  for (int c = 0; c < CIN; ++c) {
+    aw[c] = 0.f;
+    wv[c] = tof(w[c]);
+  }
+  for (long long v = (long long)blockIdx.x * 256 + threadIdx.x; v < m; v += (long long)gridDim.x * 256) {
+    const float d = y[v] - t[v], g = sc * d;
+    s += (double)d * d;
+    ab += g;
+#pragma unroll
+    for (int c0 = 0; c0 < CIN; c0 += 8) {
+      float xv[8];
+      load8(x + v * CIN + c0, xv);
+      float o[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        aw[c0 + i] = fmaf(xv[i], g, aw[c0 + i]);
+        o[i] = xv[i] > 0.f ? g * wv[c0 + i] : 0.f;
+      }
+      float4* p = reinterpret_cast<float4*>(gx + v * CIN + c0);
+      p[0] = make_float4(o[0], o[1], o[2], o[3]);
+      p[1] = make_float4(o[4], o[5], o[6], o[7]);
+    }
+  }
+  __shared__ double sh[8];
+  __shared__ float shf[8][CIN + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_down_sync(0xffffffffu, s, o);
+    ab += __shfl_down_sync(0xffffffffu, ab, o);
+#pragma unroll
+    for (int c = 0; c < CIN; ++c) aw[c] += __shfl_down_sync(0xffffffffu, aw[c], o);
+  }
+  if (lane == 0) {
+    sh[warp] = s;
+    shf[warp][CIN] = ab;
+#pragma unroll
+    for (int c = 0; c < CIN; ++c) shf[warp][c] = aw[c];
+  }
+  __syncthreads();
+  if (threadIdx.x <= CIN) {
+    float r = 0.f;
+    for (int k = 0; k < 8; ++k) r += shf[k][threadIdx.x];
+    atomicAdd(threadIdx.x < CIN ? gw + threadIdx.x : gb, r);
+  }
+  if (threadIdx.x == 32) {
+    double r = 0.0;
+    for (int k = 0; k < 8; ++k) r += sh[k];
+    atomicAdd(loss, r / (double)m);
+  }
 }
 
 // 2x2x2 average pooling: coarse n/2 grid
@@ -250,44 +480,49 @@ __global__ void pool_kernel(const T* __restrict__ x, int c, int n, T* __restrict
   }
 }
 
-__global__ void pool_backward_kernel(const float* __restrict__ g, int c, int n, float* __restrict__ gx, int accum) {
-  const long long tot = (long long)n * n * n * c;
-  const int m = n / 2;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    const long long f = i / c;
-    const int x = (int)(f / ((long long)n * n)), y = (int)((f / n) % n), z = (int)(f % n);
-    const float v = 0.125f * g[(((long long)(x >> 1) * m + (y >> 1)) * m + (z >> 1)) * c + ch];
-    gx[i] = accum ? gx[i] + v : v;
-  }
-}
-
-// nearest-neighbour 2x upsampling from the coarse n/2 grid to n
+// gx += pooled gradient / 8, then the ReLU of the pooled activation (c a multiple of 4)
 template <typename T>
-__global__ void up_kernel(const T* __restrict__ x, int c, int n, T* __restrict__ y) {
-  const long long tot = (long long)n * n * n * c;
-  const int m = n / 2;
+__global__ void pool_backward_kernel(const float* __restrict__ g, int c, int n, float* __restrict__ gx,
+                                     const T* __restrict__ mask) {
+  const int m = n / 2, c4 = c / 4;
+  const long long tot = (long long)n * n * n * c4;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    const long long f = i / c;
-    const int X = (int)(f / ((long long)n * n)), Y = (int)((f / n) % n), Z = (int)(f % n);
-    y[i] = x[(((long long)(X >> 1) * m + (Y >> 1)) * m + (Z >> 1)) * c + ch];
+    const int ch = (int)(i % c4);
+    const int f = (int)(i / c4), x = f / (n * n), y = (f / n) % n, z = f % n;
+    const float4 p = reinterpret_cast<const float4*>(g)[(((long long)(x >> 1) * m + (y >> 1)) * m + (z >> 1)) * c4 + ch];
+    float4 v = reinterpret_cast<const float4*>(gx)[i];
+    v = make_float4(v.x + 0.125f * p.x, v.y + 0.125f * p.y, v.z + 0.125f * p.z, v.w + 0.125f * p.w);
+    const T* k = mask + 4 * i;
+    if (!(tof(k[0]) > 0.f)) v.x = 0.f;
+    if (!(tof(k[1]) > 0.f)) v.y = 0.f;
+    if (!(tof(k[2]) > 0.f)) v.z = 0.f;
+    if (!(tof(k[3]) > 0.f)) v.w = 0.f;
+    reinterpret_cast<float4*>(gx)[i] = v;
   }
 }
 
-__global__ void up_backward_kernel(const float* __restrict__ g, int c, int n, float* __restrict__ gx) {
-  const int m = n / 2;
-  const long long tot = (long long)m * m * m * c;
+// sum over the 8 upsampled copies, then the ReLU of the coarse activation (c a multiple of 4)
+template <typename T>
+__global__ void up_backward_kernel(const float* __restrict__ g, int c, int n, float* __restrict__ gx,
+                                   const T* __restrict__ mask) {
+  const int m = n / 2, c4 = c / 4;
+  const long long tot = (long long)m * m * m * c4;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    const long long cv = i / c;
-    const int X = (int)(cv / ((long long)m * m)), Y = (int)((cv / m) % m), Z = (int)(cv % m);
-    float s = 0.f;
+    const int ch = (int)(i % c4);
+    const int cv = (int)(i / c4), X = cv / (m * m), Y = (cv / m) % m, Z = cv % m;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
     for (int a = 0; a < 8; ++a) {
       const long long f = ((long long)(2 * X + (a >> 2)) * n + (2 * Y + ((a >> 1) & 1))) * n + (2 * Z + (a & 1));
-      s += g[f * c + ch];
+      const float4 p = reinterpret_cast<const float4*>(g)[f * c4 + ch];
+      s = make_float4(s.x + p.x, s.y + p.y, s.z + p.z, s.w + p.w);
     }
-    gx[i] = s;
+    const T* k = mask + 4 * i;
+    if (!(tof(k[0]) > 0.f)) s.x = 0.f;
+    if (!(tof(k[1]) > 0.f)) s.y = 0.f;
+    if (!(tof(k[2]) > 0.f)) s.z = 0.f;
+    if (!(tof(k[3]) > 0.f)) s.w = 0.f;
+    reinterpret_cast<float4*>(gx)[i] = s;
   }
 }
 
@@ -297,34 +532,17 @@ __global__ void to_t_kernel(const float* __restrict__ x, T* __restrict__ y, long
     y[i] = fromf<T>(x[i]);
 }
 
-// network input for the tensor-core path: 5 float32 channels -> 8 bf16 channels (16 bytes a voxel)
-__global__ void to_x8_kernel(const float* __restrict__ x, int cin, long long nv, bf16* __restrict__ y) {
+// network input: 5 float32 channels -> 8 stored channels a voxel, the last ones zero
+template <typename T>
+__global__ void to_x8_kernel(const float* __restrict__ x, int cin, long long nv, T* __restrict__ y) {
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (long long)gridDim.x * blockDim.x) {
-    __align__(16) bf16 o[8];
+    __align__(16) T o[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) o[c] = __float2bfloat16_rn(c < cin ? x[v * cin + c] : 0.f);
-    *reinterpret_cast<uint4*>(y + v * 8) = *reinterpret_cast<const uint4*>(o);
+    for (int c = 0; c < 8; ++c) o[c] = fromf<T>(c < cin ? x[v * cin + c] : 0.f);
+#pragma unroll
+    for (int b = 0; b < (int)sizeof(T) / 2; ++b)
+      reinterpret_cast<uint4*>(y + v * 8)[b] = reinterpret_cast<const uint4*>(o)[b];
   }
-}
-
-// mean squared error: g = 2 (y - t) / m, loss = sum (y - t)^2 / m (float64 accumulation)
-__global__ void mse_kernel(const float* __restrict__ y, const float* __restrict__ t, long long m, float* __restrict__ g,
-                           double* __restrict__ loss) {
-  __shared__ double sh[256];
-  double s = 0.0;
-  const float sc = 2.f / (float)m;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
-    const float d = y[i] - t[i];
-    g[i] = sc * d;
-    s += (double)d * d;
-  }
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicAdd(loss, sh[0] / (double)m);
 }
 
 // decoupled weight decay Adam on the float32 master weights; refreshes the stored-type copy
@@ -409,7 +627,7 @@ void make_spec(recon_unet* u) {
 
 // activation layout for one grid of side n (offsets in elements of the stored type)
 struct Acts {
-  size_t x, a1a, a1b, p1, a2a, a2b, p2, a3a, a3b, u3, d2a, d2b, u2, d1a, d1b, x8, total;
+  size_t a1a, a1b, p1, a2a, a2b, p2, a3a, a3b, d2a, d2b, d1a, d1b, x8, total;
 };
 Acts act_layout(const recon_unet* u, int n) {
   const size_t V1 = (size_t)n * n * n, V2 = V1 / 8, V3 = V1 / 64;
@@ -417,18 +635,17 @@ Acts act_layout(const recon_unet* u, int n) {
   Acts a{};
   size_t o = 0;
   auto take = [&](size_t k) { size_t r = o; o += (k + 127) & ~(size_t)127; return r; };
-  a.x = take(V1 * u->cin);
   a.a1a = take(V1 * c1); a.a1b = take(V1 * c1); a.p1 = take(V2 * c1);
   a.a2a = take(V2 * c2); a.a2b = take(V2 * c2); a.p2 = take(V3 * c2);
-  a.a3a = take(V3 * c3); a.a3b = take(V3 * c3); a.u3 = take(V2 * c3);
-  a.d2a = take(V2 * c2); a.d2b = take(V2 * c2); a.u2 = take(V1 * c2);
+  a.a3a = take(V3 * c3); a.a3b = take(V3 * c3);
+  a.d2a = take(V2 * c2); a.d2b = take(V2 * c2);
   a.d1a = take(V1 * c1); a.d1b = take(V1 * c1);
   a.x8 = take(V1 * 8);
   a.total = o;
   return a;
 }
 struct Grads {
-  size_t gy, gd1b, gd1a, gu2, gs1, gd2b, gd2a, gu3, gs2, ga3b, ga3a, gp2, ga2a, gp1, ga1a, total;
+  size_t gd1b, gd1a, gu2, gs1, gd2b, gd2a, gu3, gs2, ga3b, ga3a, gp2, ga2a, gp1, ga1a, total;
 };
 Grads grad_layout(const recon_unet* u, int n) {
   const size_t V1 = (size_t)n * n * n, V2 = V1 / 8, V3 = V1 / 64;
@@ -436,7 +653,7 @@ Grads grad_layout(const recon_unet* u, int n) {
   Grads g{};
   size_t o = 0;
   auto take = [&](size_t k) { size_t r = o; o += (k + 63) & ~(size_t)63; return r; };
-  g.gy = take(V1); g.gd1b = take(V1 * c1); g.gd1a = take(V1 * c1); g.gu2 = take(V1 * c2); g.gs1 = take(V1 * c1);
+  g.gd1b = take(V1 * c1); g.gd1a = take(V1 * c1); g.gu2 = take(V1 * c2); g.gs1 = take(V1 * c1);
   g.gd2b = take(V2 * c2); g.gd2a = take(V2 * c2); g.gu3 = take(V2 * c3); g.gs2 = take(V2 * c2);
   g.ga3b = take(V3 * c3); g.ga3a = take(V3 * c3); g.gp2 = take(V3 * c2); g.ga2a = take(V2 * c2);
   g.gp1 = take(V2 * c1); g.ga1a = take(V1 * c1);
@@ -474,21 +691,27 @@ recon_status ensure(recon_unet* u, int n, bool train) {
   return RECON_OK;
 }
 
+// One 3x3x3 layer on the CUDA cores: xa holds ca channels a voxel, cina of them with weights; up: xa is
+// read from the coarse grid of half the side (nearest upsampling).
 template <typename T>
-cudaError_t conv_fwd(recon_unet* u, int li, const T* xa, int ca, const T* xb, int cb, int n, int relu,
-                     const float* res, int res_stride, T* y, float* yf) {
+cudaError_t conv_fwd(recon_unet* u, int li, const T* xa, int ca, int cina, int up, const T* xb, int cb, int n, T* y) {
   const Spec& s = u->spec[li];
   const T* w = static_cast<const T*>(u->pt) + u->woff[li];
   const float* b = u->p + u->boff[li];
   const long long nv = (long long)n * n * n;
-  const int blocks = (int)((nv + 127) / 128);
-  const size_t smem = sizeof(float) * s.cin * s.cout;
+  cudaError_t e = cudaSuccess;
   switch (s.cout) {
-#define UN_CASE(C)                                                                                   \
-  case C:                                                                                           \
-    conv_fwd_kernel<T, C><<<blocks, 128, smem, u->st>>>(xa, ca, xb, cb, w, b, s.ntap, n, relu, res, res_stride, y, yf); \
-    break;
-    UN_CASE(1) UN_CASE(8) UN_CASE(16) UN_CASE(32) UN_CASE(64) UN_CASE(128)
+#define UN_CASE(C)                                                                                              \
+  case C: {                                                                                                     \
+    using F = ConvFwd<T, C>;                                                                                    \
+    const size_t smem = sizeof(float) * F::TG * s.cin * C;                                                      \
+    e = cudaFuncSetAttribute((const void*)conv_fwd_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    if (e != cudaSuccess) return e;                                                                             \
+    conv_fwd_kernel<T, C><<<(unsigned)((nv + 256 * F::VPT - 1) / (256 * F::VPT)), 256, smem, u->st>>>(          \
+        xa, ca, cina, up, xb, cb, w, b, n, y);                                                                      \
+    break;                                                                                                      \
+  }
+    UN_CASE(8) UN_CASE(16) UN_CASE(32) UN_CASE(64)
 #undef UN_CASE
     default:
       return cudaErrorInvalidValue;
@@ -497,22 +720,37 @@ cudaError_t conv_fwd(recon_unet* u, int li, const T* xa, int ca, const T* xb, in
 }
 
 template <typename T>
-cudaError_t conv_back(recon_unet* u, int li, const T* xa, int ca, const T* xb, int cb, const float* gy, int n,
-                      float* gxa, float* gxb, int accum_b) {
+cudaError_t head_fwd(recon_unet* u, const T* x, const float* res, int res_stride, int n, float* y) {
+  const T* w = static_cast<const T*>(u->pt) + u->woff[10];
+  const float* b = u->p + u->boff[10];
+  const long long nv = (long long)n * n * n;
+  const unsigned blocks = (unsigned)((nv + 255) / 256);
+  if (u->c1 == 8) head_fwd_kernel<T, 8><<<blocks, 256, 0, u->st>>>(x, w, b, res, res_stride, nv, y);
+  else head_fwd_kernel<T, 16><<<blocks, 256, 0, u->st>>>(x, w, b, res, res_stride, nv, y);
+  return cudaGetLastError();
+}
+
+// Gradients of one 3x3x3 layer: weights and bias, and (gxa, gxb not null) its inputs.  up: xa is read
+// from the coarse grid of half the side (nearest upsampling).
+template <typename T>
+cudaError_t conv_back(recon_unet* u, int li, const T* xa, int ca, int cina, int up, const T* xb, int cb, const float* gy,
+                      int n, float* gxa, float* gxb, const T* mask) {
   const Spec& s = u->spec[li];
   const T* w = static_cast<const T*>(u->pt) + u->woff[li];
-  const long long nv = (long long)n * n * n;
-  float* gw = u->g + u->woff[li];
-  float* gb = u->g + u->boff[li];
-  if (s.cin * s.cout > 256 * kWPairs) return cudaErrorInvalidValue;
-  const int wblocks = (int)((nv + kWVox - 1) / kWVox < 304 ? (nv + kWVox - 1) / kWVox : 304);
-  conv_wgrad_kernel<T><<<dim3(wblocks, s.ntap), 256, sizeof(float) * kWVox * (s.cin + s.cout), u->st>>>(
-      xa, ca, xb, cb, gy, s.cout, s.ntap, n, gw);
-  bias_grad_kernel<<<grid_for(nv) < 304 ? grid_for(nv) : 304, 256, 0, u->st>>>(gy, s.cout, nv, gb);
-  if (gxa || gxb) {
-    dim3 grid((unsigned)((nv + 127) / 128), (unsigned)((s.cin + kDChunk - 1) / kDChunk));
-    conv_dgrad_kernel<T><<<grid, 128, sizeof(float) * kDChunk * s.cout, u->st>>>(gy, s.cout, w, ca, cb, s.ntap, n,
-                                                                                 gxa, gxb, accum_b);
+  const int tiles = TileGrid(n).count();
+  cudaError_t e = cudaFuncSetAttribute((const void*)conv_wgrad_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)wgrad_smem<T>());
+  if (e != cudaSuccess) return e;
+  const int groups = ((s.cin + 7) / 8) * (s.cout / 8);
+  // two blocks per SM over all channel groups together, at least one tile each
+  int per = (2 * 152 + groups - 1) / groups;
+  if (per > tiles) per = tiles;
+  conv_wgrad_kernel<T><<<dim3(per, groups), 256, wgrad_smem<T>(), u->st>>>(xa, ca, cina, up, xb, cb, gy, s.cout, n,
+                                                                          u->g + u->woff[li], u->g + u->boff[li]);
+  if (gxa) {
+    e = cudaFuncSetAttribute((const void*)conv_dgrad_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDSmem);
+    if (e != cudaSuccess) return e;
+    conv_dgrad_kernel<T><<<dim3(tiles, s.cin / 8), 128, kDSmem, u->st>>>(gy, s.cout, w, ca, cb, n, gxa, gxb, mask);
   }
   return cudaGetLastError();
 }
@@ -523,22 +761,20 @@ recon_status forward_t(recon_unet* u, const float* x, int n, float* out) {
   T* a = static_cast<T*>(u->acts);
   const int c1 = u->c1, c2 = 2 * c1, c3 = 4 * c1, n2 = n / 2, n4 = n / 4;
   const long long V1 = (long long)n * n * n;
-  to_t_kernel<T><<<grid_for(V1 * u->cin), 256, 0, u->st>>>(x, a + A.x, V1 * u->cin);
-  UN_CUDA(conv_fwd<T>(u, 0, a + A.x, u->cin, nullptr, 0, n, 1, nullptr, 0, a + A.a1a, nullptr));
-  UN_CUDA(conv_fwd<T>(u, 1, a + A.a1a, c1, nullptr, 0, n, 1, nullptr, 0, a + A.a1b, nullptr));
+  to_x8_kernel<T><<<grid_for(V1), 256, 0, u->st>>>(x, u->cin, V1, a + A.x8);
+  UN_CUDA(conv_fwd<T>(u, 0, a + A.x8, 8, u->cin, 0, nullptr, 0, n, a + A.a1a));
+  UN_CUDA(conv_fwd<T>(u, 1, a + A.a1a, c1, c1, 0, nullptr, 0, n, a + A.a1b));
   pool_kernel<T><<<grid_for(V1 / 8 * c1), 256, 0, u->st>>>(a + A.a1b, c1, n, a + A.p1);
-  UN_CUDA(conv_fwd<T>(u, 2, a + A.p1, c1, nullptr, 0, n2, 1, nullptr, 0, a + A.a2a, nullptr));
-  UN_CUDA(conv_fwd<T>(u, 3, a + A.a2a, c2, nullptr, 0, n2, 1, nullptr, 0, a + A.a2b, nullptr));
+  UN_CUDA(conv_fwd<T>(u, 2, a + A.p1, c1, c1, 0, nullptr, 0, n2, a + A.a2a));
+  UN_CUDA(conv_fwd<T>(u, 3, a + A.a2a, c2, c2, 0, nullptr, 0, n2, a + A.a2b));
   pool_kernel<T><<<grid_for(V1 / 64 * c2), 256, 0, u->st>>>(a + A.a2b, c2, n2, a + A.p2);
-  UN_CUDA(conv_fwd<T>(u, 4, a + A.p2, c2, nullptr, 0, n4, 1, nullptr, 0, a + A.a3a, nullptr));
-  UN_CUDA(conv_fwd<T>(u, 5, a + A.a3a, c3, nullptr, 0, n4, 1, nullptr, 0, a + A.a3b, nullptr));
-  up_kernel<T><<<grid_for(V1 / 8 * c3), 256, 0, u->st>>>(a + A.a3b, c3, n2, a + A.u3);
-  UN_CUDA(conv_fwd<T>(u, 6, a + A.u3, c3, a + A.a2b, c2, n2, 1, nullptr, 0, a + A.d2a, nullptr));
-  UN_CUDA(conv_fwd<T>(u, 7, a + A.d2a, c2, nullptr, 0, n2, 1, nullptr, 0, a + A.d2b, nullptr));
-  up_kernel<T><<<grid_for(V1 * c2), 256, 0, u->st>>>(a + A.d2b, c2, n, a + A.u2);
-  UN_CUDA(conv_fwd<T>(u, 8, a + A.u2, c2, a + A.a1b, c1, n, 1, nullptr, 0, a + A.d1a, nullptr));
-  UN_CUDA(conv_fwd<T>(u, 9, a + A.d1a, c1, nullptr, 0, n, 1, nullptr, 0, a + A.d1b, nullptr));
-  UN_CUDA(conv_fwd<T>(u, 10, a + A.d1b, c1, nullptr, 0, n, 0, x + (u->cin - 1), u->cin, nullptr, out));
+  UN_CUDA(conv_fwd<T>(u, 4, a + A.p2, c2, c2, 0, nullptr, 0, n4, a + A.a3a));
+  UN_CUDA(conv_fwd<T>(u, 5, a + A.a3a, c3, c3, 0, nullptr, 0, n4, a + A.a3b));
+  UN_CUDA(conv_fwd<T>(u, 6, a + A.a3b, c3, c3, 1, a + A.a2b, c2, n2, a + A.d2a));
+  UN_CUDA(conv_fwd<T>(u, 7, a + A.d2a, c2, c2, 0, nullptr, 0, n2, a + A.d2b));
+  UN_CUDA(conv_fwd<T>(u, 8, a + A.d2b, c2, c2, 1, a + A.a1b, c1, n, a + A.d1a));
+  UN_CUDA(conv_fwd<T>(u, 9, a + A.d1a, c1, c1, 0, nullptr, 0, n, a + A.d1b));
+  UN_CUDA(head_fwd<T>(u, a + A.d1b, x + (u->cin - 1), u->cin, n, out));
   return RECON_OK;
 }
 
@@ -611,16 +847,12 @@ recon_status forward_tc(recon_unet* u, const float* x, int n, float* out) {
   auto plain = [&](int l, const bf16* s0, int ca, bf16* y, int nl) -> cudaError_t {
     if (u->plan_ok[l]) return run(l, s0, nullptr, y);
     ++u->launches;
-    return conv_fwd<bf16>(u, l, s0, ca, nullptr, 0, nl, 1, nullptr, 0, y, nullptr);
+    return conv_fwd<bf16>(u, l, s0, ca, ca, 0, nullptr, 0, nl, y);
   };
   u->launches += 3;   // input conversion and the two poolings
-  if (u->plan_ok[0]) {
-    to_x8_kernel<<<grid_for(V1), 256, 0, u->st>>>(x, u->cin, V1, a + A.x8);
-    UN_CUDA(run(0, a + A.x8, nullptr, a + A.a1a));
-  } else {
-    to_t_kernel<bf16><<<grid_for(V1 * u->cin), 256, 0, u->st>>>(x, a + A.x, V1 * u->cin);
-    UN_CUDA(conv_fwd<bf16>(u, 0, a + A.x, u->cin, nullptr, 0, n, 1, nullptr, 0, a + A.a1a, nullptr));
-  }
+  to_x8_kernel<bf16><<<grid_for(V1), 256, 0, u->st>>>(x, u->cin, V1, a + A.x8);
+  if (u->plan_ok[0]) UN_CUDA(run(0, a + A.x8, nullptr, a + A.a1a));
+  else UN_CUDA(conv_fwd<bf16>(u, 0, a + A.x8, 8, u->cin, 0, nullptr, 0, n, a + A.a1a));
   UN_CUDA(plain(1, a + A.a1a, c1, a + A.a1b, n));
   pool_kernel<bf16><<<grid_for(V1 / 8 * c1), 256, 0, u->st>>>(a + A.a1b, c1, n, a + A.p1);
   UN_CUDA(plain(2, a + A.p1, c1, a + A.a2a, n2));
@@ -631,17 +863,15 @@ recon_status forward_tc(recon_unet* u, const float* x, int n, float* out) {
   if (u->plan_ok[6]) {
     UN_CUDA(run(6, a + A.a3b, a + A.a2b, a + A.d2a));
   } else {
-    u->launches += 2;
-    up_kernel<bf16><<<grid_for(V1 / 8 * c3), 256, 0, u->st>>>(a + A.a3b, c3, n2, a + A.u3);
-    UN_CUDA(conv_fwd<bf16>(u, 6, a + A.u3, c3, a + A.a2b, c2, n2, 1, nullptr, 0, a + A.d2a, nullptr));
+    ++u->launches;
+    UN_CUDA(conv_fwd<bf16>(u, 6, a + A.a3b, c3, c3, 1, a + A.a2b, c2, n2, a + A.d2a));
   }
   UN_CUDA(plain(7, a + A.d2a, c2, a + A.d2b, n2));
   if (u->plan_ok[8]) {
     UN_CUDA(run(8, a + A.d2b, a + A.a1b, a + A.d1a));
   } else {
-    u->launches += 2;
-    up_kernel<bf16><<<grid_for(V1 * c2), 256, 0, u->st>>>(a + A.d2b, c2, n, a + A.u2);
-    UN_CUDA(conv_fwd<bf16>(u, 8, a + A.u2, c2, a + A.a1b, c1, n, 1, nullptr, 0, a + A.d1a, nullptr));
+    ++u->launches;
+    UN_CUDA(conv_fwd<bf16>(u, 8, a + A.d2b, c2, c2, 1, a + A.a1b, c1, n, a + A.d1a));
   }
   u->head_fused = u->plan_ok[9] && u->plan[9].orient == 0;
   if (u->head_fused) {
@@ -660,7 +890,7 @@ recon_status forward_tc(recon_unet* u, const float* x, int n, float* out) {
   } else {
     ++u->launches;
     UN_CUDA(plain(9, a + A.d1a, c1, a + A.d1b, n));
-    UN_CUDA(conv_fwd<bf16>(u, 10, a + A.d1b, c1, nullptr, 0, n, 0, x + (u->cin - 1), u->cin, nullptr, out));
+    UN_CUDA(head_fwd<bf16>(u, a + A.d1b, x + (u->cin - 1), u->cin, n, out));
   }
   int flag = 0;
   UN_CUDA(cudaMemcpyAsync(&flag, u->dev_err, sizeof(int), cudaMemcpyDeviceToHost, u->st));
@@ -685,35 +915,26 @@ recon_status backward_t(recon_unet* u, const float* x, const float* target, int 
   const long long V1 = (long long)n * n * n, V2 = V1 / 8, V3 = V1 / 64;
   UN_CUDA(cudaMemsetAsync(u->g, 0, u->np * sizeof(float), u->st));
   UN_CUDA(cudaMemsetAsync(u->loss, 0, sizeof(double), u->st));
-  mse_kernel<<<grid_for(V1) < 304 ? grid_for(V1) : 304, 256, 0, u->st>>>(u->y, target, V1, g + G.gy, u->loss);
-  auto relu_b = [&](float* gp, const T* yp, long long m) {
-    relu_backward_kernel<T><<<grid_for(m), 256, 0, u->st>>>(gp, yp, m);
-  };
-  UN_CUDA(conv_back<T>(u, 10, a + A.d1b, c1, nullptr, 0, g + G.gy, n, g + G.gd1b, nullptr, 0));
-  relu_b(g + G.gd1b, a + A.d1b, V1 * c1);
-  UN_CUDA(conv_back<T>(u, 9, a + A.d1a, c1, nullptr, 0, g + G.gd1b, n, g + G.gd1a, nullptr, 0));
-  relu_b(g + G.gd1a, a + A.d1a, V1 * c1);
-  UN_CUDA(conv_back<T>(u, 8, a + A.u2, c2, a + A.a1b, c1, g + G.gd1a, n, g + G.gu2, g + G.gs1, 0));
-  up_backward_kernel<<<grid_for(V2 * c2), 256, 0, u->st>>>(g + G.gu2, c2, n, g + G.gd2b);
-  relu_b(g + G.gd2b, a + A.d2b, V2 * c2);
-  UN_CUDA(conv_back<T>(u, 7, a + A.d2a, c2, nullptr, 0, g + G.gd2b, n2, g + G.gd2a, nullptr, 0));
-  relu_b(g + G.gd2a, a + A.d2a, V2 * c2);
-  UN_CUDA(conv_back<T>(u, 6, a + A.u3, c3, a + A.a2b, c2, g + G.gd2a, n2, g + G.gu3, g + G.gs2, 0));
-  up_backward_kernel<<<grid_for(V3 * c3), 256, 0, u->st>>>(g + G.gu3, c3, n2, g + G.ga3b);
-  relu_b(g + G.ga3b, a + A.a3b, V3 * c3);
-  UN_CUDA(conv_back<T>(u, 5, a + A.a3a, c3, nullptr, 0, g + G.ga3b, n4, g + G.ga3a, nullptr, 0));
-  relu_b(g + G.ga3a, a + A.a3a, V3 * c3);
-  UN_CUDA(conv_back<T>(u, 4, a + A.p2, c2, nullptr, 0, g + G.ga3a, n4, g + G.gp2, nullptr, 0));
-  pool_backward_kernel<<<grid_for(V2 * c2), 256, 0, u->st>>>(g + G.gp2, c2, n2, g + G.gs2, 1);
-  relu_b(g + G.gs2, a + A.a2b, V2 * c2);
-  UN_CUDA(conv_back<T>(u, 3, a + A.a2a, c2, nullptr, 0, g + G.gs2, n2, g + G.ga2a, nullptr, 0));
-  relu_b(g + G.ga2a, a + A.a2a, V2 * c2);
-  UN_CUDA(conv_back<T>(u, 2, a + A.p1, c1, nullptr, 0, g + G.ga2a, n2, g + G.gp1, nullptr, 0));
-  pool_backward_kernel<<<grid_for(V1 * c1), 256, 0, u->st>>>(g + G.gp1, c1, n, g + G.gs1, 1);
-  relu_b(g + G.gs1, a + A.a1b, V1 * c1);
-  UN_CUDA(conv_back<T>(u, 1, a + A.a1a, c1, nullptr, 0, g + G.gs1, n, g + G.ga1a, nullptr, 0));
-  relu_b(g + G.ga1a, a + A.a1a, V1 * c1);
-  UN_CUDA(conv_back<T>(u, 0, a + A.x, u->cin, nullptr, 0, g + G.ga1a, n, nullptr, nullptr, 0));
+  const int hb = grid_for(V1) < 608 ? grid_for(V1) : 608;
+  float *gw10 = u->g + u->woff[10], *gb10 = u->g + u->boff[10];
+  const T* w10 = static_cast<const T*>(u->pt) + u->woff[10];
+  if (c1 == 8) head_back_kernel<T, 8><<<hb, 256, 0, u->st>>>(u->y, target, a + A.d1b, w10, V1, g + G.gd1b, gw10, gb10, u->loss);
+  else head_back_kernel<T, 16><<<hb, 256, 0, u->st>>>(u->y, target, a + A.d1b, w10, V1, g + G.gd1b, gw10, gb10, u->loss);
+  const T* none = nullptr;
+  UN_CUDA(conv_back<T>(u, 9, a + A.d1a, c1, c1, 0, none, 0, g + G.gd1b, n, g + G.gd1a, nullptr, a + A.d1a));
+  UN_CUDA(conv_back<T>(u, 8, a + A.d2b, c2, c2, 1, a + A.a1b, c1, g + G.gd1a, n, g + G.gu2, g + G.gs1, none));
+  up_backward_kernel<T><<<grid_for(V2 * c2 / 4), 256, 0, u->st>>>(g + G.gu2, c2, n, g + G.gd2b, a + A.d2b);
+  UN_CUDA(conv_back<T>(u, 7, a + A.d2a, c2, c2, 0, none, 0, g + G.gd2b, n2, g + G.gd2a, nullptr, a + A.d2a));
+  UN_CUDA(conv_back<T>(u, 6, a + A.a3b, c3, c3, 1, a + A.a2b, c2, g + G.gd2a, n2, g + G.gu3, g + G.gs2, none));
+  up_backward_kernel<T><<<grid_for(V3 * c3 / 4), 256, 0, u->st>>>(g + G.gu3, c3, n2, g + G.ga3b, a + A.a3b);
+  UN_CUDA(conv_back<T>(u, 5, a + A.a3a, c3, c3, 0, none, 0, g + G.ga3b, n4, g + G.ga3a, nullptr, a + A.a3a));
+  UN_CUDA(conv_back<T>(u, 4, a + A.p2, c2, c2, 0, none, 0, g + G.ga3a, n4, g + G.gp2, nullptr, none));
+  pool_backward_kernel<T><<<grid_for(V2 * c2 / 4), 256, 0, u->st>>>(g + G.gp2, c2, n2, g + G.gs2, a + A.a2b);
+  UN_CUDA(conv_back<T>(u, 3, a + A.a2a, c2, c2, 0, none, 0, g + G.gs2, n2, g + G.ga2a, nullptr, a + A.a2a));
+  UN_CUDA(conv_back<T>(u, 2, a + A.p1, c1, c1, 0, none, 0, g + G.ga2a, n2, g + G.gp1, nullptr, none));
+  pool_backward_kernel<T><<<grid_for(V1 * c1 / 4), 256, 0, u->st>>>(g + G.gp1, c1, n, g + G.gs1, a + A.a1b);
+  UN_CUDA(conv_back<T>(u, 1, a + A.a1a, c1, c1, 0, none, 0, g + G.gs1, n, g + G.ga1a, nullptr, a + A.a1a));
+  UN_CUDA(conv_back<T>(u, 0, a + A.x8, 8, u->cin, 0, none, 0, g + G.ga1a, n, nullptr, nullptr, none));
   UN_CUDA(cudaGetLastError());
   if (loss) {
     UN_CUDA(cudaMemcpyAsync(loss, u->loss, sizeof(double), cudaMemcpyDeviceToHost, u->st));
