@@ -212,13 +212,14 @@ recon_status recon_fft_c2r(recon_handle* h, const float* in_half, float* out_rea
  * 7-point Laplacian plus beta times the line-of-sight stencil of Sec. 2.1 (sets A, B and C; beta =
  * f / b; a fixed line of sight takes the second differences only), phi = 0 outside the box, then
  * Psi = -grad phi by central differences.  The linear system is solved with BiCGStab (float32
- * vectors, float64 inner products), right-preconditioned by the exact inverse of the periodic
- * 7-point Laplacian (the library's FFT passes on the handle's first field), until the recursive
+ * vectors; operator, updates and inner products in pairs of float32, about 45 bits, the products
+ * summed over blocks in float64), right-preconditioned by the exact inverse of the periodic
+ * 7-point Laplacian (the library's FFT passes on the handle's first two fields), until the recursive
  * residual falls below tol x |b|.  psi_out: device (3, N^3) float32.  *n_iter: iterations;
  * *rel_resid: the true residual |A phi - b| / |b| at the end (with phi stored in float32 it
  * bottoms out near 1e-5 for fields smooth over a few cells: rounding at the grid scale times the
- * Laplacian's 12 / g^2).  Allocates its 9 Krylov vectors
- * (9 N^3 float32) with cudaMalloc for the call.  The smoothed delta stays valid, so recon_iterate
+ * Laplacian's 12 / g^2).  Allocates its 7 Krylov vectors and
+ * the preconditioner's factor (7.5 N^3 + N^2 float32) with cudaMalloc for the call.  The smoothed delta stays valid, so recon_iterate
  * may follow.  NOT_CONVERGED when max_iter is reached; STATE before recon_smooth. */
 recon_status recon_fd_solve(recon_handle* h, double tol, int max_iter, int* n_iter, double* rel_resid,
                             float* psi_out);

@@ -16,22 +16,34 @@ struct FDArgs {
   const float* off;      // 3 N node offsets from the observer (radial)
 };
 
-// out = A phi: the 7-point Laplacian plus beta times the line-of-sight stencil of Sec. 2.1, phi = 0
-// outside the mesh; sums in float64.
-cudaError_t launch_fd_apply(const float* phi, float* out, const FDArgs& a, cudaStream_t st);
+// Scalars of the BiCGStab solve, on the device: written by the last block of the reduction that forms
+// them, read by the kernels behind it.
+struct FDState {
+  double bnorm, rho, rho_old, alpha, omega, res, tol, true_res;
+  int it;                // iterations done
+  int done;              // 0 running, 2 |s| small enough (x += alpha ph pending), 1 ended
+  unsigned int counter;  // blocks done in the running reduction (zero between kernels)
+};
+
+// The kernels of one iteration, in order; each returns at once when the solve has ended (st->done).
+// Reductions use partials (2 x 608 doubles).  pre: the vector the preconditioner transforms in place.
+cudaError_t launch_fd_init(const float* delta, float c, double inv_b, float* x, float* r, float* rh, size_t n, FDState* st,
+                           double tol, double* partials, cudaStream_t s);
+cudaError_t launch_fd_dir(const float* r, const float* v, float* p, float* pre, size_t n, const FDState* st, cudaStream_t s);
+// out = A phi (the 7-point Laplacian plus beta times the line-of-sight stencil of Sec. 2.1, phi = 0
+// outside the mesh) and its inner products: mode 0 alpha = rho / (w . out), mode 1 omega = (out . w) /
+// (out . out), mode 2 only |A phi - w| / bnorm (out unused).
+cudaError_t launch_fd_apply(int mode, const float* phi, float* out, const float* w, const FDArgs& a, FDState* st,
+                            double* partials, cudaStream_t s);
+cudaError_t launch_fd_s(const float* r, const float* v, float* sv, float* pre, size_t n, FDState* st, double* partials,
+                        cudaStream_t s);
+cudaError_t launch_fd_update(float* x, const float* ph, const float* sh, const float* sv, const float* t, const float* rh,
+                             float* r, size_t n, FDState* st, double* partials, cudaStream_t s);
 // Psi_j = -(phi(+j) - phi(-j)) / (2 g), phi = 0 outside the mesh; psi holds 3 N^3 values.
 cudaError_t launch_fd_gradient(const float* phi, float* psi, const FDArgs& a, cudaStream_t st);
-// The preconditioner's Fourier-space factor on the library's half grid (M: [kx][ky][kz < N/2],
+// The preconditioner's Fourier-space factor on the library's half grid (M: [kx][ky][kz < N/2], then
 // Q: kz = N/2): 1 / (N^3 lambda(k)), lambda the periodic 7-point Laplacian's eigenvalue
-// sum_i (2 cos(k_i g) - 2) / g^2, and -L^2 / (3 pi^2 N^3) at k = 0.
-cudaError_t launch_fd_precond_k(const Field& f, int n, double L, cudaStream_t st);
-// Per-block float64 partial sums of x . y (partials[b]), for the Krylov solver's inner products.
-cudaError_t launch_dot(const float* x, const float* y, size_t n, double* partials, int blocks, cudaStream_t st);
-// y = x + a (y - b z)  (BiCGStab's search direction: p = r + beta (p - omega v))
-cudaError_t launch_fd_dir(float* y, const float* x, const float* z, double a, double b, size_t n, cudaStream_t st);
-// y = x - a z
-cudaError_t launch_fd_sub(float* y, const float* x, const float* z, double a, size_t n, cudaStream_t st);
-// y += a x + b z
-cudaError_t launch_fd_acc(float* y, const float* x, const float* z, double a, double b, size_t n, cudaStream_t st);
+// sum_i (2 cos(k_i g) - 2) / g^2, and -L^2 / (3 pi^2 N^3) at k = 0; N^2 (N/2 + 1) floats.
+cudaError_t launch_fd_factor(float* fac, int n, double L, cudaStream_t st);
 
 }  // namespace rg

@@ -1068,11 +1068,22 @@ __global__ void __launch_bounds__(SThreads<N, MODE, NARROW>::v, SThreads<N, MODE
   }
 
   // ---- forward transform along the line
-  if (MODE == S_FWD || MODE == S_ITER) {
+  if (MODE == S_FWD || MODE == S_ITER || MODE == S_FACTOR) {
 #pragma unroll
     for (int q = 0; q < ((MODE == S_ITER && RED) ? 2 : NC); ++q) Plan<N>::template run<C, T, false, Lay>(s + q * N * C, tw);
   } else if (MODE == S_DELTA) {
     if (!a.d_is_k) Plan<N>::template run<C, T, false, Lay>(s, tw);
+  }
+
+  if (MODE == S_FACTOR) {
+    const float* __restrict__ fac = a.fac + (t.isQ ? (size_t)N * N * H : 0);
+    for (int e = threadIdx.x; e < N * C; e += T) {
+      // consecutive threads on consecutive elements of the field, as the tile was loaded
+      const int i = t.cs == 1 ? e / C : e % N, c = t.cs == 1 ? e % C : e / N;
+      const int p = Lay::phys(i, c);
+      s[p] = cscale(s[p], fac[t.base + (size_t)i * t.ls + (size_t)c * t.cs]);
+    }
+    __syncthreads();
   }
 
   float d2 = 0.f, s2 = 0.f;
@@ -1154,7 +1165,7 @@ __global__ void __launch_bounds__(SThreads<N, MODE, NARROW>::v, SThreads<N, MODE
   }
 
   // ---- inverse transform along the line
-  if (MODE == S_INV || MODE == S_DELTA || MODE == S_ITER) {
+  if (MODE == S_INV || MODE == S_DELTA || MODE == S_ITER || MODE == S_FACTOR) {
 #pragma unroll
     for (int q = 0; q < (RED ? 2 : NS); ++q) Plan<N>::template run<C, T, true, Lay>(s + q * N * C, tw);
   }
@@ -1997,6 +2008,7 @@ struct MeshImpl {
     // plain passes: one component per CTA, components along gridDim.y
     if (mode == S_FWD && axis == AX_Y) return slaunch<S_FWD, 1, AX_Y>(a, st, nc);
     if (mode == S_INV && axis == AX_Y) return slaunch<S_INV, 1, AX_Y>(a, st, nc);
+    if (mode == S_FACTOR && axis == AX_Y && nc == 1) return slaunch<S_FACTOR, 1, AX_Y>(a, st, 1);
     if constexpr (kFusedMesh<N>) {
       // the vector x passes next to the register-fused k-space passes carry their representation
       if ((mode == S_FWD || mode == S_INV) && axis == AX_X && !a.generic && nc == 3)

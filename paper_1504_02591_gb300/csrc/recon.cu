@@ -224,6 +224,7 @@ struct recon_handle {
     int64_t start_launches[RECON_K_COUNT] = {}, body_launches[RECON_K_COUNT] = {};
     double start_bytes[RECON_K_COUNT] = {}, body_bytes[RECON_K_COUNT] = {};
   } gcache;
+  void* pin = nullptr;  // page-locked words the finite-difference solve reads its progress from
   uint64_t epoch = 0;   // incremented whenever the per-reconstruction parameters change
 };
 
@@ -872,6 +873,7 @@ recon_status recon_destroy(recon_handle* h) {
     cudaStreamSynchronize(h->st);
     cudaFree(h->ws);
   }
+  if (h->pin) cudaFreeHost(h->pin);
   delete h;
   return RECON_OK;
 }
@@ -1566,35 +1568,29 @@ recon_status recon_fft_c2r(recon_handle* h, const float* in_half, float* out_rea
 // ---- the finite-difference method of Sec. 2.1 (the paper's comparison method) ----------------
 namespace {
 
-// x . y in float64 over n values (one synchronisation).
-recon_status fd_dot(recon_handle* h, const float* x, const float* y, size_t n, double* out) {
-  const int blocks = kDepositBlocks;
-  RG_CUDA(timed(h, RECON_K_OTHER, 8.0 * n, [&] { return launch_dot(x, y, n, h->partials, blocks, h->st); }));
-  RG_TRY(finalize(h, blocks, 1, RED_DIAG, 0));
-  RG_CUDA(cudaMemcpyAsync(out, h->red + RED_DIAG, sizeof(double), cudaMemcpyDeviceToHost, h->st));
-  RG_CUDA(cudaStreamSynchronize(h->st));
+// f <- M^-1 f: the inverse of the periodic 7-point Laplacian through the library's FFT passes, in place;
+// the factor is applied inside the y pass, between its two transforms.
+recon_status fd_precond(recon_handle* h, Field f, const float* fac) {
+  ZArgs a = zargs(h);
+  a.f[0] = f;
+  RG_TRY(run_z(h, Z_FWD, 1, a));
+  RG_TRY(xpass(h, S_FWD, 1, &f));
+  SArgs s = sargs(h);
+  s.f[0] = f;
+  s.fac = fac;
+  RG_TRY(run_s(h, S_FACTOR, 1, AX_Y, s));
+  RG_TRY(xpass(h, S_INV, 1, &f));
+  RG_TRY(run_z(h, Z_INV, 1, a));
   return RECON_OK;
 }
 
-// out = M^-1 in: the inverse of the periodic 7-point Laplacian through the library's FFT passes on
-// the handle's first field.
-recon_status fd_precond(recon_handle* h, const float* in, float* out) {
-  const size_t nr = (size_t)h->n * h->n * h->n;
-  RG_CUDA(cudaMemcpyAsync(h->V[0].M, in, nr * sizeof(float), cudaMemcpyDeviceToDevice, h->st));
-  ZArgs a = zargs(h);
-  a.f[0] = h->V[0];
-  RG_TRY(run_z(h, Z_FWD, 1, a));
-  RG_TRY(xpass(h, S_FWD, 1, h->V));
-  SArgs s = sargs(h);
-  s.f[0] = h->V[0];
-  RG_TRY(run_s(h, S_FWD, 1, AX_Y, s));
-  RG_CUDA(timed(h, RECON_K_OTHER, 2.0 * cfield(h), [&] { return launch_fd_precond_k(h->V[0], h->n, h->L, h->st); }));
-  RG_TRY(run_s(h, S_INV, 1, AX_Y, s));
-  RG_TRY(xpass(h, S_INV, 1, h->V));
-  RG_TRY(run_z(h, Z_INV, 1, a));
-  RG_CUDA(cudaMemcpyAsync(out, h->V[0].M, nr * sizeof(float), cudaMemcpyDeviceToDevice, h->st));
-  return RECON_OK;
-}
+struct EventPair {
+  cudaEvent_t e[2] = {};
+  ~EventPair() {
+    for (cudaEvent_t v : e)
+      if (v) cudaEventDestroy(v);
+  }
+};
 
 struct DeviceBuffer {
   void* p = nullptr;
@@ -1608,15 +1604,20 @@ struct DeviceBuffer {
 recon_status recon_fd_solve(recon_handle* h, double tol, int max_iter, int* n_iter, double* rel_resid, float* psi_out) {
   if (!h || !psi_out || !(tol > 0) || max_iter < 1) return RECON_ERR_INVALID_ARG;
   if (h->state < ST_SMOOTHED || !h->delta_real_valid) return RECON_ERR_STATE;
-  const size_t nr = (size_t)h->n * h->n * h->n;
+  const size_t nr = (size_t)h->n * h->n * h->n, nfac = (size_t)h->n * h->n * (h->n / 2 + 1);
   DeviceBuffer buf;
-  if (cudaMalloc(&buf.p, 9 * nr * sizeof(float)) != cudaSuccess) {
+  if (cudaMalloc(&buf.p, (7 * nr + nfac) * sizeof(float) + sizeof(FDState) + 256) != cudaSuccess) {
     cudaGetLastError();
     return RECON_ERR_OOM;
   }
-  float* v0 = static_cast<float*>(buf.p);
-  float *x = v0, *r = v0 + nr, *rh = v0 + 2 * nr, *p = v0 + 3 * nr, *v = v0 + 4 * nr, *ph = v0 + 5 * nr,
-        *sv = v0 + 6 * nr, *sh = v0 + 7 * nr, *t = v0 + 8 * nr;
+  if (!h->pin) RG_CUDA(cudaMallocHost(&h->pin, 2 * sizeof(FDState)));
+  FDState* pin = static_cast<FDState*>(h->pin);
+  FDState* st = static_cast<FDState*>(buf.p);
+  float* v0 = reinterpret_cast<float*>(static_cast<char*>(buf.p) + align256(sizeof(FDState)));
+  float *x = v0, *r = v0 + nr, *rh = v0 + 2 * nr, *p = v0 + 3 * nr, *v = v0 + 4 * nr, *sv = v0 + 5 * nr, *t = v0 + 6 * nr,
+        *fac = v0 + 7 * nr;
+  // the preconditioned vectors, transformed in place (the densities they held are spent)
+  float *ph = reinterpret_cast<float*>(h->V[0].M), *sh = reinterpret_cast<float*>(h->V[1].M);
   FDArgs fa{};
   fa.n = h->n;
   fa.g = h->L / h->n;
@@ -1624,72 +1625,48 @@ recon_status recon_fd_solve(recon_handle* h, double tol, int max_iter, int* n_it
   fa.los_mode = h->p.los_mode;
   fa.los = make_double3(h->geo.los.x, h->geo.los.y, h->geo.los.z);
   fa.off = h->cur_off;
-  // right-hand side delta / b (the lognormal constant added back, as recon_get_field does)
-  RG_CUDA(cudaMemcpyAsync(rh, h->V[2].M, nr * sizeof(float), cudaMemcpyDeviceToDevice, h->st));
+  float c = 0.f;   // the lognormal constant added back, as recon_get_field does
   if (h->p.lognormal) {
     double sl = 0;
     RG_CUDA(cudaMemcpyAsync(&sl, h->red + RED_SUM_LOG, sizeof(double), cudaMemcpyDeviceToHost, h->st));
     RG_CUDA(cudaStreamSynchronize(h->st));
-    RG_CUDA(launch_add_scalar(rh, nr, (float)(-sl / (double)nr), h->st));
+    c = (float)(-sl / (double)nr);
   }
-  RG_CUDA(cudaMemsetAsync(x, 0, nr * sizeof(float), h->st));
-  RG_CUDA(launch_fd_sub(r, x, rh, -1.0 / h->p.b, nr, h->st));     // r = 0 + delta / b
-  RG_CUDA(cudaMemcpyAsync(rh, r, nr * sizeof(float), cudaMemcpyDeviceToDevice, h->st));
-  double bnorm2 = 0;
-  RG_TRY(fd_dot(h, r, r, nr, &bnorm2));
-  const double bnorm = std::sqrt(bnorm2);
-  double rho_old = 1.0, alpha = 1.0, omega = 1.0, res = bnorm > 0 ? 1.0 : 0.0;
-  int it = 0;
-  // BiCGStab, right-preconditioned (A M^-1 y = b, x = M^-1 y)
-  while (res > tol && it < max_iter) {
-    ++it;
-    double rho = 0;
-    RG_TRY(fd_dot(h, rh, r, nr, &rho));
-    if (it == 1) {
-      RG_CUDA(cudaMemcpyAsync(p, r, nr * sizeof(float), cudaMemcpyDeviceToDevice, h->st));
-    } else {
-      RG_CUDA(launch_fd_dir(p, r, v, (rho / rho_old) * (alpha / omega), omega, nr, h->st));
+  RG_CUDA(cudaMemsetAsync(st, 0, sizeof(FDState), h->st));
+  RG_CUDA(launch_fd_factor(fac, h->n, h->L, h->st));
+  RG_CUDA(launch_fd_init(reinterpret_cast<const float*>(h->V[2].M), c, 1.0 / h->p.b, x, r, rh, nr, st, tol, h->partials,
+                         h->st));   // r = delta / b
+  // BiCGStab, right-preconditioned (A M^-1 y = b, x = M^-1 y).  Its scalars stay on the device and its
+  // kernels end themselves, so the host only follows one iteration behind.
+  EventPair ev;
+  for (cudaEvent_t& e : ev.e) RG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  for (int k = 0; k < max_iter; ++k) {
+    RG_CUDA(timed(h, RECON_K_OTHER, 20.0 * nr, [&] { return launch_fd_dir(r, v, p, ph, nr, st, h->st); }));
+    RG_TRY(fd_precond(h, h->V[0], fac));
+    RG_CUDA(timed(h, RECON_K_OTHER, 12.0 * nr, [&] { return launch_fd_apply(0, ph, v, rh, fa, st, h->partials, h->st); }));
+    RG_CUDA(timed(h, RECON_K_OTHER, 16.0 * nr, [&] { return launch_fd_s(r, v, sv, sh, nr, st, h->partials, h->st); }));
+    RG_TRY(fd_precond(h, h->V[1], fac));
+    RG_CUDA(timed(h, RECON_K_OTHER, 12.0 * nr, [&] { return launch_fd_apply(1, sh, t, sv, fa, st, h->partials, h->st); }));
+    RG_CUDA(timed(h, RECON_K_OTHER, 32.0 * nr, [&] {
+      return launch_fd_update(x, ph, sh, sv, t, rh, r, nr, st, h->partials, h->st); }));
+    RG_CUDA(cudaMemcpyAsync(pin + (k & 1), st, sizeof(FDState), cudaMemcpyDeviceToHost, h->st));
+    RG_CUDA(cudaEventRecord(ev.e[k & 1], h->st));
+    if (k > 0) {
+      RG_CUDA(cudaEventSynchronize(ev.e[(k - 1) & 1]));
+      if (pin[(k - 1) & 1].done) break;
     }
-    RG_TRY(fd_precond(h, p, ph));
-    RG_CUDA(timed(h, RECON_K_OTHER, 8.0 * nr, [&] { return launch_fd_apply(ph, v, fa, h->st); }));
-    double rv = 0;
-    RG_TRY(fd_dot(h, rh, v, nr, &rv));
-    alpha = rho / rv;
-    RG_CUDA(launch_fd_sub(sv, r, v, alpha, nr, h->st));
-    double s2 = 0;
-    RG_TRY(fd_dot(h, sv, sv, nr, &s2));
-    if (std::sqrt(s2) / bnorm <= tol) {
-      RG_CUDA(launch_fd_acc(x, ph, ph, alpha, 0.0, nr, h->st));
-      res = std::sqrt(s2) / bnorm;
-      break;
-    }
-    RG_TRY(fd_precond(h, sv, sh));
-    RG_CUDA(timed(h, RECON_K_OTHER, 8.0 * nr, [&] { return launch_fd_apply(sh, t, fa, h->st); }));
-    double ts = 0, tt = 0;
-    RG_TRY(fd_dot(h, t, sv, nr, &ts));
-    RG_TRY(fd_dot(h, t, t, nr, &tt));
-    omega = tt > 0 ? ts / tt : 0.0;
-    RG_CUDA(launch_fd_acc(x, ph, sh, alpha, omega, nr, h->st));
-    RG_CUDA(launch_fd_sub(r, sv, t, omega, nr, h->st));
-    double r2 = 0;
-    RG_TRY(fd_dot(h, r, r, nr, &r2));
-    res = std::sqrt(r2) / bnorm;
-    if (!std::isfinite(res)) return RECON_ERR_NONFINITE;
-    rho_old = rho;
-    if (omega == 0.0) break;
   }
   // the true residual |A x - b| / |b| and Psi = -grad phi
-  RG_CUDA(launch_fd_apply(x, t, fa, h->st));
-  RG_CUDA(launch_fd_sub(t, t, rh, 1.0, nr, h->st));
-  double tr2 = 0;
-  RG_TRY(fd_dot(h, t, t, nr, &tr2));
+  RG_CUDA(launch_fd_apply(2, x, nullptr, rh, fa, st, h->partials, h->st));
   RG_CUDA(timed(h, RECON_K_OTHER, 16.0 * nr, [&] { return launch_fd_gradient(x, psi_out, fa, h->st); }));
+  RG_CUDA(cudaMemcpyAsync(pin, st, sizeof(FDState), cudaMemcpyDeviceToHost, h->st));
   RG_CUDA(cudaStreamSynchronize(h->st));
-  if (n_iter) *n_iter = it;
-  const double true_res = bnorm > 0 ? std::sqrt(tr2) / bnorm : 0.0;
-  if (rel_resid) *rel_resid = true_res;
-  h->delta_real_valid = 1;   // the real delta (third field) is untouched; only the first field was used
-  return res > tol ? RECON_ERR_NOT_CONVERGED : RECON_OK;
+  const FDState end = pin[0];
+  if (!std::isfinite(end.res)) return RECON_ERR_NONFINITE;
+  if (n_iter) *n_iter = end.it;
+  if (rel_resid) *rel_resid = end.true_res;
+  h->delta_real_valid = 1;   // the real delta (third field) is untouched; only the first two were used
+  return end.res > tol ? RECON_ERR_NOT_CONVERGED : RECON_OK;
 }
 
 // ---- the paper's front end (Sec. 3.2): radial number density and FKP weights ------------------

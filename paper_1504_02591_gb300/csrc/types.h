@@ -40,7 +40,7 @@ struct Geometry {
 };
 
 enum ZMode { Z_FWD = 0, Z_INV = 1, Z_DELTA = 2, Z_PROJ = 3, Z_FINAL = 4, Z_USTART = 5, Z_RADIAL = 6, Z_WARM = 7 };
-enum SMode { S_FWD = 0, S_INV = 1, S_DELTA = 3, S_ITER = 4 };
+enum SMode { S_FWD = 0, S_INV = 1, S_DELTA = 3, S_ITER = 4, S_FACTOR = 5 };   // S_FACTOR: forward, times fac, inverse
 enum Axis { AX_X = 0, AX_Y = 1 };
 
 struct ZArgs {
@@ -86,6 +86,7 @@ struct SArgs {
   Field f[3];             // fields transformed in place
   Geometry g;
   const float2* tab;      // stage twiddles of the N-point plan
+  const float* fac;       // S_FACTOR: real factor on the half grid, M [kx][ky][kz < N/2] then Q [kx][ky]
   const float2* tabx;     // x lines of the register-fused family: their second-stage twiddles (set at launch)
   double* partials;       // per-block partials (2 per block, S_ITER)
   const double* red;      // reduction block (S_DELTA reads the lognormal sum)
