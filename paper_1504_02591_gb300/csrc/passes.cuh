@@ -1650,24 +1650,39 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kit
 }
 
 // ---- the source update with its inputs streamed by the tensor memory accelerator ---------------
-// Persistent CTAs (two per SM) walk the Fourier-x/z tiles; a tile's four inputs (A, P_y, delta(k),
-// S_(n-1): four [512 y][4 kz] float2 boxes of a 3-D map over the half grid M [kx][ky][kz < N/2]) land
-// in one shared-memory stage by cp.async.bulk.tensor, completing on an mbarrier.  As soon as the
-// threads have copied the tile into their registers the next tile's copies are issued into the same
-// stage, so they stream in while this tile's transforms and stores run.  The Nyquist tiles (a
-// different layout, 1/257 of the data) follow with plain loads.  Each CTA's norms go to its
-// partials; the rest of the regular grid's partials are zeroed so the reduction over them is
-// unchanged.  Every wait is bounded: a wait that gives up writes NaN norms (the device loop then
-// stops with RECON_ERR_NONFINITE) and the CTA returns.
+// Persistent CTAs walk the Fourier-x/z tiles; a tile's four inputs (A, P_y, delta(k), S_(n-1): boxes
+// of a 3-D map over the half grid M [kx][ky][kz < N/2], at most 256 ky by the tile's kz) land in one
+// shared-memory stage by cp.async.bulk.tensor, completing on an mbarrier.  As soon as the threads have
+// copied the tile into their registers the next tile's copies are issued into the same stage, so they
+// stream in while this tile's transforms and stores run.  The Nyquist tiles (a different layout, 2/(N+2)
+// of the data) follow with plain loads.  Each CTA's norms go to its partials; the rest of the regular
+// grid's partials are zeroed so the reduction over them is unchanged.  Every wait is bounded: a wait that
+// gives up writes NaN norms (the device loop then stops with RECON_ERR_NONFINITE), waits once more for the
+// copies and the CTA returns.
+// The kernel with direct loads is bound by the L1's data pipe, most of its wavefronts the 32-byte
+// segments of its 4-column tiles' rows, and wider tiles leave it one CTA per SM with nothing to overlap.
+// Streaming takes the loads off that pipe and overlaps them within one CTA, so the tiles are 8 columns
+// (64-byte rows; 16 at 256: 106 us, 4 at 512: 1405 us); a 1024 line leaves room for 4.  Direct against
+// streamed, us per update kernel: 256 mesh 117 / 90, 384 487 / 331, 512 1028 / 645 (5.8 TB/s),
+// 1024 9300 / 7940.
+template <int N>
+struct TCols {
+  static constexpr int v = N < 1024 ? 8 : 4;
+};
+
 template <int N, int C>
 struct KTma {
   static constexpr int T = KFused<N, C>::T;
+  static constexpr int kBoxes = (N + 255) / 256;                      // boxes of a tile's field, at most 256 rows each
+  static constexpr int kRows = N / kBoxes;
+  static_assert(N % kBoxes == 0, "equal boxes");
   static constexpr size_t kS = sizeof(float2) * ((size_t)KFused<N, C>::TAB + 2 * (size_t)N * C);
   static constexpr size_t kBufOff = (kS + 127) & ~(size_t)127;
   static constexpr size_t kField = sizeof(float2) * (size_t)N * C;   // one field's tile
   static constexpr size_t kBarOff = kBufOff + 4 * kField;
   static constexpr size_t smem = kBarOff + 16;
   static constexpr uint32_t kTx = 4u * (uint32_t)kField;
+  static constexpr int kMinBlocks = smem <= 110 * 1024 ? 2 : 1;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -1693,12 +1708,32 @@ __device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Wait for a phase of the barrier, two seconds of the global timer at most.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+  if (bar_try_wait(bar, parity)) return true;
+  unsigned long long t0, t1;
+  asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t0));
+  do {
+    if (bar_try_wait(bar, parity)) return true;
+    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t1));
+  } while (t1 - t0 <= 2000000000ull);
+  return false;
+}
+
+// hi + lo += x, the rounding of hi kept in lo.
+__device__ __forceinline__ void two_add(float& hi, float& lo, float x) {
+  const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
+  hi = t;
+}
+
 template <int N, int C>
-__global__ void __launch_bounds__(KFused<N, C>::T, 2) kiter_tma_kernel(const SArgs a,
+__global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter_tma_kernel(const SArgs a,
                                                                        const __grid_constant__ KIterMaps maps) {
   using K = KTma<N, C>;
   constexpr int T = K::T, H = N / 2, MT = N * (H / C), QT = N / C;
-  constexpr int kGridPartials = MT + QT;   // the regular grid whose partials the reduction reads
+  constexpr int kDirect = SCols<N, S_ITER>::v;
+  constexpr int kGridPartials = N * (H / kDirect) + N / kDirect;   // the regular grid whose partials the reduction reads
   extern __shared__ __align__(128) float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
   float2* s = tw + KFused<N, C>::TAB;
@@ -1722,33 +1757,24 @@ __global__ void __launch_bounds__(KFused<N, C>::T, 2) kiter_tma_kernel(const SAr
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / 2)), &maps.m[q], c0, 256 * h, kx, bar);
+      for (int h = 0; h < K::kBoxes; ++h)
+        tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, K::kRows * h, kx, bar);
   };
-  float d2 = 0.f, s2 = 0.f;
+  float dh = 0.f, dl = 0.f, sh = 0.f, sl = 0.f;   // norms over the CTA's tiles, in pairs of float32
   float2 v[2][8], dk[8], sp[8];
   uint32_t parity = 0;
   if (threadIdx.x == 0 && (int)blockIdx.x < MT) issue(blockIdx.x);
   for (int tt = blockIdx.x; tt < MT; tt += gridDim.x) {
-    // bounded wait for the tile's copies: two seconds of the global timer at most
-    bool ok = bar_try_wait(bar, parity);
-    if (!ok) {
-      unsigned long long t0;
-      asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t0));
-      for (;;) {
-        if ((ok = bar_try_wait(bar, parity))) break;
-        unsigned long long t1;
-        asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t1));
-        if (t1 - t0 > 2000000000ull) break;
-      }
-    }
-    if (!ok) give_up = 1;
+    if (!bar_wait(bar, parity)) give_up = 1;
     __syncthreads();
-    if (give_up) break;
+    if (give_up) {
+      bar_wait(bar, parity);
+      break;
+    }
     parity ^= 1u;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const int e = (j + 64 * r) * C + col;
+      const int e = (j + KFused<N, C>::NB * r) * C + col;
       v[0][r] = buf[e];
       v[1][r] = buf[N * C + e];
       dk[r] = buf[2 * N * C + e];
@@ -1759,18 +1785,24 @@ __global__ void __launch_bounds__(KFused<N, C>::T, 2) kiter_tma_kernel(const SAr
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       issue(tt + gridDim.x);
     }
+    float d2 = 0.f, s2 = 0.f;
     kiter_tile<N, C>(a, tile_of<N, C, AX_Y>(tt), v, dk, sp, s, tw, j, col, d2, s2);
+    two_add(dh, dl, d2);
+    two_add(sh, sl, s2);
   }
   if (!give_up) {
     for (int q = blockIdx.x; q < QT; q += gridDim.x) {   // Nyquist tiles: plain loads
       const Tile t = tile_of<N, C, AX_Y>(MT + q);
       kiter_load<N, C>(a, t, j, col, v, dk, sp);
       __syncthreads();   // s may be rewritten
+      float d2 = 0.f, s2 = 0.f;
       kiter_tile<N, C>(a, t, v, dk, sp, s, tw, j, col, d2, s2);
+      two_add(dh, dl, d2);
+      two_add(sh, sl, s2);
     }
   }
-  double r0 = block_sum((double)d2, red_sh);
-  double r1 = block_sum((double)s2, red_sh);
+  double r0 = block_sum((double)dh + (double)dl, red_sh);
+  double r1 = block_sum((double)sh + (double)sl, red_sh);
   if (threadIdx.x == 0) {
     if (give_up) r0 = r1 = __longlong_as_double(0x7ff8000000000000ll);   // NaN: the loop stops
     a.partials[2 * blockIdx.x + 0] = r0;
@@ -1923,27 +1955,31 @@ struct MeshImpl {
                             st);
   }
 
-  static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
+  static int kmap_cols() {
+    if constexpr (kFusedMesh<N>) return TCols<N>::v;
+    return 0;
+  }
+  
+static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
     if constexpr (kFusedMesh<N>) {
       constexpr int C = SCols<N, S_ITER>::v;
-      if constexpr (N == 512) {
-        if (a.tmaps) {   // inputs streamed by TMA into persistent CTAs, two per SM
-          const void* k = (const void*)kiter_tma_kernel<N, C>;
-          static int grid = 0;
-          if (grid == 0) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KTma<N, C>::smem);
-            if (e != cudaSuccess) return e;
-            int dev = 0, sm = 0, occ = 0;
-            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-            if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, KTma<N, C>::T, KTma<N, C>::smem)) != cudaSuccess)
-              return e;
-            if (occ < 1) return cudaErrorInvalidConfiguration;
-            grid = occ * sm;
-          }
-          void* args[] = {const_cast<SArgs*>(&a), const_cast<KIterMaps*>(a.tmaps)};
-          return cudaLaunchKernel(k, dim3(grid), dim3(KTma<N, C>::T), args, KTma<N, C>::smem, st);
+      if (a.tmaps) {   // inputs streamed by TMA into persistent CTAs
+        constexpr int CT = TCols<N>::v;
+        using K = KTma<N, CT>;
+        const void* k = (const void*)kiter_tma_kernel<N, CT>;
+        static int grid = 0;
+        if (grid == 0) {
+          cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem);
+          if (e != cudaSuccess) return e;
+          int dev = 0, sm = 0, occ = 0;
+          if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+          if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+          if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, K::T, K::smem)) != cudaSuccess) return e;
+          if (occ < 1) return cudaErrorInvalidConfiguration;
+          grid = occ * sm;
         }
+        void* args[] = {const_cast<SArgs*>(&a), const_cast<KIterMaps*>(a.tmaps)};
+        return cudaLaunchKernel(k, dim3(grid), dim3(K::T), args, K::smem, st);
       }
       const void* k = (const void*)kiter_fused_kernel<N, C>;
       static bool attr = false;
@@ -2035,7 +2071,7 @@ struct MeshImpl {
   }
 
   static const MeshKernels* table() {
-    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0,
+    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0, kmap_cols(),
                                   &zpass, &spass, &build_tables};
     return &t;
   }

@@ -174,7 +174,7 @@ struct recon_handle {
   int kspace_generic = 0;
   int plane_batch = 0;   // register-fused path: y-planes per batch of the x -> z -> x passes (0: off)
   int assign = 0;        // mass assignment of the deposit: 0 CIC, 1 NGP (the paper's binning)
-  int kiter_tma = 0;     // N = 512 fused path: 1 streams the source update's inputs by TMA
+  int kiter_tma = 1;     // register-fused path: 1 streams the source update's inputs by TMA
   int radix_order = 0;   // FFT plans: 0 default, 1 the alternative order (mk is that order's table)
   bool tmaps_ok = false; // its tensor maps were built
   KIterMaps tmaps{};
@@ -350,7 +350,7 @@ bool encode_kiter_maps(recon_handle* h) {
   const Field* fs[4] = {&h->V[2], &h->V[1], &h->D, &h->S};
   const cuuint64_t dims[3] = {(cuuint64_t)n / 2, (cuuint64_t)n, (cuuint64_t)n};
   const cuuint64_t strides[2] = {(cuuint64_t)(n / 2) * 8, (cuuint64_t)n * (n / 2) * 8};
-  const cuuint32_t box[3] = {4, (cuuint32_t)(n / 2), 1};
+  const cuuint32_t box[3] = {(cuuint32_t)h->mk->kmap_cols, (cuuint32_t)(n / ((n + 255) / 256)), 1};
   const cuuint32_t es[3] = {1, 1, 1};
   for (int q = 0; q < 4; ++q) {
     if (((uintptr_t)fs[q]->M & 255) != 0) return false;
@@ -771,7 +771,7 @@ recon_status recon_create(const recon_params* p, void* stream, void* workspace, 
     rs = RECON_ERR_CUDA;
   }
   if (rs == RECON_OK) rs = configure(h, p);
-  if (rs == RECON_OK && n == 512) h->tmaps_ok = encode_kiter_maps(h);
+  if (rs == RECON_OK && h->mk->kmap_cols) h->tmaps_ok = encode_kiter_maps(h);
   if (rs != RECON_OK) {
     if (h->own_ws) cudaFree(h->ws);
     delete h;

@@ -77,7 +77,7 @@ struct ZArgs {
 };
 
 // Tensor maps of the register-fused source update's four inputs (A, P_y, delta(k), S) over the
-// half grid M [kx][ky][kz < N/2] (N = 512), built on the host; passed to the kernel by value.
+// half grid M [kx][ky][kz < N/2] of the meshes of the register-fused family, built on the host; passed to the kernel by value.
 struct KIterMaps {
   CUtensorMap m[4];
 };
@@ -101,7 +101,7 @@ struct SArgs {
   int generic;            // k-space update: the generic staged kernel instead of the register-fused one
   int ybeg, ycount;       // paired x passes: only the lines of y-planes [ybeg, ybeg + ycount)
                           // (ycount 0: every line; both multiples of the tile width)
-  const KIterMaps* tmaps; // host memory: the source update streams its inputs by TMA (N = 512)
+  const KIterMaps* tmaps; // host memory: the source update streams its inputs by TMA
   // paired inverse x pass (N = 512) unless loop_flag && *loop_flag == 1 (the device loop has just
   // converged): leave C = dx Psi_x + dy Psi_y in f[0] and Psi_z in wf for the projection pass,
   // instead of Psi_x, Psi_y, Psi_z in f[0..2]
@@ -138,6 +138,7 @@ struct MeshKernels {
   int tab_s, tab_z;       // stage-twiddle table lengths (N-point and N/2-point plans)
   int kspace_fused;       // register-fused passes with paired vector x passes (unless the generic option
                           // is set): 7 field transfers per y pass, 4 per x and z pass
+  int kmap_cols;          // columns of a tile of the TMA-streamed source update (0: none)
   // persistent Z pass; *grid_out receives the number of CTAs launched (its reduction partials)
   cudaError_t (*zpass)(int mode, int nc, const ZArgs& a, cudaStream_t st, int* grid_out);
   cudaError_t (*spass)(int mode, int nc, int axis, const SArgs& a, cudaStream_t st);
