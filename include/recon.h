@@ -331,7 +331,8 @@ enum {
                                    test; 0: the host reads the norms after every update.  Kernel
                                    timing (recon_set_timing) always uses the host-driven loop.   */
   RECON_OPT_LINE_TILE = 3,      /* FFT tile of the x-line passes: 0 (default) 16 adjacent columns
-                                   (128-byte rows) per tile, 1: 8 columns                         */
+                                   (128-byte rows) per tile, 1: 8 columns (the register-fused vector
+                                   passes of N = 256, 384 and 512 keep 16)                        */
   RECON_OPT_REUSE_SORT = 5,     /* 0 (default); 1: a recon_shift of the catalogue last given to
                                    recon_deposit (same pointer, n, dtype and memory kind, no
                                    pos_out) reuses the brick order the sorted deposit made of it
@@ -349,7 +350,7 @@ enum {
                                    0 one CTA per tile loading its inputs itself.  Same arithmetic per
                                    element (Psi bitwise equal); the norm sums are grouped differently,
                                    so the trace differs in float32 rounding.  Streamed against direct
-                                   at N = 512 on GB300: 0.65 against 1.03 ms per update.            */
+                                   at N = 512 on GB300: 0.61 against 1.03 ms per update.            */
   RECON_OPT_ASSIGN = 7,         /* mass assignment of recon_deposit: 0 (default) cloud-in-cell, 1 the
                                    paper's nearest grid point (Sec. 3: node floor(x N / L + 1/2)),
                                    always on the direct (unsorted) deposit kernel.  The shift still

@@ -1204,7 +1204,7 @@ constexpr size_t spass_smem(int nslots) {
 // stores and the update.
 // A thread owns the edge butterfly j = tid / C of column tid % C; the middle stage's 64 butterflies of
 // each line are dealt over the same threads (N = 384: 48 threads a column, 192 a CTA and three CTAs per
-// SM, 488 us an update against 533 with 64 threads a column and two).
+// SM, 8% faster than with 64 threads a column and two).
 // ------------------------------------------------------------------------------------------------
 template <int N, int C>
 struct KFused {
@@ -1230,52 +1230,64 @@ __device__ __forceinline__ int kline_mid(int j, int p) {
   return (j + TPC * p) & 63;
 }
 
-// The N-point transforms of K lines of one column (K = 2 in the update: A and P_y forward, G and
-// Psi_y inverse; K = 1 for delta), stage by stage together (one buffer each, so a stage needs one
-// barrier for all K): v[q][r] = x_q[j + (N/8) r] in, X_q[j + (N/8) r] out.
-template <bool INV, int N, int C, int K>
+// The transform as a cube (a, b, k) of 8 x M x 8 points: stage 1's butterfly j = a + 8 b turns the 8 points
+// of a thread into k, stage 2's (a, k) turns b into c, stage 3's j = k + 8 c turns a into the output.  Every
+// stage works in place, so a transform takes two barriers, and stage 3 leaves thread j reading exactly the
+// places that the next transform's stage 1 may write when a and k swap places (ROLE 1): back-to-back
+// transforms need no barrier between them.  Point (a, b, k) of a column: rows along z, x's low bits folded
+// in so that neighbours along either fall in distinct banks.
+template <int N, int C, int ROLE>
+__device__ __forceinline__ int kcube(int a, int b, int k, int col) {
+  const int x = ROLE ? k : a, z = ROLE ? a : k;
+  return (8 * (b + KFused<N, C>::M * x) + (z ^ (x & ColLayout<C>::kMask))) * C + col;
+}
+
+struct NoHook {
+  __device__ __forceinline__ void operator()() const {}
+};
+
+// The N-point transforms of K lines of one column (the update: K = 2, A and P_y forward, G and Psi_y
+// inverse; the vector x passes and delta: K = 1), stage by stage together (one buffer each, so a stage
+// needs one barrier for all K): v[q][r] = x_q[j + (N/8) r] in, X_q[j + (N/8) r] out.  The places that stage 1
+// writes must be free: a barrier since the last transform, or that one by the same lines in the other ROLE.
+// Two barriers instead of the five of a transform that re-sorts between stages and frees its buffers: the
+// streamed update 256 90 -> 88 us, 384 318 -> 282, 512 644 -> 611, 1024 8080 -> 6960.
+template <bool INV, int N, int C, int K, int ROLE = 0, class Hook = NoHook>
 __device__ __forceinline__ void kline_fft(float2 (&v)[K][8], float2* __restrict__ s, const float2* __restrict__ tw,
-                                          int j, int col) {
+                                          int j, int col, Hook&& hook = Hook()) {
   using F = KFused<N, C>;
-  using Lay = ColLayout<C>;
   constexpr int B = N * C, M = F::M, PM = (64 * K + F::TPC - 1) / F::TPC;
 #pragma unroll
   for (int q = 0; q < K; ++q) {                            // stage 1 (NS = 1): no twiddles
     Dft<8, INV>::run(v[q]);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) s[q * B + Lay::phys(8 * j + r, col)] = v[q][r];
+    for (int r = 0; r < 8; ++r) s[q * B + kcube<N, C, ROLE>(j & 7, j >> 3, r, col)] = v[q][r];
   }
   __syncthreads();
-  float2 u[PM][M];                                         // stage 2 (NS = 8): items (line, butterfly)
+  hook();
 #pragma unroll
-  for (int p = 0; p < PM; ++p) {
+  for (int p = 0; p < PM; ++p) {                           // stage 2 (NS = 8): items (line, butterfly)
     if ((64 * K) % F::TPC == 0 || j + F::TPC * p < 64 * K) {
       const int q = kline_item<F::TPC>(j, p), jm = kline_mid<F::TPC>(j, p), k = jm & 7;
+      float2 u[M];
 #pragma unroll
-      for (int r = 0; r < M; ++r) u[p][r] = s[q * B + Lay::phys(jm + 64 * r, col)];
+      for (int r = 0; r < M; ++r) u[r] = s[q * B + kcube<N, C, ROLE>(jm >> 3, r, k, col)];
 #pragma unroll
       for (int r = 1; r < M; ++r) {
         float2 w = tw[(r - 1) * 8 + k];
         if (INV) w.y = -w.y;
-        u[p][r] = cmul(u[p][r], w);
+        u[r] = cmul(u[r], w);
       }
-      Dft<M, INV>::run(u[p]);
-    }
-  }
-  __syncthreads();
+      Dft<M, INV>::run(u);
 #pragma unroll
-  for (int p = 0; p < PM; ++p) {
-    if ((64 * K) % F::TPC == 0 || j + F::TPC * p < 64 * K) {
-      const int q = kline_item<F::TPC>(j, p), jm = kline_mid<F::TPC>(j, p), base = (jm >> 3) * (8 * M) + (jm & 7);
-#pragma unroll
-      for (int r = 0; r < M; ++r) s[q * B + Lay::phys(base + 8 * r, col)] = u[p][r];
+      for (int r = 0; r < M; ++r) s[q * B + kcube<N, C, ROLE>(jm >> 3, r, k, col)] = u[r];
     }
   }
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < K; ++q) {                            // stage 3 (NS = N/8)
 #pragma unroll
-    for (int r = 0; r < 8; ++r) v[q][r] = s[q * B + Lay::phys(j + F::NB * r, col)];
+    for (int r = 0; r < 8; ++r) v[q][r] = s[q * B + kcube<N, C, ROLE>(r, j >> 3, j & 7, col)];
 #pragma unroll
     for (int r = 1; r < 8; ++r) {
       float2 w = tw[F::OFF3 + (r - 1) * F::NB + j];
@@ -1284,7 +1296,13 @@ __device__ __forceinline__ void kline_fft(float2 (&v)[K][8], float2* __restrict_
     }
     Dft<8, INV>::run(v[q]);
   }
-  __syncthreads();                                         // the buffers are reused
+}
+
+// Signed frequency of the point j + (N/8) r of a line, r known when compiled; exact, so kf times it is what
+// kf times the integer is.
+template <int N>
+__device__ __forceinline__ float line_freq(float fj, int r) {
+  return fj + (float)(r < 4 ? (N / 8) * r : (N / 8) * r - N);
 }
 
 // The start's k-space pass along y (S_DELTA): the y transform of delta (unless delta(k)
@@ -1317,10 +1335,9 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kde
     int ix, kz;
     if (!t.isQ) { ix = t.a; kz = t.c0 + col; } else { ix = t.c0 + col; kz = H; }
     const int mx = (ix < H) ? ix : ix - N;
-    const int my = (ky < H) ? ky : ky - N;
-    const float kx = g.kf * mx, kyf = g.kf * my, kzf = g.kf * kz;
+    const float kx = g.kf * mx, kyf = g.kf * line_freq<N>((float)j, r), kzf = g.kf * kz;
     const float k2 = kx * kx + kyf * kyf + kzf * kzf;
-    const float kdy = (ky == H) ? 0.f : kyf;
+    const float kdy = (r == 4 && j == 0) ? 0.f : kyf;
     const size_t gi = t.base + (size_t)ky * t.ls + (size_t)col * t.cs;
     float2 dk = d[0][r];
     if (!a.d_is_k) {
@@ -1335,7 +1352,7 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kde
     v[0][r] = iS;
     v[1][r] = cscale(iS, kdy);
   }
-  kline_fft<true, N, C, 2>(v, s, tw, j, col);
+  kline_fft<true, N, C, 2, 1>(v, s, tw, j, col);
   // G (Psi_x = kdx G, Psi_z = kdz G) in the third field, Psi_y in the second, as the update
   // kernel leaves them
   float2* __restrict__ dy = t.isQ ? a.f[1].Q : a.f[1].M;
@@ -1412,7 +1429,7 @@ __device__ __forceinline__ void xline_io(float2* __restrict__ s, const float2* _
   }
 }
 
-// PAIR = false: one component per CTA (blockIdx.y).  PAIR = true: the vector passes between the
+// PAIR = false: one component per CTA (blockIdx.y).  PAIR = true (1024): the vector passes between the
 // register-fused k-space pass (y) and the fused z pass, which carry vectors in reduced forms: kx and
 // kz (kdx, kdz: zero at the Nyquist index) are constant along a y line, so the y pass needs
 // A = kdx P_x + kdz P_z and P_y and returns G (Psi_x = kdx G, Psi_z = kdz G) and Psi_y; and the
@@ -1578,10 +1595,9 @@ __device__ __forceinline__ void kiter_tile(const SArgs& a, const Tile& t, float2
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const int ky = j + NB * r;
-    const int my = (ky < H) ? ky : ky - N;
-    const float kyf = g.kf * my;
+    const float kyf = g.kf * line_freq<N>((float)j, r);
     const float k2 = kxz2 + kyf * kyf;
-    const float kdy = (ky == H) ? 0.f : kyf;
+    const float kdy = (r == 4 && j == 0) ? 0.f : kyf;
     const float2 pa = v[0][r], py = v[1][r];
     const float dre = fmaf(kdy, py.x, pa.x);
     const float dim = fmaf(kdy, py.y, pa.y);
@@ -1597,7 +1613,7 @@ __device__ __forceinline__ void kiter_tile(const SArgs& a, const Tile& t, float2
     v[0][r] = iS;
     v[1][r] = cscale(iS, kdy);
   }
-  kline_fft<true, N, C, 2>(v, s, tw, j, col);
+  kline_fft<true, N, C, 2, 1>(v, s, tw, j, col);
   float2* __restrict__ dy = t.isQ ? a.f[1].Q : a.f[1].M;
   float2* __restrict__ dg = t.isQ ? a.f[2].Q : a.f[2].M;
 #pragma unroll
@@ -1663,8 +1679,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kit
 // segments of its 4-column tiles' rows, and wider tiles leave it one CTA per SM with nothing to overlap.
 // Streaming takes the loads off that pipe and overlaps them within one CTA, so the tiles are 8 columns
 // (64-byte rows; 16 at 256: 106 us, 4 at 512: 1405 us); a 1024 line leaves room for 4.  Direct against
-// streamed, us per update kernel: 256 mesh 117 / 90, 384 487 / 331, 512 1028 / 645 (5.8 TB/s),
-// 1024 9300 / 7940.
+// streamed, us per update kernel: 256 mesh 114 / 88, 384 457 / 282, 512 1026 / 611 (6.1 TB/s, 0.9 of the
+// copy rate), 1024 10460 / 6960.
 template <int N>
 struct TCols {
   static constexpr int v = N < 1024 ? 8 : 4;
@@ -1740,11 +1756,10 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
   const float2* buf = reinterpret_cast<const float2*>(reinterpret_cast<char*>(ssm) + K::kBufOff);
   uint64_t* bar_p = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ssm) + K::kBarOff);
   __shared__ double red_sh[T / 32];
-  __shared__ int give_up;
+  bool give_up = false;
   const uint32_t bar = smem_addr(bar_p), dst = smem_addr(buf);
   for (int m = threadIdx.x; m < Plan<N>::kTab; m += T) tw[m] = a.tab[m];
   if (threadIdx.x == 0) {
-    give_up = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -1765,12 +1780,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
   uint32_t parity = 0;
   if (threadIdx.x == 0 && (int)blockIdx.x < MT) issue(blockIdx.x);
   for (int tt = blockIdx.x; tt < MT; tt += gridDim.x) {
-    if (!bar_wait(bar, parity)) give_up = 1;
-    __syncthreads();
-    if (give_up) {
-      bar_wait(bar, parity);
-      break;
-    }
+    const bool ok = bar_wait(bar, parity);
+    if (!ok) bar_wait(bar, parity);
     parity ^= 1u;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -1780,7 +1791,11 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
       dk[r] = buf[2 * N * C + e];
       sp[r] = buf[3 * N * C + e];
     }
-    __syncthreads();   // the stage is free (and s may be rewritten)
+    // the stage is free, and so is s
+    if (__syncthreads_or(!ok)) {
+      give_up = true;
+      break;
+    }
     if (threadIdx.x == 0 && tt + (int)gridDim.x < MT) {
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       issue(tt + gridDim.x);
@@ -1794,7 +1809,6 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
     for (int q = blockIdx.x; q < QT; q += gridDim.x) {   // Nyquist tiles: plain loads
       const Tile t = tile_of<N, C, AX_Y>(MT + q);
       kiter_load<N, C>(a, t, j, col, v, dk, sp);
-      __syncthreads();   // s may be rewritten
       float d2 = 0.f, s2 = 0.f;
       kiter_tile<N, C>(a, t, v, dk, sp, s, tw, j, col, d2, s2);
       two_add(dh, dl, d2);
@@ -1811,6 +1825,165 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
   for (int b = blockIdx.x + gridDim.x + threadIdx.x * gridDim.x; b < kGridPartials; b += T * gridDim.x) {
     a.partials[2 * b + 0] = 0.0;
     a.partials[2 * b + 1] = 0.0;
+  }
+}
+
+// ---- the vector x passes, streamed (256, 384 and 512) ---------------------------------------------
+// Three transforms of two fields a tile, in the representations that xline_kernel describes:
+//   inverse: IFFT_x(kdx G), IFFT_x(G) and IFFT_x(Psi_y) of the third and second fields, left as C and Psi_z
+//            in the first and fourth (C form) or as Psi_x, Psi_y and Psi_z in the first three;
+//   forward: FFT_x(dx psi^), FFT_x(psi^) and FFT_x(Z^) of the first and third fields, left as P_y in the second
+//            and A in the third.
+// Streamed as the source update above is: persistent CTAs whose next tile's fields (boxes of [x][1 y][kz])
+// arrive while this tile is transformed, the Nyquist tiles (and every tile where the maps could not be
+// built) by plain loads.  The lines go through one exchange buffer one after the other and a thread holds
+// 16 points at most, so one or two CTAs fill the SM's threads; each field's stage is refilled as soon as its
+// last reader has passed a barrier.  A wait that gives up leaves NaN in its tile (the norms, and the loop's
+// outcome, then are NaN too).
+// The pass is bound by the reads and writes at a stride of a whole plane, each 2 MB page giving a tile one or
+// two rows: 16 columns (128-byte rows) against 8 (64 bytes), inverse / forward us, 512 450 / 444 against
+// 563 / 537, 384 194 / 192 against 195 / 191, 256 61 / 59 against 62 / 61.  The kernel that one tile's two
+// CTAs ran with loads to registers (xline_kernel's pairs) took 585 / 573, 227 / 230 and 68 / 70.  A 1024
+// line leaves room for 8 columns (6790 / 6580 us; 4 of all three lines at once 12700 / 12300), so that mesh
+// keeps the pairs at 16 (5570 / 5580).
+template <int N>
+constexpr bool kVLine = kFusedMesh<N> && N < 1024;
+constexpr int kVCols = 16;
+
+template <int N, int C>
+struct VLine {
+  static constexpr int T = KFused<N, C>::T;
+  static constexpr int kBoxes = KTma<N, C>::kBoxes, kRows = KTma<N, C>::kRows;
+  static constexpr size_t kField = sizeof(float2) * (size_t)N * C;
+  static constexpr size_t kBufOff = (sizeof(float2) * (size_t)KFused<N, C>::TAB + kField + 127) & ~(size_t)127;
+  static constexpr size_t kBarOff = kBufOff + 2 * kField;
+  static constexpr size_t kDxOff = kBarOff + 16;
+  static constexpr size_t smem = kDxOff + sizeof(float) * (size_t)N;
+  static constexpr int kMinBlocks = T <= 512 ? 2 : 1;   // what shared memory holds
+};
+
+template <bool INV, int N, int C>
+__global__ void __launch_bounds__(KFused<N, C>::T, VLine<N, C>::kMinBlocks) vline_kernel(const SArgs a,
+                                                                                         const __grid_constant__ VLineMaps maps) {
+  using K = VLine<N, C>;
+  constexpr int T = K::T, H = N / 2, NB = KFused<N, C>::NB;
+  extern __shared__ __align__(128) float4 ssm[];
+  float2* tw = reinterpret_cast<float2*>(ssm);
+  float2* s = tw + KFused<N, C>::TAB;
+  const float2* buf = reinterpret_cast<const float2*>(reinterpret_cast<char*>(ssm) + K::kBufOff);
+  float* dxs = reinterpret_cast<float*>(reinterpret_cast<char*>(ssm) + K::kDxOff);   // dx of the line's points
+  __shared__ int give_up;
+  if (!INV && a.skip_flag && *a.skip_flag != 0) return;   // uniform: device loop already converged
+  const uint32_t bar = smem_addr(reinterpret_cast<char*>(ssm) + K::kBarOff), dst = smem_addr(buf);
+  for (int m = threadIdx.x; m < Plan<N>::kTab; m += T) tw[m] = a.tab[m];
+  for (int m = threadIdx.x; m < N; m += T) dxs[m] = a.g.los_mode == 1 ? a.g.los.x : a.g.off[m];
+  if (threadIdx.x == 0) {
+    give_up = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar + 8) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  }
+  __syncthreads();
+  // tiles of every y-plane, or of the planes [ybeg, ybeg + ycount): their M tiles (ky, kz block), then
+  // the Nyquist tiles that hold their ky columns
+  const int ny = a.ycount ? a.ycount : N, mt = ny * (H / C), tiles = mt + ny / C, streamed = maps.on ? mt : 0;
+  auto tile_id = [&](int tt) { return tt < mt ? a.ybeg * (H / C) + tt : N * (H / C) + a.ybeg / C + (tt - mt); };
+  const int col = threadIdx.x % C, j = threadIdx.x / C;
+  auto issue = [&](int q, int tt) {   // thread 0: field q's boxes of tile tt
+    if (threadIdx.x != 0 || tt >= streamed) return;
+    const int ti = tile_id(tt), ky = ti / (H / C), c0 = (ti % (H / C)) * C;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar + 8 * q), "r"((uint32_t)K::kField) : "memory");
+#pragma unroll
+    for (int h = 0; h < K::kBoxes; ++h)
+      tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, ky, K::kRows * h, bar + 8 * q);
+  };
+  const Geometry& g = a.g;
+  const bool cf = INV && a.cform && !(a.loop_flag && *a.loop_flag == 1);
+  // the line index is kx in Fourier space and x in configuration space
+  const float fj = (float)j;
+  auto kdx = [&](int r) { return r == 4 && j == 0 ? 0.f : g.kf * line_freq<N>(fj, r); };
+  auto dxv = [&](int r) { return dxs[j + NB * r]; };
+  uint32_t parity = 0;
+  issue(0, blockIdx.x);
+  issue(1, blockIdx.x);
+  for (int tt = blockIdx.x; tt < tiles; tt += gridDim.x) {
+    const int next = tt + gridDim.x;
+    const Tile t = tile_of<N, C, AX_X>(tile_id(tt));
+    // element offsets fit 32 bits (at most N^3 / 2 complex points per field)
+    const uint32_t o0 = (uint32_t)t.base + (uint32_t)(col * t.cs) + (uint32_t)j * (uint32_t)t.ls;
+    const uint32_t step = (uint32_t)NB * (uint32_t)t.ls;
+    auto at = [&](int f) { return t.isQ ? a.f[f].Q : a.f[f].M; };
+    auto wait = [&](int q) {
+      if (tt >= streamed || bar_wait(bar + 8 * q, parity)) return true;
+      give_up = 1;
+      bar_wait(bar + 8 * q, parity);
+      return false;
+    };
+    auto load = [&](int q, int f, bool ok, float2 (&x)[8]) {   // the stage's field q, which is field f
+      if (tt < streamed) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) x[r] = buf[q * N * C + (j + NB * r) * C + col];
+      } else {
+        const float2* __restrict__ p = at(f);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) x[r] = p[o0 + r * step];
+      }
+      if (!ok) x[0].x = __int_as_float(0x7fc00000);
+    };
+    const float dy = g.los_mode == 1 ? g.los.y : g.off[N + (t.isQ ? t.c0 + col : t.a)];
+    const float kdz = t.isQ ? 0.f : g.kf * (float)(t.c0 + col);   // M tiles: kz < N/2; Q tiles: kz = N/2
+    float2 v[1][8], w[8];
+    // the first field twice (kdx G, G; dx psi^, psi^), the second once (Psi_y; Z^)
+    constexpr int F0 = INV ? 2 : 0, F1 = INV ? 1 : 2;
+    bool ok = wait(0);
+    load(0, F0, ok, v[0]);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[0][r] = cscale(v[0][r], INV ? kdx(r) : dxv(r));
+    kline_fft<INV, N, C, 1, 0>(v, s, tw, j, col);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) w[r] = v[0][r];
+    load(0, F0, ok, v[0]);
+    kline_fft<INV, N, C, 1, 1>(v, s, tw, j, col, [&] { issue(0, next); });
+    {
+      float2* __restrict__ P = !INV ? at(1) : (cf ? (t.isQ ? a.wf.Q : a.wf.M) : at(2));
+      const float sc = INV ? kdz : dy;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) P[o0 + r * step] = cscale(v[0][r], sc);
+    }
+    ok = wait(1);
+    load(1, F1, ok, v[0]);
+    int stop = 0;
+    kline_fft<INV, N, C, 1, 0>(v, s, tw, j, col, [&] {
+      stop = give_up;   // no wait between this barrier and the next
+      issue(1, next);
+    });
+    float2* __restrict__ P0 = at(INV ? 0 : 2);
+    if (cf) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float d = dxv(r);
+        P0[o0 + r * step] = make_float2(fmaf(d, w[r].x, dy * v[0][r].x), fmaf(d, w[r].y, dy * v[0][r].y));
+      }
+    } else if (INV) {
+      float2* __restrict__ P1 = at(1);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        P0[o0 + r * step] = w[r];
+        P1[o0 + r * step] = v[0][r];
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float k = kdx(r);
+        const float2 x = cscale(v[0][r], kdz);
+        P0[o0 + r * step] = make_float2(fmaf(k, w[r].x, x.x), fmaf(k, w[r].y, x.y));
+      }
+    }
+    if (stop) break;
+    if (tt < streamed) parity ^= 1u;
+    __syncthreads();   // s is free
   }
 }
 
@@ -1831,6 +2004,19 @@ __global__ void build_tables_kernel(const float2* __restrict__ tw, float2* tabS,
 // ------------------------------------------------------------------------------------------------
 // Launch tables
 // ------------------------------------------------------------------------------------------------
+// CTAs of a persistent kernel: as many as the device holds at once.
+static inline cudaError_t persistent_grid(const void* k, int threads, size_t smem, int* grid) {
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sm = 0, occ = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, threads, smem)) != cudaSuccess) return e;
+  if (occ < 1) return cudaErrorInvalidConfiguration;
+  *grid = occ * sm;
+  return cudaSuccess;
+}
+
 template <class K>
 static cudaError_t launch_with_smem(K kern, int blocks, int threads, size_t smem, cudaStream_t st, const void* arg) {
   static_assert(sizeof(K) > 0, "");
@@ -1955,6 +2141,10 @@ struct MeshImpl {
                             st);
   }
 
+  static int vmap_cols() {
+    if constexpr (kVLine<N>) return kVCols;
+    return 0;
+  }
   static int kmap_cols() {
     if constexpr (kFusedMesh<N>) return TCols<N>::v;
     return 0;
@@ -1969,14 +2159,8 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
         const void* k = (const void*)kiter_tma_kernel<N, CT>;
         static int grid = 0;
         if (grid == 0) {
-          cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem);
+          const cudaError_t e = persistent_grid(k, K::T, K::smem, &grid);
           if (e != cudaSuccess) return e;
-          int dev = 0, sm = 0, occ = 0;
-          if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-          if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-          if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, K::T, K::smem)) != cudaSuccess) return e;
-          if (occ < 1) return cudaErrorInvalidConfiguration;
-          grid = occ * sm;
         }
         void* args[] = {const_cast<SArgs*>(&a), const_cast<KIterMaps*>(a.tmaps)};
         return cudaLaunchKernel(k, dim3(grid), dim3(K::T), args, K::smem, st);
@@ -2033,8 +2217,30 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
   }
   static cudaError_t xlaunch(bool inv, const SArgs& a, cudaStream_t st, int ncomp, bool pair) {
     if constexpr (kFusedMesh<N>) {
-      if (pair) return a.narrow ? xlaunch_c<8, true>(inv, a, st, ncomp) : xlaunch_c<16, true>(inv, a, st, ncomp);
+      if constexpr (!kVLine<N>)
+        if (pair) return a.narrow ? xlaunch_c<8, true>(inv, a, st, ncomp) : xlaunch_c<16, true>(inv, a, st, ncomp);
       return xlaunch_c<16, false>(inv, a, st, ncomp);
+    }
+    return cudaErrorInvalidValue;
+  }
+
+  // the vector x passes: persistent CTAs over the tiles of all y-planes or of a batch of them
+  template <bool INV>
+  static cudaError_t vlaunch(const SArgs& a, cudaStream_t st) {
+    if constexpr (kVLine<N>) {
+      constexpr int C = kVCols;
+      using K = VLine<N, C>;
+      if (a.ycount && (a.ycount % C || a.ybeg % C || a.ybeg < 0 || a.ybeg + a.ycount > N)) return cudaErrorInvalidValue;
+      const void* k = (const void*)vline_kernel<INV, N, C>;
+      static int grid = 0;
+      if (grid == 0) {
+        const cudaError_t e = persistent_grid(k, K::T, K::smem, &grid);
+        if (e != cudaSuccess) return e;
+      }
+      VLineMaps none{};
+      const int ny = a.ycount ? a.ycount : N, tiles = ny * ((N / 2) / C) + ny / C;
+      void* args[] = {const_cast<SArgs*>(&a), a.vmaps ? const_cast<VLineMaps*>(&a.vmaps[INV]) : &none};
+      return cudaLaunchKernel(k, dim3(tiles < grid ? tiles : grid), dim3(K::T), args, K::smem, st);
     }
     return cudaErrorInvalidValue;
   }
@@ -2047,8 +2253,10 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
     if (mode == S_FACTOR && axis == AX_Y && nc == 1) return slaunch<S_FACTOR, 1, AX_Y>(a, st, 1);
     if constexpr (kFusedMesh<N>) {
       // the vector x passes next to the register-fused k-space passes carry their representation
-      if ((mode == S_FWD || mode == S_INV) && axis == AX_X && !a.generic && nc == 3)
+      if ((mode == S_FWD || mode == S_INV) && axis == AX_X && !a.generic && nc == 3) {
+        if constexpr (kVLine<N>) return mode == S_INV ? vlaunch<true>(a, st) : vlaunch<false>(a, st);
         return xlaunch(mode == S_INV, a, st, nc, true);
+      }
       if ((mode == S_FWD || mode == S_INV) && axis == AX_X && !a.narrow && !a.generic)
         return xlaunch(mode == S_INV, a, st, nc, false);
     }
@@ -2071,7 +2279,7 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
   }
 
   static const MeshKernels* table() {
-    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0, kmap_cols(),
+    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0, kmap_cols(), vmap_cols(),
                                   &zpass, &spass, &build_tables};
     return &t;
   }

@@ -176,8 +176,9 @@ struct recon_handle {
   int assign = 0;        // mass assignment of the deposit: 0 CIC, 1 NGP (the paper's binning)
   int kiter_tma = 1;     // register-fused path: 1 streams the source update's inputs by TMA
   int radix_order = 0;   // FFT plans: 0 default, 1 the alternative order (mk is that order's table)
-  bool tmaps_ok = false; // its tensor maps were built
+  bool tmaps_ok = false; // the tensor maps were built
   KIterMaps tmaps{};
+  VLineMaps vmaps[2]{};  // forward and inverse
   int reuse_sort = 0;
   // the catalogue whose brick order the sort buffers hold (sorted deposit, one chunk)
   struct SortMemo {
@@ -326,15 +327,16 @@ SArgs sargs(recon_handle* h) {
   a.generic = h->kspace_generic;
   a.lognormal = h->p.lognormal;
   a.tmaps = (h->tmaps_ok && h->kiter_tma) ? &h->tmaps : nullptr;
+  a.vmaps = h->tmaps_ok ? h->vmaps : nullptr;
   a.wf = h->W;
   return a;
 }
 
-// Tensor maps of the fused source update's inputs (A in the third field, P_y in the second,
-// delta(k), S) over the half grid M [kx][ky][kz < N/2], float2 elements copied as 8-byte words: boxes
-// of 4 kz x 256 ky x 1 kx (a tile's y line is two boxes).  Needs the driver's encoder; without it the
-// update loads its inputs directly.
-bool encode_kiter_maps(recon_handle* h) {
+// Tensor maps of the register-fused kernels' inputs, float2 elements copied as 8-byte words, over
+// the half grid M [kx][ky][kz < N/2]: boxes of the tiles' kz by at most 256 ky (the source update: A in
+// the third field, P_y in the second, delta(k), S) or by at most 256 x (the vector x passes; a tile's line
+// is one to four boxes).  Needs the driver's encoder; without it the kernels load their inputs directly.
+bool encode_maps(recon_handle* h) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     void* fn = nullptr;
@@ -346,18 +348,25 @@ bool encode_kiter_maps(recon_handle* h) {
     }
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  const int n = h->n;
+  const cuuint64_t n = (cuuint64_t)h->n;
+  const cuuint32_t rows = (cuuint32_t)(n / ((n + 255) / 256));
+  auto map = [&](CUtensorMap* m, const Field& f, bool along_x) {
+    const cuuint64_t dims[3] = {n / 2, n, n}, strides[2] = {n / 2 * 8, n * (n / 2) * 8};
+    const cuuint32_t cols = (cuuint32_t)(along_x ? h->mk->vmap_cols : h->mk->kmap_cols);
+    const cuuint32_t box[3] = {cols, along_x ? 1u : rows, along_x ? rows : 1u}, es[3] = {1, 1, 1};
+    return ((uintptr_t)f.M & 255) == 0 &&
+           encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)f.M, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
   const Field* fs[4] = {&h->V[2], &h->V[1], &h->D, &h->S};
-  const cuuint64_t dims[3] = {(cuuint64_t)n / 2, (cuuint64_t)n, (cuuint64_t)n};
-  const cuuint64_t strides[2] = {(cuuint64_t)(n / 2) * 8, (cuuint64_t)n * (n / 2) * 8};
-  const cuuint32_t box[3] = {(cuuint32_t)h->mk->kmap_cols, (cuuint32_t)(n / ((n + 255) / 256)), 1};
-  const cuuint32_t es[3] = {1, 1, 1};
-  for (int q = 0; q < 4; ++q) {
-    if (((uintptr_t)fs[q]->M & 255) != 0) return false;
-    const CUresult r = encode(&h->tmaps.m[q], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)fs[q]->M, dims, strides, box, es,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return false;
+  for (int q = 0; q < 4; ++q)
+    if (!map(&h->tmaps.m[q], *fs[q], false)) return false;
+  const int vf[2][2] = {{0, 2}, {2, 1}};   // forward, inverse
+  for (int inv = 0; inv < 2 && h->mk->vmap_cols; ++inv) {
+    for (int q = 0; q < 2; ++q)
+      if (!map(&h->vmaps[inv].m[q], h->V[vf[inv][q]], true)) return false;
+    h->vmaps[inv].on = 1;
   }
   return true;
 }
@@ -771,7 +780,7 @@ recon_status recon_create(const recon_params* p, void* stream, void* workspace, 
     rs = RECON_ERR_CUDA;
   }
   if (rs == RECON_OK) rs = configure(h, p);
-  if (rs == RECON_OK && h->mk->kmap_cols) h->tmaps_ok = encode_kiter_maps(h);
+  if (rs == RECON_OK && h->mk->kmap_cols) h->tmaps_ok = encode_maps(h);
   if (rs != RECON_OK) {
     if (h->own_ws) cudaFree(h->ws);
     delete h;

@@ -76,10 +76,15 @@ struct ZArgs {
   Field wf;
 };
 
-// Tensor maps of the register-fused source update's four inputs (A, P_y, delta(k), S) over the
-// half grid M [kx][ky][kz < N/2] of the meshes of the register-fused family, built on the host; passed to the kernel by value.
+// Tensor maps over the half grids M [kx][ky][kz < N/2] of the register-fused family, built on the host and
+// passed to the kernels by value: the source update's four inputs (A, P_y, delta(k), S).
 struct KIterMaps {
   CUtensorMap m[4];
+};
+// A vector x pass's two inputs: G and Psi_y (inverse), psi^ and Z^ (forward); on: they were built.
+struct VLineMaps {
+  CUtensorMap m[2];
+  int on;
 };
 
 struct SArgs {
@@ -97,12 +102,13 @@ struct SArgs {
   int d_is_k;             // S_DELTA: dk is already fully transformed
   int lognormal;          // S_DELTA: subtract the lognormal constant at k = 0
   const int* skip_flag;   // plain passes: do nothing when *skip_flag != 0 (device-driven loop)
-  int narrow;             // plain x passes: 8-column instead of 16-column tiles
+  int narrow;             // single-field x passes: 8-column instead of 16-column tiles
   int generic;            // k-space update: the generic staged kernel instead of the register-fused one
-  int ybeg, ycount;       // paired x passes: only the lines of y-planes [ybeg, ybeg + ycount)
+  int ybeg, ycount;       // vector x passes: only the lines of y-planes [ybeg, ybeg + ycount)
                           // (ycount 0: every line; both multiples of the tile width)
   const KIterMaps* tmaps; // host memory: the source update streams its inputs by TMA
-  // paired inverse x pass (N = 512) unless loop_flag && *loop_flag == 1 (the device loop has just
+  const VLineMaps* vmaps; // host memory: the vector x passes' maps, forward and inverse (null: plain loads)
+  // vector inverse x pass unless loop_flag && *loop_flag == 1 (the device loop has just
   // converged): leave C = dx Psi_x + dy Psi_y in f[0] and Psi_z in wf for the projection pass,
   // instead of Psi_x, Psi_y, Psi_z in f[0..2]
   int cform;
@@ -139,6 +145,7 @@ struct MeshKernels {
   int kspace_fused;       // register-fused passes with paired vector x passes (unless the generic option
                           // is set): 7 field transfers per y pass, 4 per x and z pass
   int kmap_cols;          // columns of a tile of the TMA-streamed source update (0: none)
+  int vmap_cols;          // columns of a tile of the streamed vector x passes (0: none)
   // persistent Z pass; *grid_out receives the number of CTAs launched (its reduction partials)
   cudaError_t (*zpass)(int mode, int nc, const ZArgs& a, cudaStream_t st, int* grid_out);
   cudaError_t (*spass)(int mode, int nc, int axis, const SArgs& a, cudaStream_t st);
