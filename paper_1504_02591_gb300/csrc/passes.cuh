@@ -1671,8 +1671,7 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kit
 // shared-memory stage by cp.async.bulk.tensor, completing on an mbarrier.  As soon as the threads have
 // copied the tile into their registers the next tile's copies are issued into the same stage, so they
 // stream in while this tile's transforms and stores run.  The Nyquist tiles (a different layout, 2/(N+2)
-// of the data) follow with plain loads.  Each CTA's norms go to its partials; the rest of the regular
-// grid's partials are zeroed so the reduction over them is unchanged.  Every wait is bounded: a wait that
+// of the data) follow with plain loads.  Each CTA's norms go to its partials.  Every wait is bounded: a wait that
 // gives up writes NaN norms (the device loop then stops with RECON_ERR_NONFINITE), waits once more for the
 // copies and the CTA returns.
 // The kernel with direct loads is bound by the L1's data pipe, most of its wavefronts the 32-byte
@@ -1748,8 +1747,6 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
                                                                        const __grid_constant__ KIterMaps maps) {
   using K = KTma<N, C>;
   constexpr int T = K::T, H = N / 2, MT = N * (H / C), QT = N / C;
-  constexpr int kDirect = SCols<N, S_ITER>::v;
-  constexpr int kGridPartials = N * (H / kDirect) + N / kDirect;   // the regular grid whose partials the reduction reads
   extern __shared__ __align__(128) float4 ssm[];
   float2* tw = reinterpret_cast<float2*>(ssm);
   float2* s = tw + KFused<N, C>::TAB;
@@ -1821,10 +1818,6 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
     if (give_up) r0 = r1 = __longlong_as_double(0x7ff8000000000000ll);   // NaN: the loop stops
     a.partials[2 * blockIdx.x + 0] = r0;
     a.partials[2 * blockIdx.x + 1] = r1;
-  }
-  for (int b = blockIdx.x + gridDim.x + threadIdx.x * gridDim.x; b < kGridPartials; b += T * gridDim.x) {
-    a.partials[2 * b + 0] = 0.0;
-    a.partials[2 * b + 1] = 0.0;
   }
 }
 
@@ -2162,6 +2155,7 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
           const cudaError_t e = persistent_grid(k, K::T, K::smem, &grid);
           if (e != cudaSuccess) return e;
         }
+        if (a.npart) *a.npart = grid;
         void* args[] = {const_cast<SArgs*>(&a), const_cast<KIterMaps*>(a.tmaps)};
         return cudaLaunchKernel(k, dim3(grid), dim3(K::T), args, K::smem, st);
       }
@@ -2246,6 +2240,7 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
   }
 
   static cudaError_t spass(int mode, int nc, int axis, const SArgs& a, cudaStream_t st) {
+    if (a.npart) *a.npart = kSBlocks;   // S_ITER with one tile a CTA
     if (nc < 1 || nc > 3) return cudaErrorInvalidValue;
     // plain passes: one component per CTA, components along gridDim.y
     if (mode == S_FWD && axis == AX_Y) return slaunch<S_FWD, 1, AX_Y>(a, st, nc);
@@ -2279,8 +2274,8 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
   }
 
   static const MeshKernels* table() {
-    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0, kmap_cols(), vmap_cols(),
-                                  &zpass, &spass, &build_tables};
+    static const MeshKernels t = {N, kZBlocks, kSBlocks, ((Plan<N>::kTab + 1) & ~1) + kXTab<N>, Plan<N / 2>::kTab, kFusedMesh<N> ? 1 : 0,
+                                  kmap_cols(), vmap_cols(), &zpass, &spass, &build_tables};
     return &t;
   }
 };

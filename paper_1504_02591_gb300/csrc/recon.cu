@@ -987,9 +987,11 @@ recon_status iterate_start(recon_handle* h, float coef0) {
 recon_status iterate_body(recon_handle* h, cudaGraphConditionalHandle cond) {
   SArgs ia = sargs(h);
   for (int q = 0; q < 3; ++q) ia.f[q] = h->V[q];
+  int npart = 0;
+  ia.npart = &npart;
   RG_TRY(run_s(h, S_ITER, 3, AX_Y, ia));
-  RG_TRY(finalize(h, h->mk->s_blocks, 2, RED_NORM_D2, 0));
-  RG_CUDA(timed(h, RECON_K_OTHER, 0.0, [&] { return launch_loop_decide(h->loop, h->red, cond, h->st); }));
+  RG_CUDA(timed(h, RECON_K_OTHER, 16.0 * npart, [&] {
+    return launch_loop_decide(h->partials, npart, h->red, h->fin_bsum, h->fin_counter, h->loop, cond, h->st); }));
   ZArgs za = zargs(h);
   for (int q = 0; q < 3; ++q) za.f[q] = h->V[q];
   za.loop_flag = &h->loop->flag;
@@ -1194,10 +1196,12 @@ recon_status iterate_core(recon_handle* h, const StartSpec& sp, double tol, int 
     for (int q = 0; q < 3; ++q) za.f[q] = h->V[q];
     SArgs ia = sargs(h);
     for (int q = 0; q < 3; ++q) ia.f[q] = h->V[q];
+    int npart = 0;
+    ia.npart = &npart;
     double host_norm[2] = {0, 0};
     while (true) {
       RG_TRY(run_s(h, S_ITER, 3, AX_Y, ia));
-      RG_TRY(finalize(h, h->mk->s_blocks, 2, RED_NORM_D2, 0));
+      RG_TRY(finalize(h, npart, 2, RED_NORM_D2, 0));
       RG_CUDA(cudaMemcpyAsync(host_norm, h->red + RED_NORM_D2, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
       cudaEvent_t ev;
       RG_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));

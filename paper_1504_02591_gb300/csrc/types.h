@@ -94,6 +94,7 @@ struct SArgs {
   const float* fac;       // S_FACTOR: real factor on the half grid, M [kx][ky][kz < N/2] then Q [kx][ky]
   const float2* tabx;     // x lines of the register-fused family: their second-stage twiddles (set at launch)
   double* partials;       // per-block partials (2 per block, S_ITER)
+  int* npart;             // host memory: the launch of S_ITER says how many pairs of partials it leaves
   const double* red;      // reduction block (S_DELTA reads the lognormal sum)
   Field dk;               // delta: partially transformed (S_DELTA input) / k-space (S_ITER)
   Field sbuf;             // stored source S of the previous iteration
