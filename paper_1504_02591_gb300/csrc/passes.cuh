@@ -755,103 +755,117 @@ __global__ void __launch_bounds__(kZThreads, ZRow<N>::kMinBlocks) zfused_kernel(
   }
 }
 
-// Z_DELTA for N = 512 (at most 32 smoothing taps): each warp stages its row of rho_g (and rho_r)
-// with the periodic continuation the z convolution reads, each lane convolves 16 consecutive nodes
-// with the taps in registers (every staged value read once per 16 outputs; the row is stored with
-// one pad word per 16 so the lanes' windows fall in distinct banks), forms delta (mask, lognormal)
-// exactly as the generic pass, stores the real copy, and runs the r2c of the fused passes.
+// Z_DELTA of the family (at most 64 smoothing taps): each warp stages its row of rho_g, then of rho_r, with
+// the periodic continuation the z convolution reads; each lane convolves V consecutive nodes with V taps at a
+// time in registers (a staged value is read once per V outputs and V taps; one pad word per V, so the lanes'
+// windows fall in distinct banks), forms delta (mask, lognormal) exactly as the generic pass, stores the
+// real copy, and runs the r2c of the fused passes.  The generic pass reads every value once per tap:
+// 67 us against 182 at 256, 219 / 625 at 384, 518 / 637 at 512 (which had a form of 32 taps with both
+// rows staged) and 4430 / 11540 at 1024, one field.  Both fields staged at once leave fewer CTAs: 384 256,
+// 512 602, 1024 8830 us.
 template <int N>
-struct ZDelta8 {
-  static_assert(N == 512, "rows of 256 complex points");
-  static constexpr int L = N / 2, KT = 32, V = 16;
-  static constexpr int kExt = N + KT + V;                       // staged entries per row
-  static constexpr int kExtPad = kExt + kExt / 16 + 1;          // with one pad word per 16
-  static constexpr int kWarp = ZRow<N>::RPW * ZRow<N>::kRow + kExtPad;   // float2: FFT buffers + two staged rows
-  static constexpr size_t smem = sizeof(float2) * ((size_t)ZRow<N>::kHead + (size_t)kZWarps * kWarp);
-  __device__ __forceinline__ static int pad(int p) { return p + (p >> 4); }
+struct ZDeltaRow {
+  using ZR = ZRow<N>;
+  static constexpr int KT = 64, V = N <= 512 ? N / 32 : 16, PARTS = N / (32 * V);
+  static constexpr int kTaps = (KT + V - 1) / V * V;            // taps, zero beyond the last
+  static constexpr int kExt = N + kTaps;                        // staged entries per row
+  static constexpr int kExtPad = (kExt + kExt / V + 2) & ~1;    // with one pad word per V
+  static constexpr int kWarp = ZR::RPW * ZR::kRow + kExtPad / 2;   // float2: FFT buffers + a staged row
+  static constexpr size_t smem = sizeof(float2) * ((size_t)ZR::kHead + (size_t)kZWarps * kWarp) + sizeof(float) * kTaps;
+  static constexpr int kMinBlocks = N == 256 ? 4 : (N <= 512 ? 3 : 2);   // 512 at 2: 580 us
+  __device__ __forceinline__ static int pad(int p) { return p + p / V; }
 };
 
 template <int N>
-__global__ void __launch_bounds__(kZThreads, 2) zdelta8_kernel(const ZArgs a) {
-  using Z = ZDelta8<N>;
+__global__ void __launch_bounds__(kZThreads, ZDeltaRow<N>::kMinBlocks) zdelta_kernel(const ZArgs a) {
+  using Z = ZDeltaRow<N>;
   using ZR = ZRow<N>;
-  constexpr int L = Z::L, KT = Z::KT, V = Z::V, G = ZR::G, E = ZR::E;
+  constexpr int L = ZR::L, V = Z::V, PARTS = Z::PARTS, G = ZR::G, E = ZR::E;
   extern __shared__ float4 zsm[];
   float2* tw = reinterpret_cast<float2*>(zsm);
   float2* tab = tw + L + 1;
+  float* taps = reinterpret_cast<float*>(tw + ZR::kHead + kZWarps * Z::kWarp);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % G, grp = lane / G;
   float2* sw = tw + ZR::kHead + warp * Z::kWarp;                 // the rows' FFT buffers
-  float* xg = reinterpret_cast<float*>(sw + ZR::RPW * ZR::kRow); // staged rho_g row, then rho_r row
-  float* xr = xg + Z::kExtPad;
+  float* x = reinterpret_cast<float*>(sw + ZR::RPW * ZR::kRow);  // the staged row
   __shared__ double red_sh[kZWarps];
+  for (int j = threadIdx.x; j < Z::kTaps; j += kZThreads) taps[j] = j < a.ntap ? a.taps[j] : 0.f;
   zrow_tables<N>(a, tw, tab);
-  float tp[KT];
-#pragma unroll
-  for (int jt = 0; jt < KT; ++jt) tp[jt] = jt < a.ntap ? a.taps[jt] : 0.f;
   const double* red = a.red;
   const int nin = a.uniform ? 1 : 2;
   const float inv_alpha = a.uniform ? (float)((double)N * N * N / red[RED_SUM_WG]) : (float)(red[RED_SUM_WR] / red[RED_SUM_WG]);
   const float thr = a.uniform ? 0.f : (float)(a.mask_frac * red[RED_SUM_WR] / red[RED_CNT_RPOS]);
   const int partner = grp * G + (G - l) % G;
+  const int chunks = (a.ntap + V - 1) / V;
   float acc0 = 0.f, acc1 = 0.f;
 
   for (int it = blockIdx.x * kZWarps + warp; it < N * N / ZR::RPW; it += gridDim.x * kZWarps) {
 #pragma unroll 1
     for (int i = 0; i < ZR::RPW; ++i) {
       const size_t row = (size_t)it * ZR::RPW + i;
-      const float* rg = reinterpret_cast<const float*>(a.f[0].M) + row * N;
-      const float* rr = reinterpret_cast<const float*>(a.f[1].M) + row * N;
-      for (int p = lane; p < Z::kExt; p += 32) {
-        int src = (p + a.t0) % N;
-        if (src < 0) src += N;
-        xg[Z::pad(p)] = rg[src];
-        if (nin == 2) xr[Z::pad(p)] = rr[src];
-      }
-      __syncwarp();
-      const int z0 = V * lane;
-      float ag[V], ar[V];
+      float ag[PARTS][V], ar[PARTS][V];
+      auto smooth = [&](const float2* M, float (&acc)[PARTS][V]) {
+        const float* src = reinterpret_cast<const float*>(M) + row * N;
+#pragma unroll 8
+        for (int p = lane; p < Z::kExt; p += 32) {   // |t0| <= 32: one wrap at most
+          const int k = p + a.t0;
+          x[Z::pad(p)] = src[k < 0 ? k + N : (k >= N ? k - N : k)];
+        }
+        __syncwarp();
 #pragma unroll
-      for (int v = 0; v < V; ++v) ag[v] = ar[v] = 0.f;
+        for (int part = 0; part < PARTS; ++part) {
 #pragma unroll
-      for (int w = 0; w < KT + V - 1; ++w) {
-        const float g = xg[Z::pad(z0 + w)];
-        const float r = nin == 2 ? xr[Z::pad(z0 + w)] : 0.f;
+          for (int v = 0; v < V; ++v) acc[part][v] = 0.f;
+#pragma unroll 1
+          for (int c = 0; c < chunks; ++c) {
+            float tp[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-          const int jt = w - v;
-          if (jt >= 0 && jt < KT) {
-            ag[v] = fmaf(tp[jt], g, ag[v]);
-            if (nin == 2) ar[v] = fmaf(tp[jt], r, ar[v]);
+            for (int j = 0; j < V; ++j) tp[j] = taps[V * c + j];
+            const float* xo = x + (lane + 32 * part + c) * (V + 1);   // pad(V (lane + 32 part + c))
+#pragma unroll
+            for (int w = 0; w < 2 * V - 1; ++w) {
+              const float xv = xo[w + w / V];
+#pragma unroll
+              for (int v = 0; v < V; ++v)
+                if (w - v >= 0 && w - v < V) acc[part][v] = fmaf(tp[w - v], xv, acc[part][v]);
+            }
           }
         }
-      }
-      float d[V];
+        __syncwarp();                     // the staged row is rewritten by the next one
+      };
+      smooth(a.f[0].M, ag);
+      if (nin == 2) smooth(a.f[1].M, ar);
 #pragma unroll
-      for (int v = 0; v < V; ++v) {
-        float q;   // 1 + delta, kept as the ratio for the logarithm (see the generic pass)
-        if (nin == 1) {
-          q = ag[v] * inv_alpha;
-        } else {
-          const bool in = ar[v] > thr;
-          q = in ? ag[v] * inv_alpha / ar[v] : 1.f;
-          acc1 += in ? 1.f : 0.f;
+      for (int part = 0; part < PARTS; ++part) {
+        const int z0 = V * (lane + 32 * part);
+        float d[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          float q;   // 1 + delta, kept as the ratio for the logarithm (see the generic pass)
+          if (nin == 1) {
+            q = ag[part][v] * inv_alpha;
+          } else {
+            const bool in = ar[part][v] > thr;
+            q = in ? ag[part][v] * inv_alpha / ar[part][v] : 1.f;
+            acc1 += in ? 1.f : 0.f;
+          }
+          float dv = q - 1.f;
+          if (a.lognormal) {
+            dv = logf(fmaxf(q, 1e-6f));
+            acc0 += dv;
+          }
+          d[v] = dv;
         }
-        float dv = q - 1.f;
-        if (a.lognormal) {
-          dv = logf(fmaxf(q, 1e-6f));
-          acc0 += dv;
+        if (a.delta_real) {
+          float4* dr = reinterpret_cast<float4*>(a.delta_real + row * N + z0);
+#pragma unroll
+          for (int v4 = 0; v4 < V / 4; ++v4) dr[v4] = make_float4(d[4 * v4], d[4 * v4 + 1], d[4 * v4 + 2], d[4 * v4 + 3]);
         }
-        d[v] = dv;
-      }
-      if (a.delta_real) {
-        float4* dr = reinterpret_cast<float4*>(a.delta_real + row * N + z0);
 #pragma unroll
-        for (int v4 = 0; v4 < V / 4; ++v4) dr[v4] = make_float4(d[4 * v4], d[4 * v4 + 1], d[4 * v4 + 2], d[4 * v4 + 3]);
+        for (int k = 0; k < V / 2; ++k) sw[i * ZR::kRow + z0 / 2 + k] = make_float2(d[2 * k], d[2 * k + 1]);
       }
-#pragma unroll
-      for (int k = 0; k < V / 2; ++k) sw[i * ZR::kRow + z0 / 2 + k] = make_float2(d[2 * k], d[2 * k + 1]);
-      __syncwarp();                       // the staged rows are rewritten by the next one
     }
+    __syncwarp();
     float2 y[E];
 #pragma unroll
     for (int r = 0; r < E; ++r) y[r] = sw[grp * ZR::kRow + l + G * r];
@@ -2077,32 +2091,25 @@ struct MeshImpl {
   }
 
   static cudaError_t zdelta_fused(const ZArgs& a, cudaStream_t st, int* grid_out) {
-    if constexpr (N == 512) {
+    if constexpr (kFusedMesh<N>) {
       static int grid = 0;
-      const void* k = (const void*)zdelta8_kernel<N>;
-      const size_t smem = ZDelta8<N>::smem;
+      const void* k = (const void*)zdelta_kernel<N>;
       if (grid == 0) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int g = 0;
+        const cudaError_t e = persistent_grid(k, kZThreads, ZDeltaRow<N>::smem, &g);
         if (e != cudaSuccess) return e;
-        int dev = 0, sm = 0, occ = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kZThreads, smem)) != cudaSuccess) return e;
-        if (occ < 1) return cudaErrorInvalidConfiguration;
-        grid = occ * sm < kZBlocks ? occ * sm : kZBlocks;
+        grid = g < kZBlocks ? g : kZBlocks;
       }
       if (grid_out) *grid_out = grid;
       void* args[] = {const_cast<ZArgs*>(&a)};
-      return cudaLaunchKernel(k, dim3(grid), dim3(kZThreads), args, smem, st);
+      return cudaLaunchKernel(k, dim3(grid), dim3(kZThreads), args, ZDeltaRow<N>::smem, st);
     }
     return cudaErrorInvalidValue;
   }
 
   static cudaError_t zpass(int mode, int nc, const ZArgs& a, cudaStream_t st, int* grid_out) {
-    if constexpr (N == 512) {
-      if (mode == Z_DELTA && nc == 2 && !a.generic && a.ntap <= ZDelta8<N>::KT) return zdelta_fused(a, st, grid_out);
-    }
     if constexpr (kFusedMesh<N>) {
+      if (mode == Z_DELTA && nc == 2 && !a.generic && a.ntap <= ZDeltaRow<N>::KT) return zdelta_fused(a, st, grid_out);
       if (nc == 3 && !a.generic) {
         if (mode == Z_PROJ) return zfused<Z_PROJ>(a, st, grid_out);
         if (mode == Z_FINAL) return zfused<Z_FINAL>(a, st, grid_out);
