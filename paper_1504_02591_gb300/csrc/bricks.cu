@@ -38,7 +38,7 @@ template <typename PT>
 __device__ __forceinline__ void pack(const PT* __restrict__ pos, long long p, double scale21, int n,
                                      uint32_t (&q)[3]) {
 #pragma unroll
-  for (int a = 0; a < 3; ++a) q[a] = pack_axis((double)pos[3 * p + a], scale21, n);
+  for (int a = 0; a < 3; ++a) q[a] = pack_axis(widen(pos[3 * p + a]), scale21, n);
 }
 
 __device__ __forceinline__ uint32_t brick_key(const uint32_t (&q)[3], int nb) {
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(256) unsort_kernel(const float4* __restrict__ 
       double y[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        y[c] = (double)pos[3 * p + c] + d[c];
+        y[c] = widen(pos[3 * p + c]) + d[c];
         if (periodic) y[c] = wrap_box(y[c], L);
       }
       warp_store3(pos_out, p0, m, y, slots);

@@ -21,7 +21,7 @@ __device__ __forceinline__ void cic_setup(const PT* __restrict__ pos, long long 
   const double scale32 = scale * 4294967296.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const long long T = floor_scaled((double)pos[3 * p + a], scale32, 0.0);
+    const long long T = floor_scaled(widen(pos[3 * p + a]), scale32, 0.0);
     t[a] = (float)(uint32_t)T * 2.3283064365386963e-10f;   // 2^-32
     int c = (int)(T >> 32);
     if (c < 0 || c >= n) c = ((c % n) + n) % n;   // outside [0, L): periodic image
@@ -77,87 +77,166 @@ __global__ void __launch_bounds__(256) deposit_kernel(const PT* __restrict__ pos
 }
 
 // Nearest-grid-point binning (Sec. 3, the paper's scheme): node floor(u + 1/2) per axis, from the
-// same 32.32 fixed-point coordinate as the CIC kernel (u 2^32 + 2^31 rounded down).
+// same 32.32 fixed-point coordinate as the CIC kernel (u 2^32 + 2^31 rounded down).  Four particles'
+// positions are read before any is used: floor_scaled's rare branch keeps the compiler from doing so, and one
+// at a time the pass waits for memory (3e7 float64 positions with unit weights: 537 us, 657 one at a time).
 template <typename PT>
 __global__ void __launch_bounds__(256) ngp_deposit_kernel(const PT* __restrict__ pos, const float* __restrict__ w,
                                                           long long np, int n, double scale,
                                                           float* __restrict__ rho, double* __restrict__ partials) {
+  constexpr int U = 4;
   double wsum = 0.0;
   int count = 0;
   const size_t nn = (size_t)n;
   const double scale32 = scale * 4294967296.0;
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
-       p += (long long)gridDim.x * blockDim.x) {
-    int c[3];
+  const long long step = (long long)gridDim.x * blockDim.x;
+  for (long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; p0 < np; p0 += U * step) {
+    PT x[U][3];
+    float wp[U];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const long long T = floor_scaled((double)pos[3 * p + a], scale32, 2147483648.0);
-      int k = (int)(T >> 32);
-      if (k < 0 || k >= n) k = ((k % n) + n) % n;
-      c[a] = k;
+    for (int u = 0; u < U; ++u) {
+      const long long p = p0 + u * step < np ? p0 + u * step : p0;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[u][a] = __ldg(pos + 3 * p + a);
+      wp[u] = w ? __ldg(w + p) : 1.f;
     }
-    const float wp = w ? w[p] : 1.f;
-    if (w) wsum += wp;
-    else ++count;
-    atomicAdd(rho + ((size_t)c[0] * nn + c[1]) * nn + c[2], wp);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (p0 + u * step >= np) break;
+      int c[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const long long T = floor_scaled(widen(x[u][a]), scale32, 2147483648.0);
+        int k = (int)(T >> 32);
+        if (k < 0 || k >= n) k = ((k % n) + n) % n;
+        c[a] = k;
+      }
+      if (w) wsum += wp[u];
+      else ++count;
+      atomicAdd(rho + ((size_t)c[0] * nn + c[1]) * nn + c[2], wp[u]);
+    }
   }
   const double s = block_sum_d(w ? wsum : (double)count);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
+// x as the sum of two float32, by integer operations (a float64 conversion or sum costs 16 clocks a warp and
+// SM here, and a pass over 3.1e7 float64 positions spent them on little else): hi holds the 24 leading bits of
+// x and lo the 24 that follow, so x - hi - lo is less than 2^-47 |x|.  False outside 2^-60 <= |x| < 2^60
+// (but true for zero).
+__device__ __forceinline__ bool split_pair(double x, float& hi, float& lo) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const uint32_t h = (uint32_t)(b >> 32), e = (h >> 20) & 0x7ffu;
+  const uint32_t top = (uint32_t)(b >> 29) & 0x7fffffu, low = (uint32_t)(b >> 5) & 0xffffffu;
+  const uint32_t sign = h & 0x80000000u, e8 = (e - 896u) << 23;     // 1023 - 127 = 896
+  hi = __uint_as_float(sign | e8 | top);
+  lo = __uint_as_float(sign | (e8 - (47u << 23))) * (float)low;     // 2^(exponent - 47) times an integer below 2^24
+  if (b << 1 == 0) hi = lo = 0.f;
+  return b << 1 == 0 || e - 963u < 120u;                            // 1023 - 60 = 963
+}
+__device__ __forceinline__ bool split_pair(float x, float& hi, float& lo) {
+  hi = x;
+  lo = 0.f;
+  return fabsf(x) < 1e18f;
+}
+
 // Shell of a particle: floor((r - rmin) inv_dr) clamped to [-1, nbins], r its float64 distance from obs.
-// float64 square roots and quotients cost most of a pass here, so the shell is found in float32 (offsets
-// taken in float64) unless the coordinate lies so near a shell's edge that its rounding could matter: the
-// float32 coordinate is off by at most 2^-24 (3.5 r + 2 rmin) inv_dr + 2^-23 |f| (three rounded offsets, two
-// fused sums and a correctly rounded root, then one difference and one product); the margin is five times
-// that.  Near an edge, and for coordinates that are not finite, the float64 expression decides.
+// float64 operations cost most of a pass here, so the shell is found in float32 (the offsets from pairs) unless
+// the coordinate lies so near a shell's edge that its rounding could matter: the float32 coordinate is off
+// by at most 2^-24 (5 r + 2 rmin) inv_dr + 2^-23 |f| (three offsets of two roundings, two fused sums and a
+// correctly rounded root, then one difference and one product) and what the pairs leave out, less than
+// 2^-46 of |x| and |obs| on each axis; the margin is three times that and more.  Near an edge, and for
+// coordinates that are not finite, the float64 expression decides.
+struct ShellArgs {
+  double3 obs;
+  float3 hi, lo;         // obs as pairs
+  double rmin, inv_dr;
+  int nbins;
+  int pairs;             // obs fits them
+};
+
 template <typename PT>
-__device__ __forceinline__ int shell_of(const PT* __restrict__ pos, long long p, double3 obs, double rmin, double inv_dr,
-                                        int nbins) {
-  const double dx = (double)pos[3 * p] - obs.x, dy = (double)pos[3 * p + 1] - obs.y, dz = (double)pos[3 * p + 2] - obs.z;
-  const float fx = (float)dx, fy = (float)dy, fz = (float)dz;
+__device__ __forceinline__ int shell_of(PT x, PT y, PT z, const ShellArgs& a) {
+  float hx, lx, hy, ly, hz, lz;
+  const bool ok = split_pair(x, hx, lx) & split_pair(y, hy, ly) & split_pair(z, hz, lz) & (a.pairs != 0);
+  const float fx = (hx - a.hi.x) + (lx - a.lo.x), fy = (hy - a.hi.y) + (ly - a.lo.y), fz = (hz - a.hi.z) + (lz - a.lo.z);
   const float r = __fsqrt_rn(fmaf(fx, fx, fmaf(fy, fy, fz * fz)));
-  const float rm = (float)rmin, inv = (float)inv_dr;
+  const float rm = (float)a.rmin, inv = (float)a.inv_dr;
   const float f = (r - rm) * inv;
-  const float margin = fmaf(1.2e-6f * (r + fabsf(rm)), inv, 6e-7f * fabsf(f));
+  const float left = 1e-13f * ((fabsf(hx) + fabsf(a.hi.x)) + (fabsf(hy) + fabsf(a.hi.y)) + (fabsf(hz) + fabsf(a.hi.z)));
+  const float margin = fmaf(fmaf(1.2e-6f, r + fabsf(rm), left), inv, 6e-7f * fabsf(f));
   const float k = floorf(f);
-  if (f - k > margin && k + 1.f - f > margin && r > 1e-15f && r < 1e18f && fabsf(f) < 1e6f)
-    return k < 0.f ? -1 : (k >= (float)nbins ? nbins : (int)k);
-  const double b = floor((sqrt(dx * dx + dy * dy + dz * dz) - rmin) * inv_dr);
-  return b >= 0.0 ? (b < (double)nbins ? (int)b : nbins) : -1;
+  if (ok && f - k > margin && k + 1.f - f > margin && r > 1e-15f && r < 1e18f && fabsf(f) < 1e6f)
+    return k < 0.f ? -1 : (k >= (float)a.nbins ? a.nbins : (int)k);
+  const double dx = (double)x - a.obs.x, dy = (double)y - a.obs.y, dz = (double)z - a.obs.z;
+  const double b = floor((sqrt(dx * dx + dy * dy + dz * dz) - a.rmin) * a.inv_dr);
+  return b >= 0.0 ? (b < (double)a.nbins ? (int)b : a.nbins) : -1;
+}
+
+// Shells of the particles p0 + u step below np, u < U, their positions read before any is used.
+template <int U, typename PT, class Fn>
+__device__ __forceinline__ void shells(const PT* __restrict__ pos, long long p0, long long step, long long np,
+                                       const ShellArgs& a, Fn&& fn) {
+  PT x[U][3];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const long long p = p0 + u * step < np ? p0 + u * step : p0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) x[u][c] = __ldg(pos + 3 * p + c);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (p0 + u * step < np) fn(p0 + u * step, shell_of(x[u][0], x[u][1], x[u][2], a));
 }
 
 // Radial number density (Sec. 3.2 n(z), in comoving distance from the observer): counts of the
 // particles in nbins equal shells of [rmin, rmax), float64 distances; counted per block in shared memory
 // (6e5 galaxies in 50 shells: 120 us when every particle went to a global counter).
 template <typename PT>
-__global__ void __launch_bounds__(256) radial_hist_kernel(const PT* __restrict__ pos, long long np, double3 obs,
-                                                          double rmin, double inv_dr, int nbins,
+__global__ void __launch_bounds__(256) radial_hist_kernel(const PT* __restrict__ pos, long long np, const ShellArgs a,
                                                           unsigned long long* __restrict__ counts) {
+  const int nbins = a.nbins;
   __shared__ unsigned int h[4096];
   for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0u;
   __syncthreads();
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
-       p += (long long)gridDim.x * blockDim.x) {
-    const int b = shell_of(pos, p, obs, rmin, inv_dr, nbins);
-    if (b >= 0 && b < nbins) atomicAdd(h + b, 1u);
-  }
+  const long long step = (long long)gridDim.x * blockDim.x;
+  for (long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; p0 < np; p0 += 4 * step)
+    shells<4>(pos, p0, step, np, a, [&](long long, int b) {
+      if (b >= 0 && b < nbins) atomicAdd(h + b, 1u);
+    });
   __syncthreads();
   for (int b = threadIdx.x; b < nbins; b += blockDim.x)
     if (h[b]) atomicAdd(counts + b, (unsigned long long)h[b]);
 }
 
 // FKP weights (Sec. 3.2): the table's entry of the particle's shell, its last entry outside the shells.
-// A weight depends on the shell alone, so the quotients are formed once per shell on the host.
+// A weight depends on the shell alone, so the quotients are formed once per shell on the host.  Bound by the
+// positions' bytes: 3.1e7 float64 positions 355 us with float64 offsets, 220 with pairs.
 template <typename PT>
-__global__ void __launch_bounds__(256) fkp_kernel(const PT* __restrict__ pos, long long np, double3 obs, double rmin,
-                                                  double inv_dr, int nbins, const float* __restrict__ wtab,
-                                                  float* __restrict__ w) {
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np;
-       p += (long long)gridDim.x * blockDim.x) {
-    const int b = shell_of(pos, p, obs, rmin, inv_dr, nbins);
-    w[p] = __ldg(wtab + (b < 0 ? nbins : b));
+__global__ void __launch_bounds__(256) fkp_kernel(const PT* __restrict__ pos, long long np, const ShellArgs a,
+                                                  const float* __restrict__ wtab, float* __restrict__ w) {
+  const long long step = (long long)gridDim.x * blockDim.x;
+  for (long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; p0 < np; p0 += 4 * step)
+    shells<4>(pos, p0, step, np, a, [&](long long p, int b) { w[p] = __ldg(wtab + (b < 0 ? a.nbins : b)); });
+}
+
+static ShellArgs shell_args(double3 obs, double rmin, double inv_dr, int nbins) {
+  ShellArgs a{};
+  a.obs = obs;
+  a.rmin = rmin;
+  a.inv_dr = inv_dr;
+  a.nbins = nbins;
+  const double o[3] = {obs.x, obs.y, obs.z};
+  float hi[3], lo[3];
+  a.pairs = 1;
+  for (int c = 0; c < 3; ++c) {
+    hi[c] = (float)o[c];
+    lo[c] = (float)(o[c] - (double)hi[c]);
+    if (!(o[c] > -1e18 && o[c] < 1e18)) a.pairs = 0;
   }
+  a.hi = make_float3(hi[0], hi[1], hi[2]);
+  a.lo = make_float3(lo[0], lo[1], lo[2]);
+  return a;
 }
 
 __global__ void __launch_bounds__(256) pack_psi_kernel(const float4* __restrict__ x, const float4* __restrict__ y,
@@ -238,7 +317,7 @@ __global__ void __launch_bounds__(256) shift_kernel(const PT* __restrict__ pos, 
       double y[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        y[c] = (double)pos[3 * p + c] + d[c];
+        y[c] = widen(pos[3 * p + c]) + d[c];
         if (a.periodic) y[c] = wrap_box(y[c], a.L);
       }
       warp_store3(a.pos_out, p0, np, y, slots);
@@ -403,10 +482,11 @@ cudaError_t launch_radial_hist(const void* pos, int dtype, long long np, double3
   if (np <= 0) return cudaSuccess;
   const double inv_dr = nbins / (rmax - rmin);
   const int blocks = (int)((np + 255) / 256 < 152 * 16 ? (np + 255) / 256 : 152 * 16);
+  const ShellArgs sa = shell_args(obs, rmin, inv_dr, nbins);
   if (dtype == 0)
-    radial_hist_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, obs, rmin, inv_dr, nbins, counts);
+    radial_hist_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, sa, counts);
   else
-    radial_hist_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, obs, rmin, inv_dr, nbins, counts);
+    radial_hist_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, sa, counts);
   return cudaGetLastError();
 }
 
@@ -415,10 +495,11 @@ cudaError_t launch_fkp(const void* pos, int dtype, long long np, double3 obs, do
   if (np <= 0) return cudaSuccess;
   const double inv_dr = nbins / (rmax - rmin);
   const int blocks = (int)((np + 255) / 256 < 152 * 16 ? (np + 255) / 256 : 152 * 16);
+  const ShellArgs sa = shell_args(obs, rmin, inv_dr, nbins);
   if (dtype == 0)
-    fkp_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, obs, rmin, inv_dr, nbins, wtab, w);
+    fkp_kernel<double><<<blocks, 256, 0, st>>>((const double*)pos, np, sa, wtab, w);
   else
-    fkp_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, obs, rmin, inv_dr, nbins, wtab, w);
+    fkp_kernel<float><<<blocks, 256, 0, st>>>((const float*)pos, np, sa, wtab, w);
   return cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
 // cic.h: launchers of the particle kernels and the reduction helpers.
 #pragma once
 #include <cuda_runtime.h>
+#include <stdint.h>
 #include <stddef.h>
 
 namespace rg {
@@ -22,6 +23,21 @@ struct ShiftArgs {
   double* pos_out;       // (n, 3) out or null
 };
 
+// The rare branches below are calls: inlined, the compiler turns them into predicated float64 operations that
+// every particle pays (3e7 float64 positions to the nearest nodes: 652 us so, 330 with calls).
+[[maybe_unused]] static __device__ __noinline__ long long floor_far(double x, double s, double c) { return __double2ll_rd(fma(x, s, c)); }
+[[maybe_unused]] static __device__ __noinline__ double widen_far(float x) { return (double)x; }
+
+// x in float64 by integer operations (the conversion takes a float64 slot); subnormals, infinities and NaN by
+// the conversion.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e - 1u < 254u || u << 1 == 0)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (u << 1 ? 0x38000000u : 0u))), (int)(u << 29));
+  return widen_far(x);
+}
+
 // floor(x s + c) for x s + c as one exact product and sum: a fused multiply-add rounded down onto
 // 1.5 x 2^52, whose low mantissa bits are then the integer.  One float64 operation where a product and a
 // conversion take two (float64 runs at 1/64 of the float32 rate here, and positions are float64).  c is
@@ -31,7 +47,7 @@ __device__ __forceinline__ long long floor_scaled(double x, double s, double c) 
   const double v = __fma_rd(x, s, magic + c);
   const long long b = __double_as_longlong(v);
   if ((b >> 52) == 0x433) return b - 0x4338000000000000ll;
-  return __double2ll_rd(fma(x, s, c));
+  return floor_far(x, s, c);
 }
 
 // y - floor(y / L) L, stepped back once more if that rounds to L: a shifted position wrapped into the box.
