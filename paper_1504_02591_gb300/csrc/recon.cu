@@ -1332,8 +1332,8 @@ namespace {
 // gather 72 us per 1e6 up to N = 128 and, where the three fields pass the L2, 140, 210, 330 and 410 at
 // N = 256, 384, 512 and 1024 for tracers all over the box (half of that for a survey's tenth of it).
 // Measured, uniform tracers, sorted / direct us: N = 64 2e6 419 / 146; 256 1e7 719 / 1403 (packed: 747);
-// 384 2e6 508 / 452, 1e7 979 / 2131; 512 2e6 1014 / 682, 1e7 1499 / 3311; 1024 1e7 10784 / 4186, 3.3e7
-// 13328 / 13825.  The two meet near N^3 / 32 tracers on the meshes that sort at all.
+// 384 2e6 508 / 452, 1e7 948 / 2131; 512 2e6 1014 / 682, 1e7 1499 / 3311; 1024 1e7 10784 / 4186, 3.3e7
+// 10730 / 13830.  The two meet near N^3 / 32 tracers on the meshes that sort at all.
 bool shift_sorts(int n, int64_t count) { return n >= 384 && count >= (int64_t)n * n * n / 32; }
 // Packing the nodes as float4 (28 bytes moved per node: 12 us at N <= 128, 95 at 256) halves the direct
 // gather: 35 us per 1e6 tracers up to N = 128, 65 at 256; from N^3 / 8 tracers on (and 200,000) it pays.
