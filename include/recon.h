@@ -50,7 +50,8 @@ typedef enum recon_status {
   RECON_ERR_NOT_CONVERGED = 4, /* max_iter reached before tol; all outputs are still valid      */
   RECON_ERR_NONFINITE = 5,     /* a NaN or Inf appeared in the convergence norms                */
   RECON_ERR_STATE = 6,         /* calls out of order (create -> deposit -> smooth -> iterate)   */
-  RECON_ERR_TIMEOUT = 7,       /* a bounded device-side wait gave up                            */
+  RECON_ERR_TIMEOUT = 7,       /* a bounded device-side wait gave up: recon_iterate(_from) and
+                                  recon_start_features return it until the next recon_deposit   */
   RECON_ERR_UNSUPPORTED = 8    /* a valid request this build does not implement                 */
 } recon_status;
 
@@ -360,6 +361,10 @@ enum {
                                    (4 8 8, its z half-length plan 4 4 8) and N = 384 (6 8 8; 3 8 8),
                                    other meshes UNSUPPORTED.  Same transforms up to float32 rounding;
                                    the batch autotuner times both.                               */
+  RECON_OPT_DROP_COPY = 10,     /* for tests of RECON_ERR_TIMEOUT: 0 (default); the streamed kernels of the
+                                   register-fused path leave out one tile's copy, so that a bounded wait
+                                   runs out: 1 in the vector x passes (N = 256, 384, 512), 2 in the source
+                                   update                                                         */
   RECON_OPT_PLANE_BATCH = 6     /* register-fused path: 0 (off) or 16, 32, 64 y-planes per
                                    batch; each update then runs its inverse x, projection and forward
                                    x passes batch by batch, so a batch's fields stay in the L2 between
@@ -375,7 +380,7 @@ enum {
  * particles; otherwise it runs as DIRECT. */
 enum { RECON_PATH_DIRECT = 0, RECON_PATH_SORTED = 1 };
 
-/* Set a handle option (values 0 or 1, RECON_OPT_PLANE_BATCH 0/16/32/64); INVALID_ARG for an unknown
+/* Set a handle option (values 0 or 1, RECON_OPT_PLANE_BATCH 0/16/32/64, RECON_OPT_DROP_COPY 0/1/2); INVALID_ARG for an unknown
  * option or value; UNSUPPORTED for RECON_OPT_FFT_RADIX 1 on a mesh with one radix order; CUDA if
  * rebuilding the stage tables for another radix order fails. */
 recon_status recon_set_option(recon_handle* h, int option, int value);

@@ -338,10 +338,11 @@ extern "C" recon_status recon_batch_run(recon_batch_item* items, int n_items, vo
           it.n_iter = res[k].it;
           it.rel = res[k].rel;
           it.ms = (float)((double)(res[k].t1 - res[k].t0) * 1e-6);
-          if (res[k].flag == 2) it.status = RECON_ERR_NONFINITE;
+          if (res[k].flag == 3) it.status = RECON_ERR_TIMEOUT;
+          else if (res[k].flag == 2) it.status = RECON_ERR_NONFINITE;
           else if (it.tol > 0 && it.rel >= it.tol) it.status = RECON_ERR_NOT_CONVERGED;
           else it.status = RECON_OK;
-          if (it.status == RECON_ERR_NONFINITE) fail(RECON_ERR_NONFINITE);
+          if (it.status == RECON_ERR_NONFINITE || it.status == RECON_ERR_TIMEOUT) fail((recon_status)it.status);
         }
       }
     } while (0);

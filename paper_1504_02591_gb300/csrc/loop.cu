@@ -62,7 +62,7 @@ __global__ void stamp_kernel(unsigned long long* t) {
 
 __global__ void loop_record_kernel(const LoopState* s, BatchSlot* out) {
   const int it = s->it;
-  out->flag = s->flag;
+  out->flag = s->fault ? 3 : s->flag;
   out->it = it;
   out->rel = (it > 0 && it <= kMaxTrace) ? s->trace[it - 1] : 0.0;
 }

@@ -1686,8 +1686,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KFused<N, C>::kMinBlocks) kit
 // copied the tile into their registers the next tile's copies are issued into the same stage, so they
 // stream in while this tile's transforms and stores run.  The Nyquist tiles (a different layout, 2/(N+2)
 // of the data) follow with plain loads.  Each CTA's norms go to its partials.  Every wait is bounded: a wait that
-// gives up writes NaN norms (the device loop then stops with RECON_ERR_NONFINITE), waits once more for the
-// copies and the CTA returns.
+// gives up sets the fault word (the host returns RECON_ERR_TIMEOUT), waits once more for the copies, and the CTA
+// returns with NaN norms (the device loop then stops).
 // The kernel with direct loads is bound by the L1's data pipe, most of its wavefronts the 32-byte
 // segments of its 4-column tiles' rows, and wider tiles leave it one CTA per SM with nothing to overlap.
 // Streaming takes the loads off that pipe and overlaps them within one CTA, so the tiles are 8 columns
@@ -1737,7 +1737,8 @@ __device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait for a phase of the barrier, two seconds of the global timer at most.
+// Wait for a phase of the barrier, two seconds of the global timer at most; the last try comes after the limit,
+// so a process that was not scheduled meanwhile does not give up on copies that have landed.
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   if (bar_try_wait(bar, parity)) return true;
   unsigned long long t0, t1;
@@ -1746,7 +1747,7 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
     if (bar_try_wait(bar, parity)) return true;
     asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t1));
   } while (t1 - t0 <= 2000000000ull);
-  return false;
+  return bar_try_wait(bar, parity);
 }
 
 // hi + lo += x, the rounding of hi kept in lo.
@@ -1784,7 +1785,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
     for (int q = 0; q < 4; ++q)
 #pragma unroll
       for (int h = 0; h < K::kBoxes; ++h)
-        tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, K::kRows * h, kx, bar);
+        if (!(a.drop == 2 && q == 1 && tt == 0))
+          tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, K::kRows * h, kx, bar);
   };
   float dh = 0.f, dl = 0.f, sh = 0.f, sl = 0.f;   // norms over the CTA's tiles, in pairs of float32
   float2 v[2][8], dk[8], sp[8];
@@ -1792,7 +1794,10 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
   if (threadIdx.x == 0 && (int)blockIdx.x < MT) issue(blockIdx.x);
   for (int tt = blockIdx.x; tt < MT; tt += gridDim.x) {
     const bool ok = bar_wait(bar, parity);
-    if (!ok) bar_wait(bar, parity);
+    if (!ok) {
+      *a.fault = 1;
+      bar_wait(bar, parity);
+    }
     parity ^= 1u;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -1845,8 +1850,9 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
 // arrive while this tile is transformed, the Nyquist tiles (and every tile where the maps could not be
 // built) by plain loads.  The lines go through one exchange buffer one after the other and a thread holds
 // 16 points at most, so one or two CTAs fill the SM's threads; each field's stage is refilled as soon as its
-// last reader has passed a barrier.  A wait that gives up leaves NaN in its tile (the norms, and the loop's
-// outcome, then are NaN too).
+// last reader has passed a barrier.  A wait that gives up sets the fault word (the host returns
+// RECON_ERR_TIMEOUT) and leaves NaN in its tile; its CTA issues no further copy, waits once more for those on
+// their way, and returns.
 // The pass is bound by the reads and writes at a stride of a whole plane, each 2 MB page giving a tile one or
 // two rows: 16 columns (128-byte rows) against 8 (64 bytes), inverse / forward us, 512 450 / 444 against
 // 563 / 537, 384 194 / 192 against 195 / 191, 256 61 / 59 against 62 / 61.  The kernel that one tile's two
@@ -1904,7 +1910,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, VLine<N, C>::kMinBlocks) vlin
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar + 8 * q), "r"((uint32_t)K::kField) : "memory");
 #pragma unroll
     for (int h = 0; h < K::kBoxes; ++h)
-      tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, ky, K::kRows * h, bar + 8 * q);
+      if (!(a.drop == 1 && q == 1 && tt == 0))
+        tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, ky, K::kRows * h, bar + 8 * q);
   };
   const Geometry& g = a.g;
   const bool cf = INV && a.cform && !(a.loop_flag && *a.loop_flag == 1);
@@ -1925,7 +1932,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, VLine<N, C>::kMinBlocks) vlin
     auto wait = [&](int q) {
       if (tt >= streamed || bar_wait(bar + 8 * q, parity)) return true;
       give_up = 1;
-      bar_wait(bar + 8 * q, parity);
+      *a.fault = 1;
+      bar_wait(bar + 8 * q, parity);   // the copies must not land after the CTA is gone
       return false;
     };
     auto load = [&](int q, int f, bool ok, float2 (&x)[8]) {   // the stage's field q, which is field f
@@ -1952,7 +1960,11 @@ __global__ void __launch_bounds__(KFused<N, C>::T, VLine<N, C>::kMinBlocks) vlin
 #pragma unroll
     for (int r = 0; r < 8; ++r) w[r] = v[0][r];
     load(0, F0, ok, v[0]);
-    kline_fft<INV, N, C, 1, 1>(v, s, tw, j, col, [&] { issue(0, next); });
+    int stop0 = 0, stop = 0;   // give_up, each read between two barriers with no wait in between
+    kline_fft<INV, N, C, 1, 1>(v, s, tw, j, col, [&] {
+      stop0 = give_up;
+      if (!stop0) issue(0, next);
+    });
     {
       float2* __restrict__ P = !INV ? at(1) : (cf ? (t.isQ ? a.wf.Q : a.wf.M) : at(2));
       const float sc = INV ? kdz : dy;
@@ -1961,10 +1973,9 @@ __global__ void __launch_bounds__(KFused<N, C>::T, VLine<N, C>::kMinBlocks) vlin
     }
     ok = wait(1);
     load(1, F1, ok, v[0]);
-    int stop = 0;
     kline_fft<INV, N, C, 1, 0>(v, s, tw, j, col, [&] {
-      stop = give_up;   // no wait between this barrier and the next
-      issue(1, next);
+      stop = give_up;
+      if (!stop) issue(1, next);
     });
     float2* __restrict__ P0 = at(INV ? 0 : 2);
     if (cf) {
@@ -1988,7 +1999,10 @@ __global__ void __launch_bounds__(KFused<N, C>::T, VLine<N, C>::kMinBlocks) vlin
         P0[o0 + r * step] = make_float2(fmaf(k, w[r].x, x.x), fmaf(k, w[r].y, x.y));
       }
     }
-    if (stop) break;
+    if (stop) {
+      if (!stop0 && next < streamed) bar_wait(bar, parity ^ 1u);   // the next tile's first field is on its way
+      break;
+    }
     if (tt < streamed) parity ^= 1u;
     __syncthreads();   // s is free
   }

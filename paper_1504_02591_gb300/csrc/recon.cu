@@ -175,6 +175,7 @@ struct recon_handle {
   int plane_batch = 0;   // register-fused path: y-planes per batch of the x -> z -> x passes (0: off)
   int assign = 0;        // mass assignment of the deposit: 0 CIC, 1 NGP (the paper's binning)
   int kiter_tma = 1;     // register-fused path: 1 streams the source update's inputs by TMA
+  int drop_copy = 0;     // tests: a streamed pass leaves a copy out (RECON_OPT_DROP_COPY)
   int radix_order = 0;   // FFT plans: 0 default, 1 the alternative order (mk is that order's table)
   bool tmaps_ok = false; // the tensor maps were built
   KIterMaps tmaps{};
@@ -206,15 +207,13 @@ struct recon_handle {
   struct GraphKey {
     uint32_t coef0_bits;
     const float* u0;
-    int level, max_iter, d_is_k, generic, narrow, planes, tma, radix;
+    int level, max_iter, d_is_k, generic, narrow, planes, tma, radix, drop;
     uint64_t tol_bits;
     uint64_t epoch;
     bool operator==(const GraphKey& o) const {
       return coef0_bits == o.coef0_bits && u0 == o.u0 && level == o.level && max_iter == o.max_iter &&
              d_is_k == o.d_is_k && generic == o.generic && narrow == o.narrow && planes == o.planes && tma == o.tma &&
-             radix == o.radix &&
-             tol_bits == o.tol_bits &&
-             epoch == o.epoch;
+             radix == o.radix && drop == o.drop && tol_bits == o.tol_bits && epoch == o.epoch;
     }
   };
   struct GraphCache {
@@ -328,6 +327,8 @@ SArgs sargs(recon_handle* h) {
   a.lognormal = h->p.lognormal;
   a.tmaps = (h->tmaps_ok && h->kiter_tma) ? &h->tmaps : nullptr;
   a.vmaps = h->tmaps_ok ? h->vmaps : nullptr;
+  a.fault = &h->loop->fault;
+  a.drop = h->drop_copy;
   a.wf = h->W;
   return a;
 }
@@ -828,6 +829,11 @@ recon_status set_radix_order(recon_handle* h, int value);
 recon_status recon_set_option(recon_handle* h, int option, int value) {
   if (!h) return RECON_ERR_INVALID_ARG;
   if (option == RECON_OPT_PLANE_BATCH) return set_plane_batch(h, value);
+  if (option == RECON_OPT_DROP_COPY) {
+    if (value < 0 || value > 2) return RECON_ERR_INVALID_ARG;
+    h->drop_copy = value;
+    return RECON_OK;
+  }
   if (value != 0 && value != 1) return RECON_ERR_INVALID_ARG;
   if (option == RECON_OPT_FFT_RADIX) return set_radix_order(h, value);
   if (option == RECON_OPT_DEPOSIT_PATH) h->deposit_path = value;
@@ -1094,7 +1100,7 @@ recon_status build_graph(recon_handle* h, const StartSpec& sp, double tol, int m
 }
 
 recon_status iterate_graph(recon_handle* h, const StartSpec& sp, double tol, int max_iter, int* it_out,
-                           double* rel_out, int* flag_out) {
+                           double* rel_out, int* flag_out, int* fault_out) {
   recon_handle::GraphKey key{};
   std::memcpy(&key.coef0_bits, &sp.coef0, sizeof(float));
   std::memcpy(&key.tol_bits, &tol, sizeof(double));
@@ -1107,16 +1113,17 @@ recon_status iterate_graph(recon_handle* h, const StartSpec& sp, double tol, int
   key.planes = h->plane_batch;
   key.tma = h->kiter_tma;
   key.radix = h->radix_order;
+  key.drop = h->drop_copy;
   key.epoch = h->epoch;
   if (!(h->gcache.valid && h->gcache.key == key)) {
     RG_TRY(build_graph(h, sp, tol, max_iter));
     h->gcache.key = key;
   }
   RG_CUDA(cudaGraphLaunch(h->gcache.exec, h->st));
-  int hdr[2];
-  RG_CUDA(cudaMemcpyAsync(hdr, h->loop, sizeof(hdr), cudaMemcpyDeviceToHost, h->st));
+  LoopState hdr;   // all but the trace
+  RG_CUDA(cudaMemcpyAsync(&hdr, h->loop, offsetof(LoopState, trace), cudaMemcpyDeviceToHost, h->st));
   RG_CUDA(cudaStreamSynchronize(h->st));
-  const int it = hdr[1];
+  const int it = hdr.it;
   h->trace.assign(it < kMaxTrace ? it : kMaxTrace, 0.0);
   if (!h->trace.empty())
     RG_CUDA(cudaMemcpy(h->trace.data(), h->loop->trace, h->trace.size() * sizeof(double), cudaMemcpyDeviceToHost));
@@ -1127,7 +1134,8 @@ recon_status iterate_graph(recon_handle* h, const StartSpec& sp, double tol, int
   }
   *it_out = it;
   *rel_out = h->trace.empty() ? 0.0 : h->trace.back();
-  *flag_out = hdr[0];
+  *flag_out = hdr.flag;
+  *fault_out = hdr.fault;
   return RECON_OK;
 }
 
@@ -1172,6 +1180,14 @@ recon_status run_start(recon_handle* h, const StartSpec& sp) {
   return iterate_start_warm(h, sp.u0, sp.level);
 }
 
+// Whether a streamed pass's bounded wait gave up since the deposit: what the passes left is then not to be used.
+recon_status check_fault(recon_handle* h) {
+  int fault = 0;
+  RG_CUDA(cudaMemcpyAsync(&fault, &h->loop->fault, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  RG_CUDA(cudaStreamSynchronize(h->st));
+  return fault ? RECON_ERR_TIMEOUT : RECON_OK;
+}
+
 // The loop of Sec. 5.1 after a start: device-driven (one CUDA graph) or host-driven.
 recon_status iterate_core(recon_handle* h, const StartSpec& sp, double tol, int max_iter, int* n_iter,
                           double* rel_change) {
@@ -1182,10 +1198,13 @@ recon_status iterate_core(recon_handle* h, const StartSpec& sp, double tol, int 
   int it = 0;
   recon_status result = RECON_OK;
   if (h->use_graph && !h->timing && max_iter <= kMaxTrace) {
-    int flag = 0;
-    RG_TRY(iterate_graph(h, sp, tol, max_iter, &it, &rel, &flag));
+    int flag = 0, fault = 0;
+    RG_TRY(iterate_graph(h, sp, tol, max_iter, &it, &rel, &flag, &fault));
     h->d_is_k = 1;
-    if (flag == 2) {
+    if (fault) {
+      h->state = ST_SMOOTHED;
+      result = RECON_ERR_TIMEOUT;
+    } else if (flag == 2) {
       h->state = ST_SMOOTHED;
       result = RECON_ERR_NONFINITE;
     }
@@ -1236,6 +1255,13 @@ recon_status iterate_core(recon_handle* h, const StartSpec& sp, double tol, int 
       zc.cform = cf;
       RG_TRY(run_z(h, Z_PROJ, 3, zc));
       RG_TRY(xpass(h, S_FWD, 3, h->V));
+    }
+    if (h->mk->kspace_fused && !h->kspace_generic) {
+      const recon_status fs = check_fault(h);
+      if (fs != RECON_OK) {
+        h->state = ST_SMOOTHED;
+        result = fs;
+      }
     }
   }
   if (result == RECON_OK) {
@@ -1304,6 +1330,7 @@ recon_status recon_start_features(recon_handle* h, int start, int level, float* 
     return launch_radial(reinterpret_cast<const float*>(h->V[0].M), nullptr, nullptr, h->geo, 1.f, level, feat, 5, 4,
                          level ? h->ucoarse : nullptr, h->st); }));
   h->delta_real_valid = 0;
+  if (h->mk->kspace_fused && !h->kspace_generic) RG_TRY(check_fault(h));
   h->warm_level = level;
   return RECON_OK;
 }

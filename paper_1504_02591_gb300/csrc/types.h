@@ -107,6 +107,8 @@ struct SArgs {
   int generic;            // k-space update: the generic staged kernel instead of the register-fused one
   int ybeg, ycount;       // vector x passes: only the lines of y-planes [ybeg, ybeg + ycount)
                           // (ycount 0: every line; both multiples of the tile width)
+  int* fault;             // streamed passes: set to 1 by a wait that gave up (LoopState::fault)
+  int drop;               // tests: leave out the first tile's second copy, 1 in the vector x passes, 2 in the update
   const KIterMaps* tmaps; // host memory: the source update streams its inputs by TMA
   const VLineMaps* vmaps; // host memory: the vector x passes' maps, forward and inverse (null: plain loads)
   // vector inverse x pass unless loop_flag && *loop_flag == 1 (the device loop has just
@@ -123,7 +125,7 @@ struct LoopState {
   int flag;               // 0 running, 1 converged (final pass pending), 2 non-finite norms
   int it;                 // updates done
   int max_iter;
-  int pad;
+  int fault;              // a bounded wait gave up since the deposit, which clears it
   double tol;
   double trace[kMaxTrace];
 };
@@ -131,7 +133,7 @@ struct LoopState {
 // Result of one mock of a batch graph, written on the device: the loop's outcome and globaltimer
 // stamps (ns) at the start and end of the mock's work.
 struct BatchSlot {
-  int flag;               // LoopState::flag at the end of the mock's iteration
+  int flag;               // LoopState::flag at the end of the mock's iteration; 3: LoopState::fault was set
   int it;                 // updates done
   double rel;             // last |dPsi| / |Psi|
   unsigned long long t0, t1;
