@@ -326,7 +326,7 @@ recon_status recon_cic_deposit_noalloc(const void* pos, int dtype, const float* 
 /* Handle options (recon_set_option). */
 enum {
   RECON_OPT_DEPOSIT_PATH = 0,   /* RECON_PATH_DIRECT (default) or RECON_PATH_SORTED               */
-  RECON_OPT_SHIFT_PATH = 1,     /* RECON_PATH_SORTED (default) or RECON_PATH_DIRECT               */
+  RECON_OPT_SHIFT_PATH = 1,     /* RECON_PATH_AUTO (default), RECON_PATH_SORTED or RECON_PATH_DIRECT */
   RECON_OPT_GRAPH = 2,          /* 1 (default): recon_iterate runs the whole loop as one CUDA graph
                                    with a conditional WHILE node and a device-side convergence
                                    test; 0: the host reads the norms after every update.  Kernel
@@ -375,14 +375,14 @@ enum {
  * particle; 24 scattered reads per interpolated one, or 8 of nodes packed first); SORTED packs the
  * particles, counting-sorts them by 8^3-cell brick and works brick by brick in shared memory (deposit:
  * one global atomic per touched node of the brick; shift: Psi staged once per brick).  Both give the
- * same results up to float32 summation order.  A SORTED shift without a retained order
- * (RECON_OPT_REUSE_SORT) sorts only where that is the faster way: N >= 384 and at least N^3 / 32
- * particles; otherwise it runs as DIRECT. */
-enum { RECON_PATH_DIRECT = 0, RECON_PATH_SORTED = 1 };
+ * same results up to float32 summation order.  AUTO (shifts only) sorts where that is the faster way:
+ * N >= 384 and at least N^3 / 32 particles; otherwise it runs as DIRECT. */
+enum { RECON_PATH_DIRECT = 0, RECON_PATH_SORTED = 1, RECON_PATH_AUTO = 2 };
 
-/* Set a handle option (values 0 or 1, RECON_OPT_PLANE_BATCH 0/16/32/64, RECON_OPT_DROP_COPY 0/1/2); INVALID_ARG for an unknown
- * option or value; UNSUPPORTED for RECON_OPT_FFT_RADIX 1 on a mesh with one radix order; CUDA if
- * rebuilding the stage tables for another radix order fails. */
+/* Set a handle option (values 0 or 1; RECON_OPT_SHIFT_PATH and RECON_OPT_DROP_COPY 0, 1 or 2;
+ * RECON_OPT_PLANE_BATCH 0, 16, 32 or 64); INVALID_ARG for an unknown option or value; UNSUPPORTED for
+ * RECON_OPT_FFT_RADIX 1 on a mesh with one radix order; CUDA if rebuilding the stage tables for
+ * another radix order fails. */
 recon_status recon_set_option(recon_handle* h, int option, int value);
 
 /* One reconstruction of a batch (recon_batch_run). */

@@ -41,7 +41,7 @@ OPT_DEPOSIT_PATH, OPT_SHIFT_PATH, OPT_GRAPH, OPT_LINE_TILE, OPT_KSPACE_GENERIC, 
 OPT_PLANE_BATCH, OPT_ASSIGN, OPT_KITER_TMA, OPT_FFT_RADIX, OPT_DROP_COPY = 6, 7, 8, 9, 10
 ASSIGN_CIC, ASSIGN_NGP = 0, 1
 UNET_OPT_TENSOR_CORES = 0
-PATH_DIRECT, PATH_SORTED = 0, 1
+PATH_DIRECT, PATH_SORTED, PATH_AUTO = 0, 1, 2
 BATCH_TUNE, BATCH_ONE_GRAPH = 1, 2
 KERNEL_KINDS = ("deposit", "z_fwd", "z_inv", "z_delta", "z_proj", "z_final", "line_fwd", "line_inv",
                 "conv", "k_delta", "k_iter", "shift", "other", "sort")

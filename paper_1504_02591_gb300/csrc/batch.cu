@@ -30,7 +30,7 @@ namespace {
 struct Plan {
   int line_tile = 0;
   int deposit_path = RECON_PATH_DIRECT;
-  int shift_path = RECON_PATH_SORTED;
+  int shift_path = RECON_PATH_AUTO;
   int kspace_generic = 0;
   int fft_radix = 0;
 };

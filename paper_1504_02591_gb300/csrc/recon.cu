@@ -169,7 +169,7 @@ struct recon_handle {
   const MeshKernels* mk = nullptr;
   int state = ST_CREATED;
   int deposit_path = RECON_PATH_DIRECT;
-  int shift_path = RECON_PATH_SORTED;
+  int shift_path = RECON_PATH_AUTO;
   int narrow_lines = 0;
   int kspace_generic = 0;
   int plane_batch = 0;   // register-fused path: y-planes per batch of the x -> z -> x passes (0: off)
@@ -829,15 +829,14 @@ recon_status set_radix_order(recon_handle* h, int value);
 recon_status recon_set_option(recon_handle* h, int option, int value) {
   if (!h) return RECON_ERR_INVALID_ARG;
   if (option == RECON_OPT_PLANE_BATCH) return set_plane_batch(h, value);
-  if (option == RECON_OPT_DROP_COPY) {
+  if (option == RECON_OPT_DROP_COPY || option == RECON_OPT_SHIFT_PATH) {
     if (value < 0 || value > 2) return RECON_ERR_INVALID_ARG;
-    h->drop_copy = value;
+    (option == RECON_OPT_DROP_COPY ? h->drop_copy : h->shift_path) = value;
     return RECON_OK;
   }
   if (value != 0 && value != 1) return RECON_ERR_INVALID_ARG;
   if (option == RECON_OPT_FFT_RADIX) return set_radix_order(h, value);
   if (option == RECON_OPT_DEPOSIT_PATH) h->deposit_path = value;
-  else if (option == RECON_OPT_SHIFT_PATH) h->shift_path = value;
   else if (option == RECON_OPT_GRAPH) h->use_graph = value;
   else if (option == RECON_OPT_LINE_TILE) h->narrow_lines = value;
   else if (option == RECON_OPT_KSPACE_GENERIC) h->kspace_generic = value ? 1 : 0;
@@ -1354,8 +1353,8 @@ recon_status recon_get_trace(recon_handle* h, double* rel, int cap, int* n) {
 }
 
 namespace {
-// A shift that holds no brick order of its catalogue sorts it first only where that pays.  The sort and
-// the sorted gather cost about 75 us per 1e6 tracers plus the staging of every occupied brick; the direct
+// A shift on the automatic path that holds no brick order of its catalogue sorts it first only where that
+// pays.  The sort and the sorted gather cost about 75 us per 1e6 tracers plus the staging of every occupied brick; the direct
 // gather 72 us per 1e6 up to N = 128 and, where the three fields pass the L2, 140, 210, 330 and 410 at
 // N = 256, 384, 512 and 1024 for tracers all over the box (half of that for a survey's tenth of it).
 // Measured, uniform tracers, sorted / direct us: N = 64 2e6 419 / 146; 256 1e7 719 / 1403 (packed: 747);
@@ -1423,7 +1422,8 @@ recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galax
   }
   // with a retained brick order, other catalogues take the direct path so that it survives
   const bool keep_order = h->reuse_sort && h->memo.valid;
-  const bool sorted = h->shift_path == RECON_PATH_SORTED && !keep_order && shift_sorts(h->n, cat->n);
+  const bool sorted = !keep_order && (h->shift_path == RECON_PATH_SORTED ||
+                                      (h->shift_path == RECON_PATH_AUTO && shift_sorts(h->n, cat->n)));
   if (sorted) h->memo.valid = 0;
   if (!sorted && !keep_order && cat->n > 0 && shift_packs(h->n, cat->n)) {
     // nodes packed as float4, in the sort's scratch
