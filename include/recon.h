@@ -415,8 +415,9 @@ typedef struct recon_batch_item {
  * RECON_BATCH_*.  With RECON_BATCH_TUNE, a size class not seen before in this process is first
  * tuned on its first item, before the batch runs and outside every item's time: the deposit path,
  * the x-line FFT tile width, at N = 256, 384, 512 and 1024 the k-space kernel family (register-fused
- * or generic), at N = 256 and 384 the FFT radix order, and the shift path; the fastest are kept for the process
- * (recon_batch_plan).  With RECON_BATCH_ONE_GRAPH the whole batch is one CUDA graph, built before
+ * or generic), at N = 256 and 384 the FFT radix order, and, if the item's catalogue is large enough for
+ * the automatic shift path to sort it, the shift path (AUTO or DIRECT; else AUTO); the fastest are kept
+ * for the process (recon_batch_plan).  With RECON_BATCH_ONE_GRAPH the whole batch is one CUDA graph, built before
  * it is launched, with one chain of items per size class and the chains side by side (one item
  * per class in flight).  Other bits: INVALID_ARG.  Returns the first error of any item (per-item
  * statuses in items[i].status), else OK. */

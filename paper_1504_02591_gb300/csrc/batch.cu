@@ -15,7 +15,9 @@
 // class's candidate schedules on that mock (outside the items' times) and keeps the fastest for the
 // process: the deposit path (direct atomics or brick-sorted), the x-line FFT tile width (16 or 8
 // columns), the k-space kernel family where the mesh has two (register-fused or generic staged), for
-// N = 256 and 384 the FFT radix order and the shift path.
+// N = 256 and 384 the FFT radix order, and, where the automatic shift path sorts that mock's catalogue,
+// whether the direct one is faster.  Candidates that run the same kernels are not timed against each other:
+// noise would decide for every later catalogue of the class.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -100,8 +102,10 @@ recon_status tune(recon_handle* h, recon_batch_item& it, cudaStream_t st, Plan* 
   double rel = 0.0;
   for (int order = 0; order < orders; ++order) {
     if ((s = recon_set_option(h, RECON_OPT_FFT_RADIX, order)) != RECON_OK) return s;
-    for (int fam = 0; fam < fams; ++fam) {
-      for (int tile : {0, 1}) {
+    for (int fam = 0; fam < (order ? 1 : fams); ++fam) {   // the alternative order has the generic kernels alone
+      // the streamed vector x passes of the register-fused family have one tile width
+      const int tiles = !order && !fam && rg::mesh_kernels(it.params.nmesh[0])->vmap_cols ? 1 : 2;
+      for (int tile = 0; tile < tiles; ++tile) {
         recon_set_option(h, RECON_OPT_KSPACE_GENERIC, fam);
         recon_set_option(h, RECON_OPT_LINE_TILE, tile);
         recon_status si = recon_iterate(h, it.start, 0.0, 4, &n_it, &rel);   // warm (and graph build)
@@ -122,12 +126,13 @@ recon_status tune(recon_handle* h, recon_batch_item& it, cudaStream_t st, Plan* 
   if ((s = recon_set_option(h, RECON_OPT_FFT_RADIX, plan->fft_radix)) != RECON_OK) return s;
   recon_set_option(h, RECON_OPT_KSPACE_GENERIC, plan->kspace_generic);
   recon_set_option(h, RECON_OPT_LINE_TILE, plan->line_tile);
-  // shift path, on the randoms (or the galaxies when there are none)
+  // shift path, on the randoms (or the galaxies when there are none); below the size that the automatic path
+  // sorts it stays automatic, so that a later, larger catalogue of the class is sorted
   const recon_catalog* cat = ran ? ran : &it.gal;
   float* out = ran ? it.shift_ran : it.shift_gal;
-  if (out && cat->n > 0) {
+  if (out && rg::shift_sorts(it.params.nmesh[0], cat->n)) {
     best = 1e30f;
-    for (int path : {RECON_PATH_DIRECT, RECON_PATH_SORTED}) {
+    for (int path : {RECON_PATH_AUTO, RECON_PATH_DIRECT}) {
       recon_set_option(h, RECON_OPT_SHIFT_PATH, path);
       if ((s = recon_shift(h, cat, ran ? 0 : 1, out, nullptr, it.out_on_device)) != RECON_OK) return s;
       t.start();

@@ -12,6 +12,9 @@ namespace rg {
 void config_tables(int n, const recon_params* p, std::vector<float>& taps, int* t0, int* ntap,
                    std::vector<float>& off);
 
+// Whether a shift of `count` tracers sorts them on the automatic path (see recon.cu).
+bool shift_sorts(int n, int64_t count);
+
 // One mock of a batch graph: its item (device catalogues and outputs), its tables already in
 // device memory, and its result slot.
 struct BatchJob {

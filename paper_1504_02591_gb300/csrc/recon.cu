@@ -1352,7 +1352,9 @@ recon_status recon_get_trace(recon_handle* h, double* rel, int cap, int* n) {
   return RECON_OK;
 }
 
-namespace {
+}  // extern "C"
+
+namespace rg {
 // A shift on the automatic path that holds no brick order of its catalogue sorts it first only where that
 // pays.  The sort and the sorted gather cost about 75 us per 1e6 tracers plus the staging of every occupied brick; the direct
 // gather 72 us per 1e6 up to N = 128 and, where the three fields pass the L2, 140, 210, 330 and 410 at
@@ -1363,8 +1365,10 @@ namespace {
 bool shift_sorts(int n, int64_t count) { return n >= 384 && count >= (int64_t)n * n * n / 32; }
 // Packing the nodes as float4 (28 bytes moved per node: 12 us at N <= 128, 95 at 256) halves the direct
 // gather: 35 us per 1e6 tracers up to N = 128, 65 at 256; from N^3 / 8 tracers on (and 200,000) it pays.
-bool shift_packs(int n, int64_t count) { return n <= 256 && count >= 200000 && count >= (int64_t)n * n * n / 8; }
-}  // namespace
+static bool shift_packs(int n, int64_t count) { return n <= 256 && count >= 200000 && count >= (int64_t)n * n * n / 8; }
+}  // namespace rg
+
+extern "C" {
 
 recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galaxy, float* shift_out,
                          double* pos_out, int out_on_device) {
