@@ -376,7 +376,8 @@ enum {
  * particles, counting-sorts them by 8^3-cell brick and works brick by brick in shared memory (deposit:
  * one global atomic per touched node of the brick; shift: Psi staged once per brick).  Both give the
  * same results up to float32 summation order.  AUTO (shifts only) sorts where that is the faster way:
- * N >= 384 and at least N^3 / 32 particles; otherwise it runs as DIRECT. */
+ * N >= 384 and at least N^3 / 32 particles in the chunk (2^25 particles, 2^21 where positions or results
+ * are in host memory); otherwise it runs as DIRECT. */
 enum { RECON_PATH_DIRECT = 0, RECON_PATH_SORTED = 1, RECON_PATH_AUTO = 2 };
 
 /* Set a handle option (values 0 or 1; RECON_OPT_SHIFT_PATH and RECON_OPT_DROP_COPY 0, 1 or 2;

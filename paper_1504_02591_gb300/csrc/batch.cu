@@ -130,7 +130,8 @@ recon_status tune(recon_handle* h, recon_batch_item& it, cudaStream_t st, Plan* 
   // sorts it stays automatic, so that a later, larger catalogue of the class is sorted
   const recon_catalog* cat = ran ? ran : &it.gal;
   float* out = ran ? it.shift_ran : it.shift_gal;
-  if (out && rg::shift_sorts(it.params.nmesh[0], cat->n)) {
+  const bool staged = !cat->on_device || !it.out_on_device;
+  if (out && rg::shift_sorts(it.params.nmesh[0], std::min<int64_t>(cat->n, rg::shift_chunk(it.params.nmesh[0], staged)))) {
     best = 1e30f;
     for (int path : {RECON_PATH_AUTO, RECON_PATH_DIRECT}) {
       recon_set_option(h, RECON_OPT_SHIFT_PATH, path);

@@ -12,8 +12,9 @@ namespace rg {
 void config_tables(int n, const recon_params* p, std::vector<float>& taps, int* t0, int* ntap,
                    std::vector<float>& off);
 
-// Whether a shift of `count` tracers sorts them on the automatic path (see recon.cu).
+// Whether a shift sorts a chunk of `count` tracers on the automatic path, and the chunks' size (see recon.cu).
 bool shift_sorts(int n, int64_t count);
+long long shift_chunk(int n, bool staged);
 
 // One mock of a batch graph: its item (device catalogues and outputs), its tables already in
 // device memory, and its result slot.

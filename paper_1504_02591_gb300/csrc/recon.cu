@@ -1361,8 +1361,13 @@ namespace rg {
 // N = 256, 384, 512 and 1024 for tracers all over the box (half of that for a survey's tenth of it).
 // Measured, uniform tracers, sorted / direct us: N = 64 2e6 419 / 146; 256 1e7 719 / 1403 (packed: 747);
 // 384 2e6 508 / 452, 1e7 948 / 2131; 512 2e6 1014 / 682, 1e7 1499 / 3311; 1024 1e7 10784 / 4186, 3.3e7
-// 10730 / 13830.  The two meet near N^3 / 32 tracers on the meshes that sort at all.
+// 10730 / 13830.  The two meet near N^3 / 32 tracers on the meshes that sort at all.  The count is a chunk's:
+// a whole catalogue's would sort every 2^21 tracers of a host catalogue by themselves (page-locked float64
+// positions and shifts, the call so / by chunk: 512 3e7 20.9 / 16.6 ms, 1024 3.4e7 171 / 22.1) and a short last
+// chunk (1024, 3.4e7 on the device: 13.7 / 10.7).
 bool shift_sorts(int n, int64_t count) { return n >= 384 && count >= (int64_t)n * n * n / 32; }
+// Tracers that a shift handles together; staged: positions or results are in host memory.
+long long shift_chunk(int n, bool staged) { return staged && kStageParticles < sort_chunk(n) ? kStageParticles : sort_chunk(n); }
 // Packing the nodes as float4 (28 bytes moved per node: 12 us at N <= 128, 95 at 256) halves the direct
 // gather: 35 us per 1e6 tracers up to N = 128, 65 at 256; from N^3 / 8 tracers on (and 200,000) it pays.
 static bool shift_packs(int n, int64_t count) { return n <= 256 && count >= 200000 && count >= (int64_t)n * n * n / 8; }
@@ -1426,8 +1431,13 @@ recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galax
   }
   // with a retained brick order, other catalogues take the direct path so that it survives
   const bool keep_order = h->reuse_sort && h->memo.valid;
-  const bool sorted = !keep_order && (h->shift_path == RECON_PATH_SORTED ||
-                                      (h->shift_path == RECON_PATH_AUTO && shift_sorts(h->n, cat->n)));
+  const bool staged = !cat->on_device || !out_on_device;
+  const long long chunk = shift_chunk(h->n, staged);
+  // every chunk is sorted and gathered by itself, so its own size decides
+  auto sorts = [&](long long m) {
+    return !keep_order && (h->shift_path == RECON_PATH_SORTED || (h->shift_path == RECON_PATH_AUTO && shift_sorts(h->n, m)));
+  };
+  const bool sorted = sorts(cat->n < chunk ? cat->n : chunk);   // the first chunk, the largest
   if (sorted) h->memo.valid = 0;
   if (!sorted && !keep_order && cat->n > 0 && shift_packs(h->n, cat->n)) {
     // nodes packed as float4, in the sort's scratch
@@ -1437,8 +1447,6 @@ recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galax
     RG_CUDA(timed(h, RECON_K_SHIFT, 28.0 * nr, [&] { return launch_pack_psi(a.psi, psi4, nr, h->st); }));
     a.psi4 = psi4;
   }
-  const bool staged = !cat->on_device || !out_on_device;
-  const long long chunk = staged ? (kStageParticles < h->bb.chunk ? kStageParticles : h->bb.chunk) : h->bb.chunk;
   if (staged && !h->copy_st) {
     RG_CUDA(cudaStreamCreateWithFlags(&h->copy_st, cudaStreamNonBlocking));
     for (int b = 0; b < 2; ++b) {
@@ -1472,7 +1480,7 @@ recon_status recon_shift(recon_handle* h, const recon_catalog* cat, int is_galax
     ba.pos = pin;
     ba.shift = out_on_device ? shift_out + 3 * p0 : sshift;
     ba.pos_out = pos_out ? (out_on_device ? pos_out + 3 * p0 : spout) : nullptr;
-    if (sorted) {
+    if (sorts(m)) {
       RG_CUDA(timed(h, RECON_K_SORT, (double)m * (6 * es + 28),
                     [&] { return brick_sort(h->bb, pin, cat->dtype, nullptr, m, h->st); }));
       RG_CUDA(timed(h, RECON_K_SHIFT, (double)m * (16 + 16 + 4 + 16 + 12 + (pos_out ? 3 * es + 24 : 0)), [&] {

@@ -112,3 +112,26 @@ def test_retained_order_to_host_in_parts(lib):
     b = r.shift(pos, True)
     assert torch.equal(a, b.cpu())
     r.close()
+
+
+def test_automatic_path_decides_by_chunk(lib):
+    """Chunks are sorted one by one, so a chunk's own size decides: staged chunks of 2^21 tracers on a 512 mesh
+    (N^3 / 32 is twice that) and the short last chunk of a device catalogue are gathered directly."""
+    from paper_1504_02591_gb300 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(7)
+    for n, count, device_sorts, host_sorts in ((512, 512 ** 3 // 32 + 1, 1, 0), (384, (1 << 25) + 1001, 1, None)):
+        r = _solved(n, 6.0 * n)
+        tol = _tolerance(r)
+        pos = torch.rand((count, 3), generator=g, device="cuda", dtype=torch.float32) * 6.0 * n
+        s0 = _sorts(r)
+        a = r.shift(pos, True)
+        assert _sorts(r) - s0 == device_sorts
+        if host_sorts is not None:
+            s0 = _sorts(r)
+            b = torch.as_tensor(r.shift(pos.cpu().numpy(), True))
+            assert _sorts(r) - s0 == host_sorts
+            assert float((a.cpu() - b).abs().max()) <= tol
+        else:
+            r.set_option(B.OPT_SHIFT_PATH, B.PATH_DIRECT)
+            assert float((a - r.shift(pos, True)).abs().max()) <= tol
+        r.close()
