@@ -118,7 +118,10 @@ recon_status recon_workspace_bytes(const recon_params* p, size_t* bytes);
  *   workspace  device memory of at least recon_workspace_bytes bytes, 256-byte aligned, owned by
  *              the caller and kept alive until recon_destroy; NULL makes the handle allocate it
  *              itself with cudaMalloc (and free it in recon_destroy).  A workspace that is not
- *              256-byte aligned gives INVALID_ARG, one smaller than recon_workspace_bytes OOM. */
+ *              256-byte aligned gives INVALID_ARG, one smaller than recon_workspace_bytes OOM; but one
+ *              short by at most a field (4 N^3 + 8 N^2 bytes, each term rounded up to 256) on N = 256,
+ *              384, 512 and 1024 gives a handle that runs the generic kernels (as with
+ *              RECON_OPT_KSPACE_GENERIC 1), and so does a cudaMalloc that fails for that field alone. */
 recon_status recon_create(const recon_params* p, void* stream, void* workspace,
                           size_t workspace_bytes, recon_handle** out);
 

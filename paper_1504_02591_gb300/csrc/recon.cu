@@ -145,7 +145,7 @@ struct recon_handle {
   bool own_ws = false;
   Layout lay{};
   Field V[3]{}, D{}, S{};
-  Field W{};             // N = 512: Psi_z between the inverse x pass and the projection (C form)
+  Field W{};             // register-fused path: Psi_z between the inverse x pass and the projection (C form)
   float2* tw = nullptr;
   float2* tabs = nullptr;   // stage twiddles, N-point plan
   float2* tabz = nullptr;   // stage twiddles, N/2-point plan
@@ -296,6 +296,10 @@ Field field_at(char* base, const Layout& l) {
   return f;
 }
 
+// Whether the iteration runs in the mesh's register-fused kernels: it has them, the generic ones were not asked
+// for, and the workspace holds their fourth vector field.
+bool fused(const recon_handle* h) { return h->mk->kspace_fused && !h->kspace_generic && h->lay.wfield; }
+
 ZArgs zargs(recon_handle* h) {
   ZArgs a{};
   a.g = h->geo;
@@ -307,7 +311,7 @@ ZArgs zargs(recon_handle* h) {
   a.mask_frac = h->p.mask_frac;
   a.uniform = h->p.mean_density_mode == RECON_MEAN_UNIFORM;
   a.lognormal = h->p.lognormal;
-  a.generic = h->kspace_generic;
+  a.generic = !fused(h);
   a.wf = h->W;
   return a;
 }
@@ -323,7 +327,7 @@ SArgs sargs(recon_handle* h) {
   a.inv_b = (float)(1.0 / h->p.b);
   a.beta = (float)(h->p.f / h->p.b);
   a.narrow = h->narrow_lines;
-  a.generic = h->kspace_generic;
+  a.generic = !fused(h);
   a.lognormal = h->p.lognormal;
   a.tmaps = (h->tmaps_ok && h->kiter_tma) ? &h->tmaps : nullptr;
   a.vmaps = h->tmaps_ok ? h->vmaps : nullptr;
@@ -378,7 +382,7 @@ double rfield(const recon_handle* h) { return (double)h->n * h->n * h->n * 4.0; 
 
 double zbytes(const recon_handle* h, int mode, int nc, const ZArgs& a) {
   // the register-fused path hands the z pass three fields (two in C form) and takes two back (psi^, Z^)
-  const int nv = (h->mk->kspace_fused && !h->kspace_generic && nc == 3) ? 2 : nc;
+  const int nv = (fused(h) && nc == 3) ? 2 : nc;
   if (mode == Z_PROJ && a.cform) return 4.0 * cfield(h);
   if (mode == Z_DELTA) {
     const int nin = a.uniform ? 1 : 2;
@@ -392,12 +396,12 @@ double zbytes(const recon_handle* h, int mode, int nc, const ZArgs& a) {
 
 double sbytes(const recon_handle* h, int mode, int nc, int axis, int cform) {
   // the register-fused path carries the x and z components of k-space vectors as one field
-  const bool fused = h->mk->kspace_fused && !h->kspace_generic;
-  if (mode == S_DELTA) return (fused ? 5.0 : 6.0) * cfield(h);   // delta in, delta(k), S, 2 or 3 Psi
-  if (mode == S_ITER) return (fused ? 7.0 : 9.0) * cfield(h);    // 2 or 3 P + delta(k) + S in; 2 or 3 Psi + S out
+  const bool fu = fused(h);
+  if (mode == S_DELTA) return (fu ? 5.0 : 6.0) * cfield(h);   // delta in, delta(k), S, 2 or 3 Psi
+  if (mode == S_ITER) return (fu ? 7.0 : 9.0) * cfield(h);    // 2 or 3 P + delta(k) + S in; 2 or 3 Psi + S out
   // paired x passes: inverse 2 fields in, 3 out (2 in C form); forward 2 in (the pair's shared one
   // read once), 2 out
-  if (fused && axis == AX_X && nc == 3) return (mode == S_INV && !cform ? 5.0 : 4.0) * cfield(h);
+  if (fu && axis == AX_X && nc == 3) return (mode == S_INV && !cform ? 5.0 : 4.0) * cfield(h);
   return 2.0 * nc * cfield(h);
 }
 
@@ -431,13 +435,13 @@ recon_status finalize(recon_handle* h, int nblocks, int nq, int dst, int accumul
 // the x passes transform lines at fixed (y, kz) and the z pass rows at fixed (x, y), so each batch
 // of planes can go through all three before the next, and its fields stay in the L2 in between.
 int plane_batch(const recon_handle* h) {
-  return (h->plane_batch && h->mk->kspace_fused && !h->kspace_generic) ? h->plane_batch : 0;
+  return fused(h) ? h->plane_batch : 0;
 }
 
 // Whether the inverse x pass and the projection (or radial) pass exchange C = dx Psi_x + dy Psi_y
 // and Psi_z (register-fused path) rather than the three components.
 int cform(const recon_handle* h) {
-  return (h->mk->kspace_fused && !h->kspace_generic && h->lay.wfield) ? 1 : 0;
+  return fused(h) ? 1 : 0;
 }
 
 // Inverse x, the projection pass and forward x over all y-planes, batch by batch.  za and the x
@@ -716,7 +720,15 @@ recon_status recon_create(const recon_params* p, void* stream, void* workspace, 
   h->mk = mesh_kernels(h->n);
   h->lay = layout_for(h->n);
   cudaGetDevice(&h->device);
+  // memory short of the fourth vector field is enough for the generic kernels
+  auto without_w = [&] {
+    const bool has = h->lay.wfield != 0;
+    h->lay.total -= h->lay.wfield;
+    h->lay.wfield = 0;
+    return has;
+  };
   if (workspace) {
+    if (workspace_bytes < h->lay.total) without_w();
     if (workspace_bytes < h->lay.total || ((uintptr_t)workspace & 255)) {
       delete h;
       return ((uintptr_t)workspace & 255) ? RECON_ERR_INVALID_ARG : RECON_ERR_OOM;
@@ -724,10 +736,12 @@ recon_status recon_create(const recon_params* p, void* stream, void* workspace, 
     h->ws = (char*)workspace;
     h->ws_bytes = workspace_bytes;
   } else {
-    if (cudaMalloc(&h->ws, h->lay.total) != cudaSuccess) {
+    while (cudaMalloc(&h->ws, h->lay.total) != cudaSuccess) {
       cudaGetLastError();
-      delete h;
-      return RECON_ERR_OOM;
+      if (!without_w()) {
+        delete h;
+        return RECON_ERR_OOM;
+      }
     }
     h->own_ws = true;
     h->ws_bytes = h->lay.total;
@@ -1255,7 +1269,7 @@ recon_status iterate_core(recon_handle* h, const StartSpec& sp, double tol, int 
       RG_TRY(run_z(h, Z_PROJ, 3, zc));
       RG_TRY(xpass(h, S_FWD, 3, h->V));
     }
-    if (h->mk->kspace_fused && !h->kspace_generic) {
+    if (fused(h)) {
       const recon_status fs = check_fault(h);
       if (fs != RECON_OK) {
         h->state = ST_SMOOTHED;
@@ -1329,7 +1343,7 @@ recon_status recon_start_features(recon_handle* h, int start, int level, float* 
     return launch_radial(reinterpret_cast<const float*>(h->V[0].M), nullptr, nullptr, h->geo, 1.f, level, feat, 5, 4,
                          level ? h->ucoarse : nullptr, h->st); }));
   h->delta_real_valid = 0;
-  if (h->mk->kspace_fused && !h->kspace_generic) RG_TRY(check_fault(h));
+  if (fused(h)) RG_TRY(check_fault(h));
   h->warm_level = level;
   return RECON_OK;
 }
