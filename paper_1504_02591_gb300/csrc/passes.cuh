@@ -1750,13 +1750,6 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   return bar_try_wait(bar, parity);
 }
 
-// hi + lo += x, the rounding of hi kept in lo.
-__device__ __forceinline__ void two_add(float& hi, float& lo, float x) {
-  const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
-  hi = t;
-}
-
 template <int N, int C>
 __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter_tma_kernel(const SArgs a,
                                                                        const __grid_constant__ KIterMaps maps) {
@@ -1788,7 +1781,7 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
         if (!(a.drop == 2 && q == 1 && tt == 0))
           tma_load3(dst + (uint32_t)(q * K::kField + h * (K::kField / K::kBoxes)), &maps.m[q], c0, K::kRows * h, kx, bar);
   };
-  float dh = 0.f, dl = 0.f, sh = 0.f, sl = 0.f;   // norms over the CTA's tiles, in pairs of float32
+  double dsum = 0.0, ssum = 0.0;   // norms over the CTA's tiles
   float2 v[2][8], dk[8], sp[8];
   uint32_t parity = 0;
   if (threadIdx.x == 0 && (int)blockIdx.x < MT) issue(blockIdx.x);
@@ -1818,8 +1811,8 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
     }
     float d2 = 0.f, s2 = 0.f;
     kiter_tile<N, C>(a, tile_of<N, C, AX_Y>(tt), v, dk, sp, s, tw, j, col, d2, s2);
-    two_add(dh, dl, d2);
-    two_add(sh, sl, s2);
+    dsum += d2;
+    ssum += s2;
   }
   if (!give_up) {
     for (int q = blockIdx.x; q < QT; q += gridDim.x) {   // Nyquist tiles: plain loads
@@ -1827,12 +1820,12 @@ __global__ void __launch_bounds__(KFused<N, C>::T, KTma<N, C>::kMinBlocks) kiter
       kiter_load<N, C>(a, t, j, col, v, dk, sp);
       float d2 = 0.f, s2 = 0.f;
       kiter_tile<N, C>(a, t, v, dk, sp, s, tw, j, col, d2, s2);
-      two_add(dh, dl, d2);
-      two_add(sh, sl, s2);
+      dsum += d2;
+      ssum += s2;
     }
   }
-  double r0 = block_sum((double)dh + (double)dl, red_sh);
-  double r1 = block_sum((double)sh + (double)sl, red_sh);
+  double r0 = block_sum(dsum, red_sh);
+  double r1 = block_sum(ssum, red_sh);
   if (threadIdx.x == 0) {
     if (give_up) r0 = r1 = __longlong_as_double(0x7ff8000000000000ll);   // NaN: the loop stops
     a.partials[2 * blockIdx.x + 0] = r0;
