@@ -15,7 +15,8 @@
 // of 1600 us an iteration at 128^3 for 8 MB of data.  The kernels work in pairs of float32 (hi + lo, sums and
 // products with their exact rounding errors carried along: Dekker 1971, Knuth's two-sum), about 45
 // bits, and round once to float32 on output; the sums over the mesh keep such pairs per thread and
-// continue in float64 per block.  BiCGStab's scalars live on the device: each reduction's last block
+// continue in float64 per block.  Powers of two (exact) keep them inside float32's range: a node's offsets are
+// taken over the largest of them, the operator's sums times about 1 / g^2, the right-hand side over about 1 / b.  BiCGStab's scalars live on the device: each reduction's last block
 // forms the scalar the next kernel needs, so an iteration runs without the host.
 #include "cic.h"
 #include "fd.h"
@@ -72,26 +73,32 @@ __device__ __forceinline__ float at(const float* __restrict__ p, int n, int x, i
 // (the last term is the rounding of a fixed direction's length; zero for a radial one, and at the
 // observer's node, where n = 0, the whole line-of-sight term is zero).
 struct Coef {
-  F2 b, g, ig2, u[3], k0;   // beta, g, 1 / g^2, fixed direction, -2 beta (1 - |u|^2)
+  F2 b, g, ig2, u[3], k0;   // beta sp, g, 1 / (sp g^2), fixed direction, -2 beta sp (1 - |u|^2)
 };
 
 __device__ __forceinline__ float fd_operator(const float* __restrict__ phi, int n, int x, int y, int z, const FDArgs& a,
                                              const Coef& k) {
   const float p0 = at(phi, n, x, y, z);
   F2 acc;
-  F2 fp[3];   // beta n_d / r (radial: x_d / r^2), beta u_d (fixed)
+  F2 fp[3];   // sp beta times n_d / r (radial: x_d / r^2) or u_d (fixed)
   const bool rsd = a.beta != 0.0;
   float xs[3] = {0.f, 0.f, 0.f};
-  F2 inv = {0.f, 0.f};
+  F2 inv = {0.f, 0.f}, gs = k.g;
   if (rsd && a.los_mode != 1) {
     xs[0] = a.off[x];
     xs[1] = a.off[n + y];
     xs[2] = a.off[2 * n + z];
+    // lengths over the power of two at or below the largest offset, so that r^2 is 1 to 12
+    const int ex = (int)(__float_as_uint(fmaxf(fabsf(xs[0]), fmaxf(fabsf(xs[1]), fabsf(xs[2])))) >> 23);
+    const float us = __uint_as_float((uint32_t)(254 - min(ex, 253)) << 23);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) xs[d] *= us;
     const F2 r2 = add(add(two_prod(xs[0], xs[0]), two_prod(xs[1], xs[1])), two_prod(xs[2], xs[2]));
     if (r2.h > 0.f) {
       const float i0 = __frcp_rn(r2.h);
       const float e = __fmaf_rn(-r2.l, i0, __fmaf_rn(-r2.h, i0, 1.f));
       inv = {i0, __fmul_rn(e, i0)};
+      gs = {k.g.h * us, k.g.l * us};
     }
   }
   acc = {0.f, 0.f};
@@ -107,6 +114,8 @@ __device__ __forceinline__ float fd_operator(const float* __restrict__ phi, int 
     dm[d] = two_sum(f1, -f0);
     acc = add(acc, q);
   }
+  acc.h *= a.sp;
+  acc.l *= a.sp;
   if (rsd) {
     const bool fixed = a.los_mode == 1;
 #pragma unroll
@@ -115,7 +124,7 @@ __device__ __forceinline__ float fd_operator(const float* __restrict__ phi, int 
     for (int d = 0; d < 3; ++d) {
       const F2 xd = fixed ? k.u[d] : F2{xs[d], 0.f};
       acc = add(acc, mul(mul(fp[d], xd), dp[d]));
-      if (!fixed) acc = add(acc, mul(mul(fp[d], k.g), dm[d]));
+      if (!fixed) acc = add(acc, mul(mul(fp[d], gs), dm[d]));
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d)
@@ -144,13 +153,13 @@ __device__ __forceinline__ float fd_operator(const float* __restrict__ phi, int 
 
 __device__ __forceinline__ Coef coefficients(const FDArgs& a) {
   Coef k;
-  k.b = split(a.beta);
+  k.b = split(a.beta * a.sp);
   k.g = split(a.g);
-  k.ig2 = split(1.0 / (a.g * a.g));
+  k.ig2 = split(1.0 / (a.sp * a.g * a.g));
   k.u[0] = split(a.los.x);
   k.u[1] = split(a.los.y);
   k.u[2] = split(a.los.z);
-  k.k0 = split(-2.0 * a.beta * (1.0 - (a.los.x * a.los.x + a.los.y * a.los.y + a.los.z * a.los.z)));
+  k.k0 = split(-2.0 * a.beta * a.sp * (1.0 - (a.los.x * a.los.x + a.los.y * a.los.y + a.los.z * a.los.z)));
   return k;
 }
 
@@ -225,8 +234,8 @@ __global__ void __launch_bounds__(256) fd_init_kernel(const float* __restrict__ 
 // Start of an iteration: p = r + (rho / rho_old)(alpha / omega)(p - omega v) (p = r in the first), and
 // its copy for the preconditioner.
 __global__ void __launch_bounds__(256) fd_dir_kernel(const float* __restrict__ r, const float* __restrict__ v,
-                                                     float* __restrict__ p, float* __restrict__ pre, size_t n,
-                                                     const FDState* __restrict__ st) {
+                                                     float* __restrict__ p, float* __restrict__ pre, float scale,
+                                                     size_t n, const FDState* __restrict__ st) {
   if (st->done) return;
   const bool first = st->it == 0;
   const F2 bt = split((st->rho / st->rho_old) * (st->alpha / st->omega)), om = split(-st->omega);
@@ -234,7 +243,7 @@ __global__ void __launch_bounds__(256) fd_dir_kernel(const float* __restrict__ r
     float y = r[i];
     if (!first) y = round2(add(F2{y, 0.f}, mul(bt, add(F2{p[i], 0.f}, mul(om, F2{v[i], 0.f})))));
     p[i] = y;
-    pre[i] = y;
+    pre[i] = y * scale;
   }
 }
 
@@ -272,15 +281,15 @@ __global__ void __launch_bounds__(256) fd_apply_kernel(const float* __restrict__
 // s = r - alpha v and its copy for the preconditioner; ends the solve (with x += alpha ph still to do)
 // when |s| is small enough.
 __global__ void __launch_bounds__(256) fd_s_kernel(const float* __restrict__ r, const float* __restrict__ v,
-                                                   float* __restrict__ s, float* __restrict__ pre, size_t n,
-                                                   FDState* __restrict__ st, double* __restrict__ partials) {
+                                                   float* __restrict__ s, float* __restrict__ pre, float scale,
+                                                   size_t n, FDState* __restrict__ st, double* __restrict__ partials) {
   if (st->done) return;
   const F2 al = split(-st->alpha);
   F2 acc[1] = {{0.f, 0.f}};
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
     const float y = round2(add(F2{r[i], 0.f}, mul(al, F2{v[i], 0.f})));
     s[i] = y;
-    pre[i] = y;
+    pre[i] = y * scale;
     acc_prod(acc[0], y, y);
   }
   double tot[1];
@@ -338,18 +347,18 @@ __global__ void __launch_bounds__(256) fd_gradient_kernel(const float* __restric
   const F2 h = split(-0.5 / a.g);
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const int x = (int)(e / ((size_t)n * n)), y = (int)((e / n) % n), z = (int)(e % n);
-    psi[e] = round2(mul(two_sum(at(phi, n, x + 1, y, z), -at(phi, n, x - 1, y, z)), h));
-    psi[total + e] = round2(mul(two_sum(at(phi, n, x, y + 1, z), -at(phi, n, x, y - 1, z)), h));
-    psi[2 * total + e] = round2(mul(two_sum(at(phi, n, x, y, z + 1), -at(phi, n, x, y, z - 1)), h));
+    psi[e] = a.un * round2(mul(two_sum(at(phi, n, x + 1, y, z), -at(phi, n, x - 1, y, z)), h));
+    psi[total + e] = a.un * round2(mul(two_sum(at(phi, n, x, y + 1, z), -at(phi, n, x, y - 1, z)), h));
+    psi[2 * total + e] = a.un * round2(mul(two_sum(at(phi, n, x, y, z + 1), -at(phi, n, x, y, z - 1)), h));
   }
 }
 
 // 1 / (N^3 lambda) of the periodic 7-point Laplacian on the half grid, formed once per solve in float64
 // (per application it took 231 us at 128^3): [kx][ky][kz < N/2] then the Nyquist plane [kx][ky].
-__global__ void __launch_bounds__(256) fd_factor_kernel(float* __restrict__ fac, int n, double L) {
+__global__ void __launch_bounds__(256) fd_factor_kernel(float* __restrict__ fac, int n, double L, double scale) {
   const int h = n / 2;
   const size_t nm = (size_t)n * n * h, nq = (size_t)n * n;
-  const double g = L / n, n3 = (double)n * n * n;
+  const double g = L / n, n3 = (double)n * n * n * scale;
   const double k0 = -L * L / (3.0 * M_PI * M_PI) / n3;
   extern __shared__ double cs[];   // 2 cos(2 pi m / N) - 2
   for (int m = threadIdx.x; m < n; m += blockDim.x) cs[m] = 2.0 * cospi(2.0 * m / n) - 2.0;
@@ -379,8 +388,9 @@ cudaError_t launch_fd_init(const float* delta, float c, double inv_b, float* x, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_fd_dir(const float* r, const float* v, float* p, float* pre, size_t n, const FDState* st, cudaStream_t s) {
-  fd_dir_kernel<<<kGrid, 256, 0, s>>>(r, v, p, pre, n, st);
+cudaError_t launch_fd_dir(const float* r, const float* v, float* p, float* pre, float scale, size_t n, const FDState* st,
+                          cudaStream_t s) {
+  fd_dir_kernel<<<kGrid, 256, 0, s>>>(r, v, p, pre, scale, n, st);
   return cudaGetLastError();
 }
 
@@ -392,9 +402,9 @@ cudaError_t launch_fd_apply(int mode, const float* phi, float* out, const float*
   return cudaGetLastError();
 }
 
-cudaError_t launch_fd_s(const float* r, const float* v, float* sv, float* pre, size_t n, FDState* st, double* partials,
-                        cudaStream_t s) {
-  fd_s_kernel<<<kGrid, 256, 0, s>>>(r, v, sv, pre, n, st, partials);
+cudaError_t launch_fd_s(const float* r, const float* v, float* sv, float* pre, float scale, size_t n, FDState* st,
+                        double* partials, cudaStream_t s) {
+  fd_s_kernel<<<kGrid, 256, 0, s>>>(r, v, sv, pre, scale, n, st, partials);
   return cudaGetLastError();
 }
 
@@ -409,8 +419,8 @@ cudaError_t launch_fd_gradient(const float* phi, float* psi, const FDArgs& a, cu
   return cudaGetLastError();
 }
 
-cudaError_t launch_fd_factor(float* fac, int n, double L, cudaStream_t st) {
-  fd_factor_kernel<<<kGrid, 256, n * sizeof(double), st>>>(fac, n, L);
+cudaError_t launch_fd_factor(float* fac, int n, double L, double scale, cudaStream_t st) {
+  fd_factor_kernel<<<kGrid, 256, n * sizeof(double), st>>>(fac, n, L, scale);
   return cudaGetLastError();
 }
 

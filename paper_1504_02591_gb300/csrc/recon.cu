@@ -11,6 +11,7 @@
 //   shift    CIC interpolation of Psi to the particles, d = -(Psi + f (Psi.r) r) or -Psi (Sec. 1)
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1691,6 +1692,11 @@ recon_status recon_fd_solve(recon_handle* h, double tol, int max_iter, int* n_it
   fa.los_mode = h->p.los_mode;
   fa.los = make_double3(h->geo.los.x, h->geo.los.y, h->geo.los.z);
   fa.off = h->cur_off;
+  auto near = [](double v) { return v > 0 && std::isfinite(v) ? std::min(std::max(std::ilogb(v), -60), 60) : 0; };
+  const int eg = near(fa.g), eb = near(1.0 / h->p.b);
+  fa.sp = std::ldexp(1.f, -2 * eg);
+  fa.pre = std::ldexp(1.f, eg);
+  fa.un = std::ldexp(1.f, eb);
   float c = 0.f;   // the lognormal constant added back, as recon_get_field does
   if (h->p.lognormal) {
     double sl = 0;
@@ -1699,18 +1705,18 @@ recon_status recon_fd_solve(recon_handle* h, double tol, int max_iter, int* n_it
     c = (float)(-sl / (double)nr);
   }
   RG_CUDA(cudaMemsetAsync(st, 0, sizeof(FDState), h->st));
-  RG_CUDA(launch_fd_factor(fac, h->n, h->L, h->st));
-  RG_CUDA(launch_fd_init(reinterpret_cast<const float*>(h->V[2].M), c, 1.0 / h->p.b, x, r, rh, nr, st, tol, h->partials,
-                         h->st));   // r = delta / b
+  RG_CUDA(launch_fd_factor(fac, h->n, h->L, fa.pre, h->st));
+  RG_CUDA(launch_fd_init(reinterpret_cast<const float*>(h->V[2].M), c, 1.0 / h->p.b / fa.un, x, r, rh, nr, st, tol,
+                         h->partials, h->st));   // r = delta / (b un)
   // BiCGStab, right-preconditioned (A M^-1 y = b, x = M^-1 y).  Its scalars stay on the device and its
   // kernels end themselves, so the host only follows one iteration behind.
   EventPair ev;
   for (cudaEvent_t& e : ev.e) RG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   for (int k = 0; k < max_iter; ++k) {
-    RG_CUDA(timed(h, RECON_K_OTHER, 20.0 * nr, [&] { return launch_fd_dir(r, v, p, ph, nr, st, h->st); }));
+    RG_CUDA(timed(h, RECON_K_OTHER, 20.0 * nr, [&] { return launch_fd_dir(r, v, p, ph, fa.pre, nr, st, h->st); }));
     RG_TRY(fd_precond(h, h->V[0], fac));
     RG_CUDA(timed(h, RECON_K_OTHER, 12.0 * nr, [&] { return launch_fd_apply(0, ph, v, rh, fa, st, h->partials, h->st); }));
-    RG_CUDA(timed(h, RECON_K_OTHER, 16.0 * nr, [&] { return launch_fd_s(r, v, sv, sh, nr, st, h->partials, h->st); }));
+    RG_CUDA(timed(h, RECON_K_OTHER, 16.0 * nr, [&] { return launch_fd_s(r, v, sv, sh, fa.pre, nr, st, h->partials, h->st); }));
     RG_TRY(fd_precond(h, h->V[1], fac));
     RG_CUDA(timed(h, RECON_K_OTHER, 12.0 * nr, [&] { return launch_fd_apply(1, sh, t, sv, fa, st, h->partials, h->st); }));
     RG_CUDA(timed(h, RECON_K_OTHER, 32.0 * nr, [&] {
