@@ -458,7 +458,8 @@ recon_status recon_unet_get_grads(recon_unet* u, float* host, size_t count);
  * storage, the convolutions of every level whose side is 64 or a multiple of 128 run on the tensor
  * cores (tcgen05.mma, float32 accumulation in tensor memory); the others on the CUDA cores.  Both
  * round every stored activation to bfloat16 at the same points, so they differ only in the order
- * of the float32 sums.  Returns ERR_CUDA if a tensor-core wait timed out. */
+ * of the float32 sums.  Returns ERR_CUDA if a tensor-core wait timed out, OOM for a grid that the device
+ * cannot hold or of 2^31 voxels and more (sides above 1288). */
 recon_status recon_unet_forward(recon_unet* u, const float* x, int n, float* y);
 /* Forward, mean squared error against target (device, n^3) and all parameter gradients; *loss
  * (host) receives the loss when not NULL. */

@@ -9,6 +9,7 @@
 // w[tap][cin][cout] computes y[v][co] = b[co] + sum_tap sum_ci x[v + d(tap)][ci] w[tap][ci][co].
 #include <cuda_bf16.h>
 
+#include <climits>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(256) conv_fwd_kernel(const T* __restrict__ xa,
   extern __shared__ float4 wsm4[];
   float* wsm = reinterpret_cast<float*>(wsm4);
   const int cin = cina + cb;
-  const int nv = n * n * n;   // at most 256^3 voxels times 32 channels: 32-bit offsets
+  const int nv = n * n * n;   // below 2^31 (ensure)
   float2 acc[VPT][COUT / 2];
   int vx[VPT], vy[VPT], vz[VPT], vv[VPT];
 #pragma unroll
@@ -672,6 +673,9 @@ Grads grad_layout(const recon_unet* u, int n) {
 
 recon_status ensure(recon_unet* u, int n, bool train) {
   if (n < 8 || n % 8 != 0) return RECON_ERR_INVALID_ARG;
+  // The layers index voxels in 32 bits.  Only the narrowest network's inference at sides 1296 to 1312 would fit
+  // 288 GB beyond that.
+  if ((long long)n * n * n > INT_MAX) return RECON_ERR_OOM;
   if (n <= u->n_alloc && (!train || u->grads)) return RECON_OK;
   const int nn = n > u->n_alloc ? n : u->n_alloc;
   if (u->acts) cudaFree(u->acts);
