@@ -684,6 +684,7 @@ recon_status ensure(recon_unet* u, int n, bool train) {
   u->acts = nullptr;
   u->grads = nullptr;
   u->y = nullptr;
+  u->n_alloc = 0;   // until all of them are there: a call after one that ran out of memory allocates again
   const size_t es = u->bf16 ? 2 : 4;
   if (cudaMalloc(&u->acts, act_layout(u, nn).total * es) != cudaSuccess ||
       cudaMalloc(&u->y, (size_t)nn * nn * nn * sizeof(float)) != cudaSuccess ||

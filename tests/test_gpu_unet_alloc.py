@@ -32,3 +32,17 @@ def test_grids_past_32bit_voxel_indices_are_refused(lib, n):
     assert st == B.ERR_OOM
     assert np.array_equal(net.get_layer(0, 16, 8), layer)
     net.close()
+
+
+def test_forward_after_out_of_memory(lib):
+    """A grid whose activations do not fit (c1 = 8, 1288^3: 223 GB, with 120 GB held) gives OOM; the next forward, on
+    a side that had been allocated before, allocates again and gives the same output."""
+    B, net, x = _net()
+    y = net.forward(x)
+    ballast = torch.empty(120 * 10 ** 9, dtype=torch.uint8, device="cuda")
+    st = net.lib.recon_unet_forward(net.h, C.c_void_p(x.data_ptr()), 1288, C.c_void_p(y.data_ptr()))
+    del ballast
+    torch.cuda.empty_cache()
+    assert st == B.ERR_OOM
+    assert torch.equal(net.forward(x), y)
+    net.close()
