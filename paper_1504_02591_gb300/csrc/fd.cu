@@ -15,9 +15,10 @@
 // of 1600 us an iteration at 128^3 for 8 MB of data.  The kernels work in pairs of float32 (hi + lo, sums and
 // products with their exact rounding errors carried along: Dekker 1971, Knuth's two-sum), about 45
 // bits, and round once to float32 on output; the sums over the mesh keep such pairs per thread and
-// continue in float64 per block.  Powers of two (exact) keep them inside float32's range: a node's offsets are
-// taken over the largest of them, the operator's sums times about 1 / g^2, the right-hand side over about 1 / b.  BiCGStab's scalars live on the device: each reduction's last block
-// forms the scalar the next kernel needs, so an iteration runs without the host.
+// continue in float64 per block.  Powers of two (exact) keep them inside float32's range: a node's offsets
+// are taken over the largest of them, the operator's sums times about 1 / g^2, the right-hand side over
+// about 1 / b.  BiCGStab's scalars live on the device: each reduction's last block forms the scalar the next
+// kernel needs, so an iteration runs without the host.
 #include "cic.h"
 #include "fd.h"
 

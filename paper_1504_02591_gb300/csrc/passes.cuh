@@ -1476,10 +1476,10 @@ __global__ void __launch_bounds__(XLine<N, C>::T, XLine<N, C>::kMinBlocks) xline
   if (!INV && a.skip_flag && *a.skip_flag != 0) return;   // uniform: device loop already converged
   for (int m = threadIdx.x; m < X::kTab; m += T) tw[m] = a.tabx[m];
   const int role = PAIR ? (int)(blockIdx.x & 1) : (int)blockIdx.y;
-  // tiles of every y-plane, or of the planes [ybeg, ybeg + ycount): their M tiles (ky, kz block)
-  // and the Nyquist tiles that hold their ky columns
+  // tiles of every y-plane, or (vector passes) of the planes [ybeg, ybeg + ycount): their M tiles
+  // (ky, kz block) and the Nyquist tiles that hold their ky columns
   int ti = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-  if (a.ycount) {
+  if (PAIR && a.ycount) {
     const int mt = a.ycount * (H / C);
     ti = ti < mt ? a.ybeg * (H / C) + ti : N * (H / C) + a.ybeg / C + (ti - mt);
   }
@@ -2031,15 +2031,6 @@ static inline cudaError_t persistent_grid(const void* k, int threads, size_t sme
   return cudaSuccess;
 }
 
-template <class K>
-static cudaError_t launch_with_smem(K kern, int blocks, int threads, size_t smem, cudaStream_t st, const void* arg) {
-  static_assert(sizeof(K) > 0, "");
-  cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  void* args[] = {const_cast<void*>(arg)};
-  return cudaLaunchKernel((const void*)kern, dim3(blocks), dim3(threads), args, smem, st);
-}
-
 template <int N>
 struct MeshImpl {
   static constexpr int kZBlocks = N * N / kZWarps;   // rows / warps per CTA: upper bound of the Z grid
@@ -2156,8 +2147,8 @@ struct MeshImpl {
     if constexpr (kFusedMesh<N>) return TCols<N>::v;
     return 0;
   }
-  
-static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
+
+  static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
     if constexpr (kFusedMesh<N>) {
       constexpr int C = SCols<N, S_ITER>::v;
       if (a.tmaps) {   // inputs streamed by TMA into persistent CTAs
@@ -2214,11 +2205,12 @@ static cudaError_t klaunch(const SArgs& a, cudaStream_t st) {
       if (e != cudaSuccess) return e;
       attr[inv] = true;
     }
-    if (a.ycount && (a.ycount % C || a.ybeg % C || a.ybeg < 0 || a.ybeg + a.ycount > N)) return cudaErrorInvalidValue;
+    const int ny = PAIR && a.ycount ? a.ycount : N;
+    if (PAIR && a.ycount && (ny % C || a.ybeg % C || a.ybeg < 0 || a.ybeg + ny > N)) return cudaErrorInvalidValue;
     SArgs ax = a;
     ax.tabx = a.tab + ((Plan<N>::kTab + 1) & ~1);
     void* args[] = {&ax};
-    const int tiles = a.ycount ? a.ycount * ((N / 2) / C) + a.ycount / C : N * ((N / 2) / C) + N / C;
+    const int tiles = ny * ((N / 2) / C) + ny / C;
     // pairs: the two CTAs of a tile on adjacent block indices; single fields: components along y
     const dim3 grid = PAIR ? dim3(2 * tiles) : dim3(tiles, ncomp);
     return cudaLaunchKernel(k, grid, dim3(X::T), args, X::smem, st);

@@ -103,7 +103,8 @@ struct SArgs {
   int d_is_k;             // S_DELTA: dk is already fully transformed
   int lognormal;          // S_DELTA: subtract the lognormal constant at k = 0
   const int* skip_flag;   // plain passes: do nothing when *skip_flag != 0 (device-driven loop)
-  int narrow;             // single-field x passes: 8-column instead of 16-column tiles
+  int narrow;             // x passes that are not streamed (single fields, the pairs of N = 1024): 8-column
+                          // instead of 16-column tiles
   int generic;            // k-space update: the generic staged kernel instead of the register-fused one
   int ybeg, ycount;       // vector x passes: only the lines of y-planes [ybeg, ybeg + ycount)
                           // (ycount 0: every line; both multiples of the tile width)
