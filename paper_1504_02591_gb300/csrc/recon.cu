@@ -1195,7 +1195,11 @@ recon_status run_start(recon_handle* h, const StartSpec& sp) {
 }
 
 // Whether a streamed pass's bounded wait gave up since the deposit: what the passes left is then not to be used.
+// While the stream is captured nothing can be asked; the word stays set for the next recon_iterate.
 recon_status check_fault(recon_handle* h) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  RG_CUDA(cudaStreamIsCapturing(h->st, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return RECON_OK;
   int fault = 0;
   RG_CUDA(cudaMemcpyAsync(&fault, &h->loop->fault, sizeof(int), cudaMemcpyDeviceToHost, h->st));
   RG_CUDA(cudaStreamSynchronize(h->st));
