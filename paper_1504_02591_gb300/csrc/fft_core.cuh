@@ -32,6 +32,11 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
+// a (b + lo), lo the rounding of b
+__device__ __forceinline__ float2 cmul_fine(float2 a, float2 b, float2 lo) {
+  return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, fmaf(a.x, lo.x, -a.y * lo.y))),
+                     fmaf(a.x, b.y, fmaf(a.y, b.x, fmaf(a.x, lo.y, a.y * lo.x))));
+}
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 // multiply by -i (forward sign) or +i (inverse sign)
@@ -166,33 +171,33 @@ struct Dft<6, INV> {
 // Radix 8 Q = Q x 8 (Q = 3, 4): y[k1 + 8 k2] = sum_n2 w^(n2 k1) wQ^(n2 k2) sum_n1 w8^(n1 k1) x[Q n1 + n2],
 // w = exp(-+ 2 pi i / (8 Q)); the factors w^m from the cosine table of the radix (sin(m) = cos(m - R/4)).
 template <int R>
-__device__ __forceinline__ constexpr float dft_cos(int m);
+__device__ __forceinline__ constexpr double dft_cos(int m);
 template <>
-__device__ __forceinline__ constexpr float dft_cos<24>(int m) {
-  constexpr float c[24] = {
-      1.f, 0.96592582628906831f, 0.86602540378443871f, 0.70710678118654757f,
-      0.5f, 0.25881904510252074f, 0.f, -0.25881904510252063f,
-      -0.5f, -0.70710678118654746f, -0.86602540378443871f, -0.9659258262890682f,
-      -1.f, -0.96592582628906831f, -0.86602540378443882f, -0.70710678118654791f,
-      -0.5f, -0.25881904510252063f, 0.f, 0.2588190451025203f,
-      0.5f, 0.70710678118654735f, 0.86602540378443837f, 0.96592582628906809f};
+__device__ __forceinline__ constexpr double dft_cos<24>(int m) {
+  constexpr double c[24] = {
+      1.0, 0.96592582628906831, 0.86602540378443871, 0.70710678118654757,
+      0.5, 0.25881904510252074, 0.0, -0.25881904510252063,
+      -0.5, -0.70710678118654746, -0.86602540378443871, -0.9659258262890682,
+      -1.0, -0.96592582628906831, -0.86602540378443882, -0.70710678118654791,
+      -0.5, -0.25881904510252063, 0.0, 0.2588190451025203,
+      0.5, 0.70710678118654735, 0.86602540378443837, 0.96592582628906809};
   return c[((m % 24) + 24) % 24];
 }
 template <>
-__device__ __forceinline__ constexpr float dft_cos<32>(int m) {
-  constexpr float c[32] = {
-      1.f, 0.98078528040323043f, 0.92387953251128674f, 0.83146961230254524f,
-      0.70710678118654757f, 0.55557023301960229f, 0.38268343236508984f, 0.19509032201612833f,
-      0.f, -0.19509032201612819f, -0.38268343236508973f, -0.55557023301960196f,
-      -0.70710678118654746f, -0.83146961230254535f, -0.92387953251128674f, -0.98078528040323043f,
-      -1.f, -0.98078528040323043f, -0.92387953251128685f, -0.83146961230254546f,
-      -0.70710678118654768f, -0.55557023301960218f, -0.38268343236509034f, -0.19509032201612866f,
-      0.f, 0.1950903220161283f, 0.38268343236509f, 0.55557023301960184f,
-      0.70710678118654735f, 0.83146961230254524f, 0.92387953251128652f, 0.98078528040323032f};
+__device__ __forceinline__ constexpr double dft_cos<32>(int m) {
+  constexpr double c[32] = {
+      1.0, 0.98078528040323043, 0.92387953251128674, 0.83146961230254524,
+      0.70710678118654757, 0.55557023301960229, 0.38268343236508984, 0.19509032201612833,
+      0.0, -0.19509032201612819, -0.38268343236508973, -0.55557023301960196,
+      -0.70710678118654746, -0.83146961230254535, -0.92387953251128674, -0.98078528040323043,
+      -1.0, -0.98078528040323043, -0.92387953251128685, -0.83146961230254546,
+      -0.70710678118654768, -0.55557023301960218, -0.38268343236509034, -0.19509032201612866,
+      0.0, 0.1950903220161283, 0.38268343236509, 0.55557023301960184,
+      0.70710678118654735, 0.83146961230254524, 0.92387953251128652, 0.98078528040323032};
   return c[((m % 32) + 32) % 32];
 }
 
-template <int Q, bool INV>
+template <int Q, bool INV, bool FINE = false>
 struct Dft8Q {
   static constexpr int R = 8 * Q;
   __device__ __forceinline__ static void run(float2* v) {
@@ -209,8 +214,12 @@ struct Dft8Q {
 #pragma unroll
       for (int n2 = 0; n2 < Q; ++n2) {
         const int m = n2 * k1;
-        const float c = dft_cos<R>(m), sn = dft_cos<R>(m - R / 4);
-        b[n2] = m == 0 ? t[n2][k1] : cmul(t[n2][k1], make_float2(c, INV ? sn : -sn));
+        const double c = dft_cos<R>(m), sn = dft_cos<R>(m - R / 4), si = INV ? sn : -sn;
+        const float2 w = make_float2((float)c, (float)si);
+        if (FINE && m % (R / 4) != 0)
+          b[n2] = cmul_fine(t[n2][k1], w, make_float2((float)(c - w.x), (float)(si - w.y)));
+        else
+          b[n2] = m == 0 ? t[n2][k1] : cmul(t[n2][k1], w);
       }
       Dft<Q, INV>::run(b);
 #pragma unroll
@@ -222,6 +231,14 @@ template <bool INV>
 struct Dft<24, INV> : Dft8Q<3, INV> {};
 template <bool INV>
 struct Dft<32, INV> : Dft8Q<4, INV> {};
+// The radices of the x lines: 32 with its factors' own rounding carried along.  Without, a 32 x 32 line rounds worse
+// than radices 8 16 8 or 8 8 4 4: r2c of white noise at 1024, 2.026e-7 against 1.977e-7 with staged x lines, with it
+// 1.910e-7; the 1024 box's solve against float64 2.48e-7, 2.29e-7 with staged kernels, with it 2.30e-7 (two seeds).
+// The x passes wait for memory: the 1024 box takes 233 ms either way.
+template <int R, bool INV>
+struct DftFine : Dft<R, INV> {};
+template <bool INV>
+struct DftFine<32, INV> : Dft8Q<4, INV, true> {};
 
 // ----------------------------------------------------------------------------------------------
 // Shared-memory layouts.  Element i of line col lives at phys(i, col).  The swizzles make every

@@ -1419,7 +1419,7 @@ __device__ __forceinline__ void xline_io(float2* __restrict__ s, const float2* _
   {
     float2 x[E];
     ld(x);
-    Dft<E, INV>::run(x);
+    DftFine<E, INV>::run(x);
 #pragma unroll
     for (int r = 0; r < E; ++r) s[X::row(jb, r, col)] = x[r];
   }
@@ -1437,7 +1437,7 @@ __device__ __forceinline__ void xline_io(float2* __restrict__ s, const float2* _
         if (INV) w.y = -w.y;
         y[r] = cmul(y[r], w);
       }
-      Dft<G, INV>::run(y);
+      DftFine<G, INV>::run(y);
       st(h, y);
     }
   }
